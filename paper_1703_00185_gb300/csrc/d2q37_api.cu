@@ -28,57 +28,54 @@ void split_df(double v, float* hi, float* lo) {
   *lo = (float)(v - (double)*hi);
 }
 
-// round((hi + lo) 2^Q) as hi 2^32 + lo with a signed low word (below 2^63 - 2^31 in magnitude).
-FxConst fixed_const(double hi, double lo, int Q) {
+// round((hi + lo) 2^Q) as an unsigned 64-bit integer (0 <= value < 2^64).
+unsigned long long fixed_u64(double hi, double lo, int Q) {
   const double H = std::ldexp(hi, Q), L = std::ldexp(lo, Q);
   const double Hr = std::nearbyint(H);
-  const long long v = (long long)Hr + std::llround((H - Hr) + L);
-  const int low = (int)(unsigned)((unsigned long long)v & 0xFFFFFFFFull);
-  return {low, (int)((v - low) >> 32)};
+  return (unsigned long long)Hr + (unsigned long long)std::llround((H - Hr) + L);
 }
 
-// A double-double (unevaluated sum hi + lo) product.
-struct DD {
-  double h, l;
-};
-DD dd_mul(DD a, DD b) {
-  const double h = a.h * b.h;
-  return {h, std::fma(a.h, b.h, -h) + (a.h * b.l + a.l * b.h)};
-}
-
-// Constants of the fixed-point equilibrium (see StepParams), from double-double
-// products of s, the shift tau g_y and omega w_k = (c_k hi + c_k lo) 2^E_k.
+// Constants of the fixed-point equilibrium (see StepParams), from the
+// double-double product omega w_k = (c_k hi + c_k lo) 2^E_k.
 void fill_fixed_consts(StepParams& sp) {
   const ShellConsts& c = g_consts;
-  const DD s = {c.s, 0.0}, s2 = dd_mul(s, s), s4 = dd_mul(s2, s2), sd = dd_mul(s, {sp.uy_shift, 0.0});
-  const double is2 = 1.0 / s2.h;  // 1 / s^2, with one Newton step on its low part
-  const DD inv = {is2, is2 * (std::fma(-is2, s2.h, 1.0) - is2 * s2.l)};
-  // tau g_y must fit the shifted-field formats (other lattices take FP64 everywhere)
-  sp.fx_on = std::fabs(sp.uy_shift) < 0.35;
-  if (!sp.fx_on) return;
-  sp.fx_one = 1;
-  sp.fx_two = 2;
-  sp.fx_s2_62 = fixed_const(s2.h, s2.l, 62);
-  sp.fx_sd_64 = fixed_const(sd.h, sd.l, 64);
-  sp.fx_sd_60 = fixed_const(sd.h, sd.l, 60);
-  sp.fx_lim_63 = fixed_const(0.35 * c.s, 0.0, 63);
-  sp.fx_is2_63 = fixed_const(inv.h, inv.l, 63);
-  sp.fx_is2_61 = fixed_const(inv.h, inv.l, 61);
-  sp.fx_hs2_63 = fixed_const(s2.h, s2.l, 62);
-  sp.fx_s4_64 = fixed_const(s4.h, s4.l, 61);  // s^4 / 8
-  const double sixth = 1.0 / 6.0;
-  sp.fx_sixth_61 = fixed_const(sixth, std::fma(-sixth, 6.0, 1.0) / 6.0, 61);
   for (int k = 0; k < kShells; ++k) {
-    const DD w = dd_mul({sp.omega, 0.0}, {c.w[k], 0.0});
+    const double wh = sp.omega * c.w[k];
+    const double wl = std::fma(sp.omega, c.w[k], -wh);
     int E;
-    std::frexp(shell_hop(k) == 3 ? 1.125 * w.h : w.h, &E);
-    sp.fx_es[k] = (E - fx_q(k)) * (1 << 20);
-    double hm = 1.0;
-    for (int m = 0; m < 3; ++m, hm *= shell_hop(k)) {
-      const double v = w.h * hm;
-      sp.fx_w[k][m] = fixed_const(v, std::fma(w.h, hm, -v) + w.l * hm, fx_q(k) + 3 - E);
-    }
+    std::frexp(wh, &E);  // wh = m 2^E, m in [0.5, 1)
+    sp.fx_e[k] = E;
+    const double ch = std::ldexp(wh, -E), cl = std::ldexp(wl, -E);
+    const double x2 = c.s2 * shell_c2(k);
+    const double x2h = x2, x2l = std::fma(c.s2, (double)shell_c2(k), -x2);  // exact: c.s2 times a small integer
+    // c x2 and c x2^2 in double-double
+    const double p1h = ch * x2h, p1l = std::fma(ch, x2h, -p1h) + (cl * x2h + ch * x2l);
+    const double p2h = p1h * x2h, p2l = std::fma(p1h, x2h, -p2h) + (p1l * x2h + p1h * x2l);
+    sp.fx_c60[k] = fixed_u64(ch, cl, 60);
+    sp.fx_c62[k] = fixed_u64(ch, cl, 62);
+    sp.fx_c64[k] = fixed_u64(ch, cl, 64);
+    sp.fx_cx2_59[k] = fixed_u64(p1h, p1l, 59);
+    sp.fx_cx2_60[k] = fixed_u64(p1h, p1l, 60);
+    sp.fx_cx4_55[k] = fixed_u64(p2h, p2l, 55);
+    const double q6 = ch / 6.0, q6l = (std::fma(-q6, 6.0, ch) + cl) / 6.0;
+    sp.fx_c6[k] = fixed_u64(q6, q6l, 64);  // also (c/24) 2^66: one product serves R3 and R4
+    // R0 = K0 c60 + (K1 + 2^63) cx2_59 + K2 cx4_55, R1 = (L0 + 2^63) c62 +
+    // (L1 + 2^63) cx2_59, R2 = (M0 + 2^63) c64 + (M1 + 2^63) cx2_60, with
+    // corrections for their floors and those of the pair's product each
+    // feeds (b t, b R3, b R4; with the conversion's lowest bit for R0): +2 for
+    // R0, +1 for R1 and R2; the shell-0 population, K0 c60 alone, needs none
+    sp.fx_d0[k] = k == 0 ? 0ull : (sp.fx_cx2_59[k] >> 1) - 2ull;
+    sp.fx_d1[k] = (sp.fx_c62[k] >> 1) + (sp.fx_cx2_59[k] >> 1) - 1ull;
+    sp.fx_d2[k] = (sp.fx_c64[k] >> 1) + (sp.fx_cx2_60[k] >> 1) - 1ull;
   }
+  sp.fx_s62 = fixed_u64(c.s, 0.0, 62);
+  sp.fx_s63 = fixed_u64(c.s, 0.0, 63);
+  const double s2h = c.s * c.s, s2l = std::fma(c.s, c.s, -s2h);
+  sp.fx_s2_63 = fixed_u64(s2h, s2l, 63);
+  // the shifted-field constants: tau g_y in Q64 and theta_shift in Q60 (signed)
+  sp.fx_on = std::fabs(sp.uy_shift) < 0.35 && sp.theta_shift > -4.0 && sp.theta_shift < 4.0;
+  sp.fx_uy_shift = sp.fx_on ? std::llround(std::ldexp(sp.uy_shift, 64)) : 0;
+  sp.fx_th_shift = sp.fx_on ? std::llround(std::ldexp(sp.theta_shift, 60)) : 0;
 }
 
 void solve_once() {

@@ -107,51 +107,39 @@ __device__ __forceinline__ void site_moments_fp64(const double (&f)[kQ], double&
 // NaN take the FP64 form.
 constexpr long long kFloorR = 16, kFloorE = 105;
 
-// top2 = 2 (2^20 emax + 2^20 - 1): the shift emax - e in two instructions, the
-// doubling dropping the sign bit (the mantissa bits borrow nothing).
-__device__ __forceinline__ long long fixed_term(double v, unsigned top2) {
+__device__ __forceinline__ long long fixed_term(double v, int emax) {
   const int hi = __double2hiint(v);
-  const unsigned sh = (top2 - 2u * (unsigned)hi) >> 21;
-  const int s = hi >> 31;  // 0 or -1
+  const unsigned lo = (unsigned)__double2loint(v);
+  const int e = (hi >> 20) & 0x7FF;
   // the implicit one is set for zero and subnormal inputs too: with emax >= 64
-  // their shift is above 62 and they round to 0 (-1 for a negative zero).  A
-  // negative v enters as the one's complement of its magnitude, -mant - 1: its
+  // their shift is the full 62 and they round to 0 (-1 for a negative zero)
+  const long long mant = ((long long)((hi & 0xFFFFF) | 0x100000) << 32) | lo;
+  const int sh = min(emax - e, 62);
+  const long long s = hi >> 31;  // 0 or -1
+  // a negative v as the one's complement of its magnitude, -mant - 1: its
   // arithmetic shift is floor(v 2^-sh) or, when the dropped bits are all zero,
   // one below it
-  const int mh = ((hi & 0xFFFFF) | 0x100000) ^ s;
-  const int ml = __double2loint(v) ^ s;
-  long long r;  // PTX clamps shifts above 63 (C++ leaves them undefined)
-  asm("{\n\t.reg .b64 m;\n\tmov.b64 m, {%1, %2};\n\tshr.s64 %0, m, %3;\n\t}" : "=l"(r) : "r"(ml), "r"(mh), "r"(sh));
-  return r;
+  return (mant ^ s) >> sh;
 }
 
 // The exact sums r = sum f, jx, jy = sum c f, e = sum |c|^2 f on the grid
 // 2^(emax - 1075); false for the sites that take the FP64 sums.
 __device__ __forceinline__ bool site_sums(const double (&f)[kQ], long long& r, long long& jx, long long& jy,
                                           long long& e, int& emax) {
-  // the largest |high word| (its exponent field is the largest exponent): the
-  // signed maximum finds the largest positive one, the unsigned one the
-  // largest negative one
-  int hs = 0;
-  unsigned hu = 0;
+  int hmax = 0;  // the largest |high word|: its exponent field is the largest exponent
 #pragma unroll
-  for (int l = 0; l < kQ; ++l) {
-    hs = max(hs, __double2hiint(f[l]));
-    hu = max(hu, (unsigned)__double2hiint(f[l]));
-  }
-  const int hmax = max(hs, (int)(hu & 0x7FFFFFFFu));
+  for (int l = 0; l < kQ; ++l) hmax = max(hmax, __double2hiint(f[l]) & 0x7FFFFFFF);
   emax = hmax >> 20;
   if (emax < 64 || emax > 2046) return false;
-  const unsigned top2 = 2u * (unsigned)(hmax | 0xFFFFF);
   long long sh[kShells];
-  sh[0] = fixed_term(f[0], top2);
+  sh[0] = fixed_term(f[0], emax);
 #pragma unroll
   for (int k = 1; k < kShells; ++k) sh[k] = 0;
   jx = jy = 0;
 #pragma unroll
   for (int p = 0; p < kPairs; ++p) {
-    const long long vp = fixed_term(f[1 + 2 * p], top2);
-    const long long vm = fixed_term(f[2 + 2 * p], top2);
+    const long long vp = fixed_term(f[1 + 2 * p], emax);
+    const long long vm = fixed_term(f[2 + 2 * p], emax);
     sh[pair_shell(p)] += vp + vm;
     const long long d = vp - vm;
     jx += pair_cx(p) * d;
@@ -201,183 +189,216 @@ __device__ __forceinline__ double hop_dot(int cx, int cy, const double (&mx)[3],
 
 // ---- the equilibrium in 64-bit fixed point ---------------------------------
 //
-// GB300 issues 2 FP64 operations per SM per clock, while a 32 x 32 -> 64-bit
-// multiply-add (IMAD.WIDE) runs at about 32.  So the equilibrium of the FP64
-// step is evaluated in fixed point: each quantity is a signed 64-bit integer
-// scaled by its own power of two ("Qn": v 2^-n), and a product is the high
-// word of a 128-bit product (fx_mul: three multiply-adds).
+// GB300 issues 2 FP64 operations per SM per clock, while the high 64 bits of
+// a 64 x 64-bit integer product take about four IMAD.WIDE on the integer
+// pipes.  So the equilibrium of the FP64 step is evaluated in fixed point:
+// each quantity is an int64 scaled by its own power of two ("Qn": v 2^-n),
+// chosen from its range so that every product is the high word of a 128-bit
+// product and keeps 2^-55 or better absolute precision on the order-1
+// quantities; exact integer sums remove the cancellation that
+// limits the FP64 form near T = 0.5 for the outer shells.  Per population
+// the result is turned into an FP64 number (fx_to_double: the FP64 pipe's
+// integer conversion, or integer operations for the shells of
+// D2Q37_INT_CVT_MASK) and relaxed with one FP64 FMA.  The shell factor omega w_k is carried as
+// c_k 2^E_k with c_k in [0.5, 1).  The ranges that keep every intermediate
+// inside its format hold for rho in (0, 4), |T_bar - 1| < 1 and |u_bar| < 0.35
+// per component; other sites take the FP64 evaluation.
 //
-// The equilibrium is a polynomial of degree 4 in the integer hop c = (cx, cy),
-//   f^eq_l = w_l rho P(c_l),   P(c) = sum_{i+j<=4} p_ij cx^i cy^j,
-// whose 15 coefficients are site values.  With U = s u_x, V = s u_bar_y,
-// A = U^2, B = V^2, theta = T_bar - 1 and q = (A + B) / s^2:
-//   L0 = 1 - q/2 - 2 theta,  M0 = (L0 - theta) / 2,  G = s^2 theta / 2,
-//   p00 = 1 - q/2 + q^2/8 - theta + theta q + theta^2,
-//   p20 = K1 + A M0,  p02 = K1 + B M0,  p11 = 2 U V M0,
-//   p40 = K2 + A (G/2 + A/24),  p04 = K2 + B (G/2 + B/24),
-//   p22 = 2 K2 + A (G/2 + B/4) + B G/2,
-//   p10 = U L0,  p30 = U (G + A/6),  p12 = U (G + B/2),
-//   p01 = V L0,  p03 = V (G + B/6),  p21 = V (G + A/2),
-//   p31 = V p30,  p13 = U p03,
-//   K1 = s^2 (theta/2 - theta q/4 - theta^2),  K2 = s^4 theta^2 / 8,
-// all times rho below.  The hops of one class (|cx|, |cy|) differ by signs
-// only: with the parts of P even in both components (ee), odd in cx (oe), odd
-// in cy (eo) and odd in both (oo), their four values are (ee +- oo) +- (oe +-
-// eo), and every part is one or two products with the class's weight, the
-// powers of a hop of 2 or 3 folded into it.  So the 37 equilibria take 42
-// products with constants after about 40 site products; a chain per pair of
-// opposite hops (Horner in a = xi.u, after eight products per shell) took
-// about 165 products and a longer dependency chain: 2048 x 8192 step 2.71 ms
-// against 2.16 ms with this form.
-//
-// rho enters as rho^ in [0.5, 1) (the moment sum shifted to its leading one,
-// a power of two taken out that joins the result's exponent).  The ranges
-// |theta| < 1 and |u_bar| < 0.35 per component keep every value inside its
-// format; other sites take the FP64 evaluation.  Products round to nearest
-// (within 0.75 of the last place, no bias: both low words are signed and the
-// half is added), so neither the momentum nor the energy drifts.
-// tests/test_hop_moment_formats.py restates these integers and holds them
-// to 2^-52 of omega w rho against rational arithmetic (the FP64 evaluation
-// loses about 1e-14 for the outer shells near T = 0.5).
+// With K0 = rho (A0 - theta + theta q + theta^2), K1 = rho (theta/2 - theta q/4
+// - theta^2), K2 = rho theta^2 / 8, L0 = rho (B1 - 2 theta), L1 = rho theta / 2,
+// M0 = rho (B2 - 3 theta / 2), M1 = rho theta / 4 (site values), the shell
+// coefficients of collide_site times c_k rho are
+//   R0 = c (K0 + x2 K1 + x2^2 K2),  R1 = c (L0 + x2 L1),  R2 = c (M0 + x2 M1),
+//   R3 = c rho / 6,  R4 = c rho / 24 (one product: (c/6) 2^64 is (c/24) 2^66),
+// and per pair even = R0 + b (R2 + b R4), odd = a (R1 + b R3), b = a^2.
+// A signed site value x meets the unsigned shell constants as x + 2^63 (its
+// sign bit flipped), which needs no sign fix: x y 2^-64 = (x + 2^63) y 2^-64
+// - y / 2, and the y / 2 terms of a shell are one constant subtracted from R0,
+// R1 and R2 (fx_d0, fx_d1, fx_d2), together with corrections for the
+// roundings of its sums and per-pair products (0.5 below on average for an
+// exact high word, 0.75 for umulhi_t).  K0 > 0.74 rho inside the ranges and
+// needs no shift.  With the set lowest bit of the conversion (+0.5 on
+// average) and two corrections in fx_d0, the equilibrium's mass bias is
+// +1.7e-17 per collision relative to omega rho (without the corrections:
+// -7.6e-17), which the moment sums' -1.2e-17 nearly cancels.
+// The odd part takes a rounded product: a bias there would act on the
+// momentum the same way every step.
+constexpr int kFxOut = 55;  // format of R0 and of the results G = even +- odd
+
 using u64 = unsigned long long;
 
-// hi 2^32 + lo with a signed low word, the operand form of fx_mul
-struct FxOp {
-  int lo, hi;
-};
-
-// |v| < 2^63 - 2^31
-__device__ __forceinline__ FxOp fx_op(long long v) {
-  const int lo = (int)v;
-  return {lo, (int)((u64)v >> 32) + (int)((unsigned)lo >> 31)};
+// floor(x y 2^-64) for signed x, unsigned y
+__device__ __forceinline__ long long mulhi_su(long long x, u64 y) {
+  return (long long)(__umul64hi((u64)x, y) - (y & (u64)(x >> 63)));  // x >> 63: 0 or all ones
 }
 
-__device__ __forceinline__ FxOp fx_op(const FxConst& c) { return {c.lo, c.hi}; }
-
-// x y 2^-64 to within 1.25 of the last place, unbiased: the high word of each
-// cross product is a floor (0.5 low on average, together one) and `one` = 1
-// takes that back; the product of the low words (below 2^62, signed) is left
-// out.  One comes from the launch's parameters: as a value the compiler does
-// not know it enters the multiply-add as its addend, while a literal 1 cost an
-// addition of its own.  Five instructions, three of them 32-bit multiplies;
-// with 64-bit cross sums rounded by 2^31 (error 0.75) seven to fourteen.
-__device__ __forceinline__ long long fx_mul(FxOp x, FxOp y, int one) {
-  const int t = __mulhi(x.lo, y.hi) + (__mulhi(x.hi, y.lo) + one);
-  return (long long)x.hi * y.hi + t;
+// The high word of a y with the low-by-low partial product left out: three
+// 32 x 32 -> 64-bit multiply-adds and one add, the floor of a y 2^-64 or one
+// below it (0.75 below a y 2^-64 on average).  More instructions than the
+// exact high word but a shorter dependency chain: the per-pair products,
+// which form one chain per pair, take this form.
+__device__ __forceinline__ u64 umulhi_t(u64 a, u64 y) {
+  const unsigned al = (unsigned)a, ah = (unsigned)(a >> 32);
+  const unsigned yl = (unsigned)y, yh = (unsigned)(y >> 32);
+  const u64 lh = (u64)al * yh;
+  const u64 hl = (u64)ah * yl + (lh & 0xFFFFFFFFull);  // < 2^64
+  return (u64)ah * yh + (lh >> 32) + (hl >> 32);
 }
 
-// (x y + z w) 2^-64, two = 2
-__device__ __forceinline__ long long fx_mul2(FxOp x, FxOp y, FxOp z, FxOp w, int two) {
-  const int t = __mulhi(z.lo, w.hi) + (__mulhi(z.hi, w.lo) + (__mulhi(x.lo, y.hi) + (__mulhi(x.hi, y.lo) + two)));
-  return (long long)x.hi * y.hi + ((long long)z.hi * w.hi + t);
+// umulhi_t for signed x: x y = (x mod 2^64) y - 2^64 y [x < 0]
+__device__ __forceinline__ long long mulhi_su_t(long long x, u64 y) {
+  return (long long)(umulhi_t((u64)x, y) - (y & (u64)(x >> 63)));
 }
 
-// v 2^n without undefined behaviour for negative v
-__device__ __forceinline__ long long fx_shl(long long v, int n) { return (long long)((u64)v << n); }
+// round(x y 2^-64) (half up) for signed x, unsigned y.  Used where a biased
+// rounding would act the same way every step: the odd part of a pair, whose
+// magnitude a floor after the sign split would always shrink (a momentum
+// damping of 2^-56 per step relative to the odd part).
+// The four 32 x 32-bit partial products are independent; the rounding half
+// (2^63 of the 128-bit product) enters the middle column as 2^31.
+__device__ __forceinline__ long long mulhi_su_rn(long long x, u64 y) {
+  const unsigned xl = (unsigned)x, xh = (unsigned)((u64)x >> 32);
+  const unsigned yl = (unsigned)y, yh = (unsigned)(y >> 32);
+  const u64 ll = (u64)xl * yl, lh = (u64)xl * yh, hl = (u64)xh * yl, hh = (u64)xh * yh;
+  const u64 mid = (ll >> 32) + (lh & 0xFFFFFFFFull) + (hl & 0xFFFFFFFFull) + 0x80000000ull;  // < 2^34
+  const u64 hi = hh + (lh >> 32) + (hl >> 32) + (mid >> 32);  // floor(((x mod 2^64) y + 2^63) 2^-64)
+  return (long long)(hi - (y & (u64)(x >> 63)));
+}
 
-// g 2^E as an FP64 number by integer operations (round half away from zero),
-// es = E 2^20.  The FP64 pipe converts too (I2F, one of its slots, as long as
-// an FMA's), but it is the busiest unit and the integer pipes have room: 2048
-// x 8192 step 2.16 ms with every population converted here, 2.27-2.34 ms with
-// half of them, 2.51 ms with none.
+// floor(x y 2^-sh) for signed x, y and 0 < sh < 64 (the result fits 64 bits)
+__device__ __forceinline__ long long mul_shift(long long x, long long y, int sh) {
+  const u64 h = (u64)__mul64hi(x, y);
+  const u64 l = (u64)x * (u64)y;
+  return (long long)((h << (64 - sh)) | (l >> sh));
+}
+
+// g 2^(E - 55) as an FP64 number, two ways: with the FP64 pipe's 64-bit
+// integer conversion (round to nearest even) and the power of two added to
+// the exponent field, or with integer operations only (round half away from
+// zero).  The shells k whose bit is set in D2Q37_INT_CVT_MASK take the
+// integer form.  On GB300, with the FP64 pipe about 75 % busy, the last
+// shell's 8 populations that way (0x80) ran the 2048 x 8192 step in 2.742 ms,
+// against 2.784 ms for none, 2.802 / 2.847 ms for the last two / three
+// shells and 2.74-2.82 ms for shell 7 with one of shells 1, 3, 4, 5 (all of
+// them, with 4 blocks of 128 per SM: 4.37 against 4.12).
+#ifndef D2Q37_INT_CVT_MASK
+#define D2Q37_INT_CVT_MASK 0x80
+#endif
+
+// g != 0
+__device__ __forceinline__ double fx_to_double_fp64(long long g, int E) {
+  const double d = (double)g;  // exact up to its one rounding
+  const u64 bits = (u64)__double_as_longlong(d) + ((u64)(long long)(E - kFxOut) << 52);
+  return __longlong_as_double((long long)bits);
+}
+
 // |g| < 2^32 (including 0): the general normalisation
-__device__ __noinline__ double fx_to_double_small(unsigned m, int es, int sign) {
+__device__ __noinline__ double fx_to_double_small(u64 m, int E, u64 sign) {
   if (!m) return 0.0;
-  const int lz = __clz((int)m);
-  const u64 mant = (u64)(m << lz) << 21;  // leading one at bit 52
-  const int hi = (int)(mant >> 32) + es + ((1023 + 31 - lz - 1) << 20);
-  return __hiloint2double(hi | sign, (int)mant);
+  const int lz = __clzll((long long)m);
+  const u64 n = m << (lz - 1);  // leading one at bit 62
+  const u64 mant = (n + 0x200) >> 10;
+  const u64 bits = ((u64)(long long)(1023 + 62 - kFxOut + E - lz) << 52) + mant;
+  return __longlong_as_double((long long)(bits | sign));
 }
 
-// The magnitude is the one's complement for negative g: one less than |g|.
-__device__ __forceinline__ double fx_to_double(long long g, int es) {
-  const int gh = (int)(g >> 32), sm = gh >> 31;
-  const unsigned mh = (unsigned)(gh ^ sm), ml = (unsigned)g ^ (unsigned)sm;
-  const int sign = sm & (int)0x80000000;
-  if (mh == 0u) return fx_to_double_small(ml, es, sign);
-  // the leading one moved to bit 62 (|g| < 2^63), rounded to 53 bits, 54 when
-  // the rounding carries; it adds 1 to the exponent field, a carry one more
-  const int lz = __clz((int)mh) - 1;
-  const u64 n = ((u64)__funnelshift_l(ml, mh, lz) << 32 | (ml << lz)) + 0x200;
-  const u64 mant = n >> 10;
-  const int hi = (int)(mant >> 32) + es + ((1023 + 61 - lz) << 20);
-  return __hiloint2double(hi | sign, (int)mant);
+__device__ __forceinline__ double fx_to_double_int(long long g, int E) {
+  const u64 sm = (u64)(g >> 63);
+  const u64 sign = sm & 0x8000000000000000ull;
+  const u64 m = ((u64)g ^ sm) - sm;  // |g| < 2^63
+  const unsigned mh = (unsigned)(m >> 32);
+  if (mh == 0u) return fx_to_double_small(m, E, sign);
+  // value = m 2^(E - 55); with the leading one moved to bit 62,
+  // n = m 2^(lz - 1) and value = (n / 2^62) 2^(E + 8 - lz); lz >= 1 as m < 2^63
+  const int lz = __clz(mh);
+  const u64 n = m << (lz - 1);
+  const u64 mant = (n + 0x200) >> 10;  // 53 bits, 54 when the rounding carries
+  // the leading one of mant adds 1 to the exponent field (and a carry one more)
+  const u64 bits = ((u64)(long long)(1023 + 62 - kFxOut + E - lz) << 52) + mant;
+  return __longlong_as_double((long long)(bits | sign));
 }
 
-// The site values the equilibrium starts from (formats beside each).
+// The population of shell k.  The lowest bit of g is set first: g is never
+// zero (which the exponent add of the FP64 form needs), and it is 0.5 larger
+// on average, which the per-shell corrections of the equilibrium take into
+// account.
+__device__ __forceinline__ double fx_to_double(long long g, int E, int k) {
+  return ((D2Q37_INT_CVT_MASK >> k) & 1) ? fx_to_double_int(g | 1, E) : fx_to_double_fp64(g | 1, E);
+}
+
+// c v for a hop component c in -3..3 given the multiples m = {v, 2v, 3v}.
+__device__ __forceinline__ long long fx_hop_term(int c, const long long (&m)[3]) {
+  return c > 0 ? m[c - 1] : -m[-c - 1];
+}
+
+__device__ __forceinline__ long long fx_hop_dot(int cx, int cy, const long long (&mx)[3],
+                                                const long long (&my)[3]) {
+  if (cx == 0) return fx_hop_term(cy, my);
+  if (cy == 0) return fx_hop_term(cx, mx);
+  return fx_hop_term(cx, mx) + fx_hop_term(cy, my);
+}
+
+// Fixed-point site values: rho (Q61), u_x and u_bar_y = u_y + tau g_y (Q64),
+// theta = T_bar - 1 (Q62).
 struct FxSite {
-  long long R61;         // rho^
-  long long mx, my;      // Q64: rho^ U, rho^ V
-  long long U, V;        // Q64
-  long long rA, rB, AB;  // Q64: rho^ A, rho^ B, A + B
-  long long rq63;        // rho^ q
-  long long rth60;       // rho^ theta
-  long long X61;         // 1 / rho^
-  FxOp A, B;             // Q64
-  long long A64, B64;
-  int es;                // 2^20 log2(rho / rho^)
+  u64 R;
+  long long UX, UY, TH;
 };
 
-// 2^125 / rn for rn in [2^63, 2^64), within 3: the float reciprocal r0 of the
-// top 24 bits (24 bits, as an integer), e = 1 - rn r0 exactly, r0 (1 + e + e^2).
-__device__ __forceinline__ long long fx_recip61(u64 rn) {
-  const unsigned hi = (unsigned)(rn >> 32), lo = (unsigned)rn;
-  const unsigned rb = __float_as_uint(__frcp_rn(__int_as_float(0x4B000000 | (int)((hi >> 8) & 0x7FFFFF))));
-  // 2^47 / top: top = 2^23 gives 2^24, else below it
-  const unsigned s = ((rb & 0x7FFFFF) | 0x800000) << ((rb >> 23) - 103);
-  long long e = -(long long)((((u64)hi * s) << 24) + (((u64)lo * s) >> 8));  // Q79, mod 2^64; |e| < 2^57
-  const int eh = (int)(e >> 32);
-  e += ((long long)eh * eh) >> 15;
-  return (long long)((u64)s << 38) + (((e >> 18) * (long long)s) >> 23);
-}
-
-// The fixed-point site values from the exact moment sums (no FP64
-// arithmetic): rho^ = r 2^n 2^-64, rho^ U = s^2 jx / r rho^, 2 rho^ theta =
-// s^2 e - rho^ (|u|^2 + ...) with the shifts of Eq. MASTERSHIFT3 (unshifted u
-// in T, reading R6).  False when the site is outside the fixed-point ranges
-// (|u_x|, |u_bar_y| < 0.35, |theta| < 1) or its sums do not fit the scaled
-// forms; those sites take the FP64 collision.
+// The fixed-point site values straight from the exact moment sums (no FP64
+// arithmetic): with r normalised to rn = r 2^n in [2^63, 2^64), X = 2^126 / rn
+// from a float seed and two Newton steps (about 2^-60 relative), then
+// j / r = (j 2^n) X 2^-126, u = s j / r, 2 T = s^2 e / r - |u|^2 (unshifted u,
+// reading R6), rho = r 2^(emax - 1075).  False when the site is outside the
+// fixed-point ranges (rho in (0, 4), |u_x|, |u_bar_y| < 0.35, |theta| < 1) or
+// its sums do not fit the scaled forms; those sites take the FP64 collision.
 __device__ __forceinline__ bool fx_site_from_sums(long long r, long long jx, long long jy, long long e, int emax,
                                                   const StepParams& p, FxSite& o) {
-  if (!p.fx_on || r <= 0) return false;
+  if (!p.fx_on || r <= 0 || e < 0) return false;
   const u64 ur = (u64)r;
-  const long long h = (r >> 1) - (r >> 4);
-  const u64 h2 = 2 * (u64)h;
-  // |j| <= 7/16 r and 0 <= e < 3 r keep the scaled sums inside an fx_op (r <
-  // 37 2^53); the exponents leave room for those of the weights
-  if ((u64)(jx + h) >= h2 || (u64)(jy + h) >= h2 || (u64)e >= ur + ur + ur || emax < 256 || emax > 1792)
-    return false;
-  const int one = p.fx_one;
+  const u64 ajx = jx < 0 ? 0ull - (u64)jx : (u64)jx, ajy = jy < 0 ? 0ull - (u64)jy : (u64)jy;
+  // |j| < r / 2 and e < 3 r keep the scaled sums inside 64 bits (r < 37 2^53)
+  if ((ajx << 1) >= ur || (ajy << 1) >= ur || (u64)e >= ur + ur + ur) return false;
   const int n = __clzll(r);  // >= 5
-  const u64 rn = ur << n;    // Q64
-  const long long R60 = (long long)(rn >> 4);
-  const FxOp R62 = fx_op((long long)(rn >> 2));
-  const FxOp jnx = fx_op(fx_shl(jx, n)), jny = fx_op(fx_shl(jy, n));  // Q64
-  const FxOp s2 = fx_op(p.fx_s2_62);
-  const long long mx62 = fx_mul(jnx, s2, one);
-  const long long my62 = fx_mul(jny, s2, one) + fx_mul(R62, fx_op(p.fx_sd_64), one);
-  const long long lim = fx_shl(fx_mul(R62, fx_op(p.fx_lim_63), one), 1);  // Q62: 0.35 s rho^
-  if (mx62 >= lim || mx62 <= -lim || my62 >= lim || my62 <= -lim) return false;
-  o.X61 = fx_recip61(rn);
-  const FxOp X = fx_op(o.X61);
-  o.mx = fx_shl(mx62, 2);
-  o.my = fx_shl(my62, 2);
-  const FxOp mx = fx_op(o.mx), my = fx_op(o.my);
-  o.U = fx_shl(fx_mul(mx, X, one), 3);
-  o.V = fx_shl(fx_mul(my, X, one), 3);
-  const FxOp U = fx_op(o.U), V = fx_op(o.V);
-  o.A64 = fx_mul(U, U, one);
-  o.B64 = fx_mul(V, V, one);
-  o.AB = o.A64 + o.B64;
-  o.rA = fx_mul(mx, U, one);
-  o.rB = fx_mul(my, V, one);
-  o.rq63 = fx_mul(fx_op(o.rA + o.rB), fx_op(p.fx_is2_63), one);
-  // rho theta = s^2 e / 2 - rho q / 2 + tau g_y rho u_y - rho (u_y unshifted)
-  o.rth60 = fx_mul(fx_op(fx_shl(e, n - 3)), s2, one) - (o.rq63 >> 4) + fx_mul(jny, fx_op(p.fx_sd_60), one) - R60;
-  const long long tl = R60 - (1LL << 29);  // a margin that keeps 8 rho^ theta an fx_op
-  if (o.rth60 >= tl || o.rth60 <= -tl) return false;
-  o.R61 = (long long)(rn >> 3);
-  o.es = (emax - 1011 - n) << 20;  // rho = r 2^(emax - 1075) = rho^ 2^(64 - n + emax - 1075)
+  const u64 rn = ur << n;
+  const unsigned top = (unsigned)(rn >> 40);  // [2^23, 2^24), exactly a float below
+  const unsigned rb = __float_as_uint(__frcp_rn(__int_as_float(0x4B000000 | (int)(top & 0x7FFFFF))));
+  u64 X = (u64)((rb & 0x7FFFFF) | 0x800000) << (((rb >> 23) & 0xFF) - 64);  // 1/top 2^86, Q62 of 2^64/rn
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const u64 pq = __umul64hi(rn, X);          // Q62 of rn X, about 1
+    X = __umul64hi(X, (1ull << 63) - pq) << 2;  // X (2 - rn X), Q62; never above 2^64 / rn
+  }
+  const long long qx = mulhi_su((long long)((u64)jx << n), X);  // Q62 of jx / r
+  const long long qy = mulhi_su((long long)((u64)jy << n), X);
+  const long long ux61 = mulhi_su(qx, p.fx_s63);  // Q61 of u_x = s jx / r
+  const long long uy61 = mulhi_su(qy, p.fx_s63);
+  constexpr long long kU = 0x0B33333333333333LL;  // 0.35 2^61
+  if (ux61 >= kU || ux61 <= -kU) return false;
+  const long long UX = (long long)((u64)ux61 << 3);                      // Q64
+  const long long UY0 = (long long)((u64)uy61 << 3);                     // Q64, unshifted
+  const long long UY = UY0 + p.fx_uy_shift;                              // Q64 of u_bar_y
+  if (UY >= 0x5999999999999999LL || UY <= -0x5999999999999999LL) return false;  // 0.35 2^64
+  const u64 aux = UX < 0 ? 0ull - (u64)UX : (u64)UX, auy = UY0 < 0 ? 0ull - (u64)UY0 : (u64)UY0;
+  const u64 er = __umul64hi((u64)e << (n - 2), X);                      // Q60 of e / r (< 3)
+  const u64 s2er = __umul64hi(er, p.fx_s2_63);                           // Q59 of s^2 e / r
+  const u64 q0 = __umul64hi(aux, aux) + __umul64hi(auy, auy);            // Q64 of |u|^2
+  const long long th60 = (long long)s2er - (long long)(q0 >> 5) + p.fx_th_shift;  // Q60 of T + shift
+  if (th60 >= (1LL << 60) || th60 <= -(1LL << 60)) return false;
+  const int sR = emax - 1014;  // rho 2^61 = r 2^sR
+  u64 R;
+  if (sR >= 0) {
+    if (sR >= n) return false;
+    R = ur << sR;
+  } else {
+    const int rs = min(-sR, 63);
+    R = (ur + (1ull << (rs - 1))) >> rs;
+  }
+  if (R == 0 || R >= (1ull << 63)) return false;
+  o.R = R;
+  o.UX = UX;
+  o.UY = UY;
+  o.TH = (long long)((u64)th60 << 2);
   return true;
 }
 
@@ -395,103 +416,65 @@ struct ToPlanesStride {  // the same with the planes addressed as multiples of t
   __device__ __forceinline__ void put(int l, double v) const { d[l * plane] = v; }
 };
 
-// The relaxation of population l towards the equilibrium g 2^(es / 2^20).
-template <class O>
-__device__ __forceinline__ void fx_relax(const double (&f)[kQ], double keep, int es, int l, long long g, const O& out) {
-  out.put(l, fma(keep, f[l], fx_to_double(g, es)));
-}
-
-// The populations of one class of hops (shell K) from its parts; PX: the pair
-// of (cx, cy) (or of (cx, 0)), PY: the pair of (cx, -cy) (or of (0, cy)).
-// (cx, 0), (-cx, 0), (0, cy), (0, -cy)
-template <int K, int PX, int PY, class O>
-__device__ __forceinline__ void fx_axis(const double (&f)[kQ], const StepParams& p, int es0, long long ex, long long ox,
-                                        long long ey, long long oy, const O& out) {
-  const int es = es0 + p.fx_es[K];
-  const double keep = p.one_minus_omega;
-  fx_relax(f, keep, es, 1 + 2 * PX, ex + ox, out);
-  fx_relax(f, keep, es, 2 + 2 * PX, ex - ox, out);
-  fx_relax(f, keep, es, 1 + 2 * PY, ey + oy, out);
-  fx_relax(f, keep, es, 2 + 2 * PY, ey - oy, out);
-}
-
-// (cx, cy), (-cx, -cy), (cx, -cy), (-cx, cy)
-template <int K, int PX, int PY, class O>
-__device__ __forceinline__ void fx_diag(const double (&f)[kQ], const StepParams& p, int es0, long long ee, long long oe,
-                                        long long eo, long long oo, const O& out) {
-  const int es = es0 + p.fx_es[K];
-  const double keep = p.one_minus_omega;
-  const long long s = ee + oo, d = ee - oo, t = oe + eo, u = oe - eo;
-  fx_relax(f, keep, es, 1 + 2 * PX, s + t, out);
-  fx_relax(f, keep, es, 2 + 2 * PX, s - t, out);
-  fx_relax(f, keep, es, 1 + 2 * PY, d + u, out);
-  fx_relax(f, keep, es, 2 + 2 * PY, d - u, out);
-}
-
 // The collision of collide_site_fp64 below with the equilibrium in fixed
-// point, for a site inside the fixed-point ranges.  Every p is Q61; a part's
-// product with fx_w (c_k h^m 2^(fx_q(k) + 3), h the class's larger hop) is at
-// Q fx_q(k).
+// point (formats in the comments), for a site inside the fixed-point ranges.
 template <class O>
-__device__ __forceinline__ void collide_site_fx(const double (&f)[kQ], const StepParams& p, const FxSite& v,
+__device__ __forceinline__ void collide_site_fx(const double (&f)[kQ], const StepParams& p, const FxSite& fs,
                                                 const O& out) {
-  const int one = p.fx_one, two = p.fx_two;
-  const FxOp mx = fx_op(v.mx), my = fx_op(v.my), U = fx_op(v.U), V = fx_op(v.V);
-  const FxOp rA = fx_op(v.rA), rB = fx_op(v.rB), s2 = fx_op(p.fx_s2_62);
-  const long long rC = fx_mul(mx, V, one);
-  const long long q61 = fx_mul(fx_op(v.AB), fx_op(p.fx_is2_61), one);
-  const FxOp rth63 = fx_op(fx_shl(v.rth60, 3)), rq = fx_op(v.rq63);
-  const long long th62 = fx_shl(fx_mul(rth63, fx_op(v.X61), one), 2);
-  const FxOp th = fx_op(th62);
-  const long long Pq = fx_mul(rq, th, one), Pt = fx_mul(rth63, th, one);  // Q61: rho theta q, rho theta^2
-  const long long qq = fx_mul(rq, fx_op(q61), one);                 // Q60: rho q^2
-  const long long p00 = v.R61 - (v.rq63 >> 3) - fx_shl(v.rth60, 1) + (qq >> 2) + Pq + Pt;
-  const long long G = fx_mul(th, fx_op(p.fx_hs2_63), one), G2 = G >> 1;
-  const long long K1 = fx_shl(fx_mul(fx_op(fx_shl(v.rth60, 1) - (Pq >> 1) - fx_shl(Pt, 1)), s2, one), 1);
-  const long long K2 = fx_mul(fx_op(Pt), fx_op(p.fx_s4_64), one);
-  const long long L0 = (1LL << 61) - (q61 >> 1) - th62;
-  const FxOp M0 = fx_op((L0 - (th62 >> 1)) >> 1);
-  const long long A6 = fx_mul(fx_op(v.A64), fx_op(p.fx_sixth_61), one), B6 = fx_mul(fx_op(v.B64), fx_op(p.fx_sixth_61), one);
-  const long long p20 = K1 + fx_mul(rA, M0, one), p02 = K1 + fx_mul(rB, M0, one);
-  const long long p11 = fx_shl(fx_mul(fx_op(rC), M0, one), 1);
-  const long long p40 = K2 + fx_mul(rA, fx_op(G2 + (A6 >> 2)), one), p04 = K2 + fx_mul(rB, fx_op(G2 + (B6 >> 2)), one);
-  const long long p22 = fx_shl(K2, 1) + fx_mul2(rA, fx_op(G2 + (v.B64 >> 5)), rB, fx_op(G2), two);
-  const long long p30 = fx_mul(mx, fx_op(G + A6), one), p12 = fx_mul(mx, fx_op(G + (v.B64 >> 4)), one);
-  const long long p03 = fx_mul(my, fx_op(G + B6), one), p21 = fx_mul(my, fx_op(G + (v.A64 >> 4)), one);
-  const long long p31 = fx_mul(V, fx_op(p30), one), p13 = fx_mul(U, fx_op(p03), one);
-  const long long p10 = fx_mul(mx, fx_op(L0), one), p01 = fx_mul(my, fx_op(L0), one);
-  const int es = v.es;
-#define W(k, m) fx_op(p.fx_w[k][m])
-#define EE(k, t) fx_mul(fx_op(t), W(k, 0), one)
-#define EE2(k, t, t2) fx_mul2(fx_op(t), W(k, 0), fx_op(t2), W(k, 2), two)
-#define OD(k, m, t) fx_mul(fx_op(t), W(k, m), one)
-  fx_relax(f, p.one_minus_omega, es + p.fx_es[0], 0, EE(0, p00), out);
-  const long long ex1 = p00 + p20 + p40, ey1 = p00 + p02 + p04;  // p00 + X1, p00 + Y1
-  {
-    const long long a = p10 + p30, b = p01 + p03;
-    fx_axis<1, 0, 1>(f, p, es, EE(1, ex1), OD(1, 0, a), EE(1, ey1), OD(1, 0, b), out);
-    fx_diag<2, 2, 3>(f, p, es, EE(2, ex1 + p02 + p04 + p22), OD(2, 0, a + p12), OD(2, 0, b + p21),
-                     OD(2, 0, p11 + p31 + p13), out);
+  const long long UX = fs.UX, UY = fs.UY;  // Q64
+  const long long TH = fs.TH;              // Q62
+  const u64 R = fs.R;                      // Q61
+  const u64 AUX = UX < 0 ? 0ull - (u64)UX : (u64)UX, AUY = UY < 0 ? 0ull - (u64)UY : (u64)UY;
+  const u64 q = __umul64hi(AUX, AUX) + __umul64hi(AUY, AUY);  // Q64
+  const u64 q2 = __umul64hi(q, q);                            // Q64
+  const u64 B1 = (1ull << 62) - (q >> 3);                     // Q62: 1 - q/2
+  const u64 B2 = (1ull << 61) - (q >> 4);                     //      1/2 - q/4
+  const u64 A0 = B1 + (q2 >> 5);                              //      1 - q/2 + q^2/8
+  const long long SX = mulhi_su(UX, p.fx_s62), SY = mulhi_su(UY, p.fx_s62);  // Q62
+  const long long rA0 = (long long)__umul64hi(R, A0);        // Q59
+  const long long rB1 = (long long)__umul64hi(R, B1);        // Q59
+  const long long rB2 = (long long)__umul64hi(R, B2);        // Q59
+  const long long rth = mul_shift((long long)R, TH, 62);     // Q61: rho theta
+  const long long rth2 = mul_shift(rth, TH, 62);             // Q61: rho theta^2
+  const long long rthq = mulhi_su(rth, q);                   // Q61: rho theta q
+  const long long K0 = rA0 - (rth >> 2) + (rthq >> 2) + (rth2 >> 2);  // Q59
+  const long long K1 = (rth >> 2) - (rthq >> 3) - (rth2 >> 1);        // Q60
+  const u64 K2 = (u64)rth2;                                           // Q64 (rho theta^2 / 8)
+  const long long L0 = rB1 - (rth >> 1);                              // Q59
+  const long long M0 = rB2 - (rth >> 2) - (rth >> 3);                 // Q59
+  const long long mx[3] = {SX, SX + SX, SX + SX + SX};                // Q62
+  const long long my[3] = {SY, SY + SY, SY + SY + SY};
+  const u64 kSign = 1ull << 63;
+  const u64 uK0 = (u64)K0, uK1 = (u64)K1 ^ kSign, uL0 = (u64)L0 ^ kSign;  // x + 2^63
+  const u64 uM0 = (u64)M0 ^ kSign, uTH = (u64)rth ^ kSign;                // L1 = M1 = rth
+  const double keep = p.one_minus_omega;
+  out.put(0, fma(keep, f[0], fx_to_double((long long)(__umul64hi(uK0, p.fx_c60[0]) - p.fx_d0[0]), p.fx_e[0], 0)));  // x2 = 0
+#pragma unroll
+  for (int k = 1; k < kShells; ++k) {
+    const long long R0 = (long long)(__umul64hi(uK0, p.fx_c60[k]) + __umul64hi(uK1, p.fx_cx2_59[k]) +
+                                     __umul64hi(K2, p.fx_cx4_55[k]) - p.fx_d0[k]);  // Q55
+    const long long R1 = (long long)(__umul64hi(uL0, p.fx_c62[k]) + __umul64hi(uTH, p.fx_cx2_59[k]) -
+                                     p.fx_d1[k]);  // Q57
+    const long long R2 = (long long)(__umul64hi(uM0, p.fx_c64[k]) + __umul64hi(uTH, p.fx_cx2_60[k]) -
+                                     p.fx_d2[k]);  // Q59
+    const u64 R3 = __umul64hi(R, p.fx_c6[k]);  // Q61 of c rho / 6, and Q63 of R4 = c rho / 24
+    const int E = p.fx_e[k];
+#pragma unroll
+    for (int pr = 0; pr < kPairs; ++pr) {
+      if (pair_shell(pr) != k) continue;
+      const long long a = fx_hop_dot(pair_cx(pr), pair_cy(pr), mx, my);  // Q62
+      const long long sa = a >> 63;                                      // 0 or -1
+      const u64 A = (u64)((a ^ sa) - sa);
+      const u64 b = umulhi_t(A, A);                                      // Q60
+      const long long t = R2 + (long long)umulhi_t(b, R3);              // Q59: R2 + b R4
+      const long long even = R0 + mulhi_su_t(t, b);                      // Q55
+      const long long s = R1 + (long long)umulhi_t(b, R3);              // Q57
+      const long long oa = mulhi_su_rn(s, A);                            // Q55: |a| (R1 + b R3)
+      const long long odd = (oa ^ sa) - sa;                              // the sign of a
+      out.put(1 + 2 * pr, fma(keep, f[1 + 2 * pr], fx_to_double(even + odd, E, k)));
+      out.put(2 + 2 * pr, fma(keep, f[2 + 2 * pr], fx_to_double(even - odd, E, k)));
+    }
   }
-  const long long a1 = p10 + p30, a2 = p10 + 4 * p30, b1 = p01 + p03, b2 = p01 + 4 * p03;
-  const long long x2 = p20 + 4 * p40, y2 = p02 + 4 * p04;
-  fx_axis<3, 4, 5>(f, p, es, EE2(3, p00, x2), OD(3, 1, a2), EE2(3, p00, y2), OD(3, 1, b2), out);
-  fx_diag<4, 6, 7>(f, p, es, EE2(4, ey1, x2 + p22), OD(4, 1, a2 + p12), OD(4, 0, b1 + 4 * p21),
-                   OD(4, 1, p11 + 4 * p31 + p13), out);
-  fx_diag<4, 8, 9>(f, p, es, EE2(4, ex1, y2 + p22), OD(4, 0, a1 + 4 * p12), OD(4, 1, b2 + p21),
-                   OD(4, 1, p11 + p31 + 4 * p13), out);
-  fx_diag<5, 10, 11>(f, p, es, EE2(5, p00, x2 + y2 + 4 * p22), OD(5, 1, a2 + 4 * p12), OD(5, 1, b2 + 4 * p21),
-                     OD(5, 2, p11 + 4 * (p31 + p13)), out);
-  const long long a3 = p10 + 9 * p30, b3 = p01 + 9 * p03, x3 = p20 + 9 * p40, y3 = p02 + 9 * p04;
-  fx_axis<6, 12, 13>(f, p, es, EE2(6, p00, x3), OD(6, 1, a3), EE2(6, p00, y3), OD(6, 1, b3), out);
-  fx_diag<7, 14, 15>(f, p, es, EE2(7, ey1, x3 + p22), OD(7, 1, a3 + p12), OD(7, 0, b1 + 9 * p21),
-                     OD(7, 1, p11 + 9 * p31 + p13), out);
-  fx_diag<7, 16, 17>(f, p, es, EE2(7, ex1, y3 + p22), OD(7, 0, a1 + 9 * p12), OD(7, 1, b3 + p21),
-                     OD(7, 1, p11 + p31 + 9 * p13), out);
-#undef W
-#undef EE
-#undef EE2
-#undef OD
 }
 
 // BGK collision of one site, f <- f - (f - f^eq(rho, u_bar, T_bar)) / tau with

@@ -115,19 +115,6 @@ struct ShellConsts32 {
   float delta[kShells], eps[kShells];  // (x2 - 4)/2, (x2 - 6)/4
 };
 
-// A constant of the fixed-point equilibrium as hi 2^32 + lo with a signed low
-// word (the operand form of its products).
-struct FxConst {
-  int lo, hi;
-};
-
-// Format of the fixed-point results of shell k (see collide_site_fx): the
-// largest for which the products with its weights fit.
-__host__ __device__ constexpr int fx_q(int k) { return k < 3 ? 59 : k == 5 ? 56 : 57; }
-
-// The larger component of shell k's hops.
-__host__ __device__ constexpr int shell_hop(int k) { return k == 0 ? 0 : k < 3 ? 1 : k < 6 ? 2 : 3; }
-
 // Per-lattice parameters of one step, passed by value to every kernel.
 struct StepParams {
   int Lx, Ly;
@@ -152,22 +139,23 @@ struct StepParams {
   float fwmw32[2][kQ];  // fw - w
   float wall_e32[2][2];   // (hi, lo): sum_M fwmw32 - sum_O w + sum_M w (M missing, O leaving pairs)
   float wall_inv32[2][2]; // (hi, lo): 1 / sum_M fw32
-  // Fixed-point equilibrium constants of the FP64 step, each at the scale its
-  // name ends in (d = tau g_y):
-  FxConst fx_s2_62;             // s^2
-  FxConst fx_sd_64, fx_sd_60;   // s d
-  FxConst fx_lim_63;            // 0.35 s
-  FxConst fx_is2_63, fx_is2_61; // 1 / s^2
-  FxConst fx_hs2_63;            // s^2 / 2
-  FxConst fx_s4_64;             // s^4 / 8
-  FxConst fx_sixth_61;          // 1 / 6
-  // per shell k, omega w_k = c_k 2^E_k with c_k in [0.5, 1) (hops of 3: in
-  // [4/9, 8/9), so that 9 c_k < 8): c_k h^m
-  // 2^(fx_q(k) + 3), h = max(|cx|, |cy|) of the shell's hops, m = 0, 1, 2, and
-  // (E_k - fx_q(k)) 2^20
-  FxConst fx_w[kShells][3];
-  int fx_es[kShells];
-  int fx_one, fx_two;         // 1 and 2 (see fx_mul)
+  // Fixed-point equilibrium constants of the FP64 step: per shell k,
+  // omega w_k = c_k 2^fx_e[k] with c_k in [0.5, 1); as unsigned integers, each
+  // at the scale that puts its product straight into the format it feeds:
+  // c 2^60, 2^62, 2^64; c x2 2^59, 2^60; c x2^2 2^55; (c/6) 2^64, which is
+  // also (c/24) 2^66 (x2 = s^2 |c_l|^2).
+  unsigned long long fx_c60[kShells], fx_c62[kShells], fx_c64[kShells];
+  unsigned long long fx_cx2_59[kShells], fx_cx2_60[kShells], fx_cx4_55[kShells];
+  unsigned long long fx_c6[kShells];
+  // subtracted from R0, R1, R2 (mod 2^64): y / 2 for each product whose site
+  // value enters with its sign bit flipped (x + 2^63), less a rounding
+  // correction
+  unsigned long long fx_d0[kShells], fx_d1[kShells], fx_d2[kShells];
+  int fx_e[kShells];
+  unsigned long long fx_s62;  // s 2^62
+  unsigned long long fx_s63, fx_s2_63;  // s 2^63, s^2 2^63
+  long long fx_uy_shift;      // tau g_y 2^64
+  long long fx_th_shift;      // (theta_shift) 2^60 = (-tau^2 g^2 / 2 - 1) 2^60
   int fx_on;                  // 0: the shifts do not fit the formats, every site takes FP64
 };
 
