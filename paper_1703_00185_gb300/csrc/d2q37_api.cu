@@ -44,7 +44,7 @@ void fill_fixed_consts(StepParams& sp) {
     const double wl = std::fma(sp.omega, c.w[k], -wh);
     int E;
     std::frexp(wh, &E);  // wh = m 2^E, m in [0.5, 1)
-    sp.fx_e[k] = E;
+    sp.fx_es[k] = (E - 55) * (1 << 20);
     const double ch = std::ldexp(wh, -E), cl = std::ldexp(wl, -E);
     const double x2 = c.s2 * shell_c2(k);
     const double x2h = x2, x2l = std::fma(c.s2, (double)shell_c2(k), -x2);  // exact: c.s2 times a small integer
@@ -119,6 +119,13 @@ int ensure_device_consts() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return LBM_ECUDA;
   std::lock_guard<std::mutex> lock(g_dev_mutex);
   if (!g_dev_ready[dev]) {
+    if (!g_consts.late) {  // one word for the process, mapped on every device
+      void* w = nullptr;
+      if (cudaHostAlloc(&w, sizeof(unsigned), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess)
+        return LBM_ENOMEM;
+      g_consts.late = (unsigned*)w;
+      *g_consts.late = 0;
+    }
     if (upload_shell_consts(g_consts) != cudaSuccess) return LBM_ECUDA;
     if (upload_shell_consts32(g_consts32) != cudaSuccess) return LBM_ECUDA;
     g_dev_ready[dev] = true;
@@ -417,6 +424,14 @@ int handle_prepare_halos(lbm_t* h, cudaStream_t stream) {
   return LBM_OK;
 }
 
+int handle_sync(cudaStream_t stream) {
+  const int rc = check(cudaStreamSynchronize(stream));
+  volatile unsigned* late = g_consts.late;
+  if (rc || !late || !*late) return rc;
+  *late = 0;
+  return LBM_ETIMEOUT;
+}
+
 int handle_device_consts() {
   if (!quadrature_ready()) return LBM_ESTATE;
   return ensure_device_consts();
@@ -648,7 +663,7 @@ int lbm_fields(lbm_t* h, double* rho, double* u, double* T) {
 
 int lbm_synchronize(lbm_t* h) {
   if (!h) return LBM_EINVAL;
-  return check(cudaStreamSynchronize(h->stream));
+  return handle_sync(h->stream);
 }
 
 int64_t lbm_launch_count(const lbm_t* h) { return h ? h->launches : 0; }

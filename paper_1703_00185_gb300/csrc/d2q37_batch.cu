@@ -476,7 +476,7 @@ int lbm_batch_autotune(lbm_batch_t* b, int trial_steps, int* block_y, int* block
 
 int lbm_batch_synchronize(lbm_batch_t* b) {
   if (!b) return LBM_EINVAL;
-  return check(cudaStreamSynchronize(b->stream));
+  return handle_sync(b->stream);
 }
 
 int64_t lbm_batch_launch_count(const lbm_batch_t* b) { return b ? b->launches : 0; }

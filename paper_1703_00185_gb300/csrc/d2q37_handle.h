@@ -63,6 +63,10 @@ constexpr int kLongGraphSteps = 16;
 // Launch the pbc kernel on `stream` if the handle's halos are stale.
 int handle_prepare_halos(lbm_t* h, cudaStream_t stream);
 
+// Wait for the stream; LBM_ETIMEOUT when a kernel's bounded wait has run out
+// since the last call.
+int handle_sync(cudaStream_t stream);
+
 // Quadrature constants on the current device (0 or an LBM_E* code).
 int handle_device_consts();
 

@@ -34,13 +34,6 @@ namespace {
 constexpr int kBlockY = 256;
 constexpr int kWallBlock = 128;
 
-// Minimum resident blocks per SM requested for the FP64 site kernels (caps
-// their registers at 65536 / (kBlockY * blocks)); tuned on GB300: 2 blocks of
-// 256 (128 registers) ran the 2048 x 8192 fused step in 2.79 ms, against
-// 2.84 ms with 8 of 64, 2.87 ms with 4 of 128 and 3.53 ms with 1 of 512.
-#ifndef D2Q37_SITE_MIN_BLOCKS
-#define D2Q37_SITE_MIN_BLOCKS 2
-#endif
 // The batched kernel (D2Q37_BATCH_MIN_BLOCKS x 128 threads per SM, whatever
 // its block_y) reads its parameters from memory instead of the constant bank
 // and spills a little at 128 registers (20 bytes per thread); with 3 blocks of
@@ -56,6 +49,13 @@ template <class P>
 __device__ __forceinline__ long long site_index(const P& p, int x, int y) {
   return (long long)(x + kHx) * p.NY + (y + p.Hy);
 }
+
+// Where a site's populations are: in registers, or in the block's shared
+// memory (RowPops), read again each time they are needed.
+struct RegPops {
+  const double (&f)[kQ];
+  __device__ __forceinline__ double get(int l) const { return f[l]; }
+};
 
 // rho, u and T of one site (Sec. "Lattice Boltzmann methods"):
 // rho = sum f, rho u = s sum c f, D rho T = sum |xi|^2 f - rho |u|^2 (D = 2),
@@ -107,39 +107,59 @@ __device__ __forceinline__ void site_moments_fp64(const double (&f)[kQ], double&
 // NaN take the FP64 form.
 constexpr long long kFloorR = 16, kFloorE = 105;
 
-__device__ __forceinline__ long long fixed_term(double v, int emax) {
+// top2 = 2 (2^20 emax + 2^20 - 1): the shift emax - e in two instructions, the
+// doubling dropping the sign bit (the mantissa bits borrow nothing).
+__device__ __forceinline__ long long fixed_term(double v, unsigned top2, unsigned& wrap) {
   const int hi = __double2hiint(v);
-  const unsigned lo = (unsigned)__double2loint(v);
-  const int e = (hi >> 20) & 0x7FF;
+  const unsigned d = top2 - 2u * (unsigned)hi;
+  wrap = max(wrap, d);  // above top2: v has a larger exponent than emax
+  const unsigned sh = d >> 21;
+  const int s = hi >> 31;  // 0 or -1
   // the implicit one is set for zero and subnormal inputs too: with emax >= 64
-  // their shift is the full 62 and they round to 0 (-1 for a negative zero)
-  const long long mant = ((long long)((hi & 0xFFFFF) | 0x100000) << 32) | lo;
-  const int sh = min(emax - e, 62);
-  const long long s = hi >> 31;  // 0 or -1
-  // a negative v as the one's complement of its magnitude, -mant - 1: its
+  // their shift is above 62 and they round to 0 (-1 for a negative zero).  A
+  // negative v enters as the one's complement of its magnitude, -mant - 1: its
   // arithmetic shift is floor(v 2^-sh) or, when the dropped bits are all zero,
   // one below it
-  return (mant ^ s) >> sh;
+  const int mh = ((hi & 0xFFFFF) | 0x100000) ^ s;
+  const int ml = __double2loint(v) ^ s;
+  long long r;  // PTX clamps shifts above 63 (C++ leaves them undefined)
+  asm("{\n\t.reg .b64 m;\n\tmov.b64 m, {%1, %2};\n\tshr.s64 %0, m, %3;\n\t}" : "=l"(r) : "r"(ml), "r"(mh), "r"(sh));
+  return r;
+}
+
+// The population of the largest magnitude (by its high word).
+template <class F>
+__device__ __forceinline__ double largest(const F& f) {
+  double m = 0.0;
+#pragma unroll
+  for (int l = 0; l < kQ; ++l) {
+    const double v = f.get(l);
+    if ((__double2hiint(v) & 0x7FFFFFFF) > (__double2hiint(m) & 0x7FFFFFFF)) m = v;
+  }
+  return m;
 }
 
 // The exact sums r = sum f, jx, jy = sum c f, e = sum |c|^2 f on the grid
-// 2^(emax - 1075); false for the sites that take the FP64 sums.
-__device__ __forceinline__ bool site_sums(const double (&f)[kQ], long long& r, long long& jx, long long& jy,
+// 2^(emax - 1075), emax the largest exponent.  ANY = false takes the rest
+// population's for it, which near equilibrium it is (w_0 is twice the next
+// weight), and returns false when it is not; then, with ANY = true, false is
+// left for the sites that take the FP64 sums.
+template <bool ANY, class F>
+__device__ __forceinline__ bool site_sums(const F& f, long long& r, long long& jx, long long& jy,
                                           long long& e, int& emax) {
-  int hmax = 0;  // the largest |high word|: its exponent field is the largest exponent
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) hmax = max(hmax, __double2hiint(f[l]) & 0x7FFFFFFF);
-  emax = hmax >> 20;
-  if (emax < 64 || emax > 2046) return false;
+  const int top = __double2hiint(ANY ? largest(f) : f.get(0));
+  emax = top >> 20 & 0x7FF;
+  const unsigned top2 = 2u * (unsigned)(top | 0xFFFFF);
+  unsigned wrap = 0;
   long long sh[kShells];
-  sh[0] = fixed_term(f[0], emax);
+  sh[0] = fixed_term(f.get(0), top2, wrap);
 #pragma unroll
   for (int k = 1; k < kShells; ++k) sh[k] = 0;
   jx = jy = 0;
 #pragma unroll
   for (int p = 0; p < kPairs; ++p) {
-    const long long vp = fixed_term(f[1 + 2 * p], emax);
-    const long long vm = fixed_term(f[2 + 2 * p], emax);
+    const long long vp = fixed_term(f.get(1 + 2 * p), top2, wrap);
+    const long long vm = fixed_term(f.get(2 + 2 * p), top2, wrap);
     sh[pair_shell(p)] += vp + vm;
     const long long d = vp - vm;
     jx += pair_cx(p) * d;
@@ -152,7 +172,7 @@ __device__ __forceinline__ bool site_sums(const double (&f)[kQ], long long& r, l
     r += sh[k];
     e += shell_c2(k) * sh[k];
   }
-  return true;
+  return wrap <= top2 && emax >= 64 && emax <= 2046;
 }
 
 __device__ __forceinline__ void moments_from_sums(long long r, long long jx, long long jy, long long e, int emax,
@@ -169,7 +189,7 @@ __device__ __forceinline__ void site_moments(const double (&f)[kQ], double& rho,
                                              double& T) {
   long long r, jx, jy, e;
   int emax;
-  if (site_sums(f, r, jx, jy, e, emax))
+  if (site_sums<true>(RegPops{f}, r, jx, jy, e, emax))
     moments_from_sums(r, jx, jy, e, emax, rho, ux, uy, T);
   else
     site_moments_fp64(f, rho, ux, uy, T);
@@ -232,17 +252,27 @@ __device__ __forceinline__ long long mulhi_su(long long x, u64 y) {
   return (long long)(__umul64hi((u64)x, y) - (y & (u64)(x >> 63)));  // x >> 63: 0 or all ones
 }
 
-// The high word of a y with the low-by-low partial product left out: three
-// 32 x 32 -> 64-bit multiply-adds and one add, the floor of a y 2^-64 or one
-// below it (0.75 below a y 2^-64 on average).  More instructions than the
-// exact high word but a shorter dependency chain: the per-pair products,
-// which form one chain per pair, take this form.
+// The high word of a y with the low-by-low partial product left out, the floor
+// of a y 2^-64 or one below it (0.75 below on average).
 __device__ __forceinline__ u64 umulhi_t(u64 a, u64 y) {
   const unsigned al = (unsigned)a, ah = (unsigned)(a >> 32);
   const unsigned yl = (unsigned)y, yh = (unsigned)(y >> 32);
   const u64 lh = (u64)al * yh;
   const u64 hl = (u64)ah * yl + (lh & 0xFFFFFFFFull);  // < 2^64
   return (u64)ah * yh + (lh >> 32) + (hl >> 32);
+}
+
+// The same for a, y < 2^63, whose cross sum fits 64 bits: three 32 x 32 ->
+// 64-bit multiply-adds (the per-pair products, which form one chain per pair).
+__device__ __forceinline__ u64 umulhi_t63(u64 a, u64 y) {
+  const unsigned al = (unsigned)a, ah = (unsigned)(a >> 32);
+  const unsigned yl = (unsigned)y, yh = (unsigned)(y >> 32);
+  u64 r;
+  asm("{\n\t.reg .b64 m;\n\tmul.wide.u32 m, %1, %4;\n\tmad.wide.u32 m, %2, %3, m;\n\tshr.u64 m, m, 32;\n\t"
+      "mad.wide.u32 %0, %2, %4, m;\n\t}"
+      : "=l"(r)
+      : "r"(al), "r"(ah), "r"(yl), "r"(yh));
+  return r;
 }
 
 // umulhi_t for signed x: x y = (x mod 2^64) y - 2^64 y [x < 0]
@@ -272,58 +302,50 @@ __device__ __forceinline__ long long mul_shift(long long x, long long y, int sh)
   return (long long)((h << (64 - sh)) | (l >> sh));
 }
 
-// g 2^(E - 55) as an FP64 number, two ways: with the FP64 pipe's 64-bit
-// integer conversion (round to nearest even) and the power of two added to
-// the exponent field, or with integer operations only (round half away from
-// zero).  The shells k whose bit is set in D2Q37_INT_CVT_MASK take the
-// integer form.  On GB300, with the FP64 pipe about 75 % busy, the last
-// shell's 8 populations that way (0x80) ran the 2048 x 8192 step in 2.742 ms,
-// against 2.784 ms for none, 2.802 / 2.847 ms for the last two / three
-// shells and 2.74-2.82 ms for shell 7 with one of shells 1, 3, 4, 5 (all of
-// them, with 4 blocks of 128 per SM: 4.37 against 4.12).
-#ifndef D2Q37_INT_CVT_MASK
-#define D2Q37_INT_CVT_MASK 0x80
-#endif
-
-// g != 0
-__device__ __forceinline__ double fx_to_double_fp64(long long g, int E) {
+// g 2^(E - 55) as an FP64 number for odd g, es = (E - 55) 2^20 added to the
+// exponent field, two ways: the FP64 pipe's 64-bit integer conversion (round
+// to nearest even), or integer operations only (half away from zero).  The
+// last shell's 8 populations take the integer form: the FP64 pipe is the
+// busiest unit (70 %) and the ALU second (55 %); 2048 x 8192 step 2.46 ms,
+// the last two shells 2.45 ms, the last four 2.49 ms, all of them 2.61 ms.
+__device__ __forceinline__ double fx_to_double_fp64(long long g, int es) {
   const double d = (double)g;  // exact up to its one rounding
-  const u64 bits = (u64)__double_as_longlong(d) + ((u64)(long long)(E - kFxOut) << 52);
-  return __longlong_as_double((long long)bits);
+  return __hiloint2double(__double2hiint(d) + es, __double2loint(d));
 }
 
-// |g| < 2^32 (including 0): the general normalisation
-__device__ __noinline__ double fx_to_double_small(u64 m, int E, u64 sign) {
-  if (!m) return 0.0;
-  const int lz = __clzll((long long)m);
-  const u64 n = m << (lz - 1);  // leading one at bit 62
-  const u64 mant = (n + 0x200) >> 10;
-  const u64 bits = ((u64)(long long)(1023 + 62 - kFxOut + E - lz) << 52) + mant;
-  return __longlong_as_double((long long)(bits | sign));
+// |g| >= 2^32
+__device__ __forceinline__ double fx_to_double_int(long long g, int es) {
+  const int gh = (int)(g >> 32), sm = gh >> 31;
+  const unsigned mh = (unsigned)(gh ^ sm), ml = ((unsigned)g ^ (unsigned)sm) | 1u;  // |g|: odd
+  // the leading one moved to bit 62 (|g| < 2^63), rounded to 53 bits, 54 when
+  // the rounding carries; it adds 1 to the exponent field, a carry one more
+  const int lz = __clz((int)mh) - 1;
+  const u64 n = ((u64)__funnelshift_l(ml, mh, lz) << 32 | (ml << lz)) + 0x200;
+  const u64 mant = n >> 10;
+  const int hi = (int)(mant >> 32) + (es + ((1023 + 61) << 20)) - (lz << 20);
+  return __hiloint2double(hi | (sm & (int)0x80000000), (int)mant);
 }
 
-__device__ __forceinline__ double fx_to_double_int(long long g, int E) {
-  const u64 sm = (u64)(g >> 63);
-  const u64 sign = sm & 0x8000000000000000ull;
-  const u64 m = ((u64)g ^ sm) - sm;  // |g| < 2^63
-  const unsigned mh = (unsigned)(m >> 32);
-  if (mh == 0u) return fx_to_double_small(m, E, sign);
-  // value = m 2^(E - 55); with the leading one moved to bit 62,
-  // n = m 2^(lz - 1) and value = (n / 2^62) 2^(E + 8 - lz); lz >= 1 as m < 2^63
-  const int lz = __clz(mh);
-  const u64 n = m << (lz - 1);
-  const u64 mant = (n + 0x200) >> 10;  // 53 bits, 54 when the rounding carries
-  // the leading one of mant adds 1 to the exponent field (and a carry one more)
-  const u64 bits = ((u64)(long long)(1023 + 62 - kFxOut + E - lz) << 52) + mant;
-  return __longlong_as_double((long long)(bits | sign));
+// The same for any odd g.
+__device__ __forceinline__ double fx_to_double_int_any(long long g, int es) {
+  const u64 m = g < 0 ? 0ull - (u64)g : (u64)g;
+  const int lz = __clzll((long long)m) - 1;
+  const u64 mant = ((m << lz) + 0x200) >> 10;
+  const int hi = (int)(mant >> 32) + es + ((1023 + 61 - lz) << 20);
+  return __hiloint2double(g < 0 ? hi | (int)0x80000000 : hi, (int)mant);
 }
 
-// The population of shell k.  The lowest bit of g is set first: g is never
-// zero (which the exponent add of the FP64 form needs), and it is 0.5 larger
-// on average, which the per-shell corrections of the equilibrium take into
-// account.
-__device__ __forceinline__ double fx_to_double(long long g, int E, int k) {
-  return ((D2Q37_INT_CVT_MASK >> k) & 1) ? fx_to_double_int(g | 1, E) : fx_to_double_fp64(g | 1, E);
+// The equilibrium of a population of shell k from its fixed-point value, whose
+// lowest bit is set first: it is never zero, and 0.5 larger on average, which
+// the per-shell corrections of the equilibrium take into account.  ANY =
+// false: the integer form's short version, keeping in `low` the smallest |high
+// word| (0: some value needed the other).
+template <bool ANY>
+__device__ __forceinline__ double fx_convert(int k, long long g, int es, int& low) {
+  if (k != kShells - 1) return fx_to_double_fp64(g | 1, es);
+  if (ANY) return fx_to_double_int_any(g | 1, es);
+  low = min(low, (int)(g >> 32) ^ (int)(g >> 63));
+  return fx_to_double_int(g, es);
 }
 
 // c v for a hop component c in -3..3 given the multiples m = {v, 2v, 3v}.
@@ -352,8 +374,9 @@ struct FxSite {
 // reading R6), rho = r 2^(emax - 1075).  False when the site is outside the
 // fixed-point ranges (rho in (0, 4), |u_x|, |u_bar_y| < 0.35, |theta| < 1) or
 // its sums do not fit the scaled forms; those sites take the FP64 collision.
+template <class P>
 __device__ __forceinline__ bool fx_site_from_sums(long long r, long long jx, long long jy, long long e, int emax,
-                                                  const StepParams& p, FxSite& o) {
+                                                  const P& p, FxSite& o) {
   if (!p.fx_on || r <= 0 || e < 0) return false;
   const u64 ur = (u64)r;
   const u64 ajx = jx < 0 ? 0ull - (u64)jx : (u64)jx, ajy = jy < 0 ? 0ull - (u64)jy : (u64)jy;
@@ -418,9 +441,12 @@ struct ToPlanesStride {  // the same with the planes addressed as multiples of t
 
 // The collision of collide_site_fp64 below with the equilibrium in fixed
 // point (formats in the comments), for a site inside the fixed-point ranges.
-template <class O>
-__device__ __forceinline__ void collide_site_fx(const double (&f)[kQ], const StepParams& p, const FxSite& fs,
-                                                const O& out) {
+// ANY = false: false is returned when some equilibrium needs the general
+// conversion (it is within 2^32 units of 0); the populations written are then
+// to be written again with ANY = true.  One test a site: in each conversion it
+// cost as much as the conversion.
+template <bool ANY, class F, class P, class O>
+__device__ __forceinline__ bool collide_site_fx(const F& f, const P& p, const FxSite& fs, const O& out) {
   const long long UX = fs.UX, UY = fs.UY;  // Q64
   const long long TH = fs.TH;              // Q62
   const u64 R = fs.R;                      // Q61
@@ -448,7 +474,9 @@ __device__ __forceinline__ void collide_site_fx(const double (&f)[kQ], const Ste
   const u64 uK0 = (u64)K0, uK1 = (u64)K1 ^ kSign, uL0 = (u64)L0 ^ kSign;  // x + 2^63
   const u64 uM0 = (u64)M0 ^ kSign, uTH = (u64)rth ^ kSign;                // L1 = M1 = rth
   const double keep = p.one_minus_omega;
-  out.put(0, fma(keep, f[0], fx_to_double((long long)(__umul64hi(uK0, p.fx_c60[0]) - p.fx_d0[0]), p.fx_e[0], 0)));  // x2 = 0
+  int low = 0x7FFFFFFF;
+  out.put(0, fma(keep, f.get(0),
+                 fx_convert<ANY>(0, (long long)(__umul64hi(uK0, p.fx_c60[0]) - p.fx_d0[0]), p.fx_es[0], low)));  // x2 = 0
 #pragma unroll
   for (int k = 1; k < kShells; ++k) {
     const long long R0 = (long long)(__umul64hi(uK0, p.fx_c60[k]) + __umul64hi(uK1, p.fx_cx2_59[k]) +
@@ -458,31 +486,35 @@ __device__ __forceinline__ void collide_site_fx(const double (&f)[kQ], const Ste
     const long long R2 = (long long)(__umul64hi(uM0, p.fx_c64[k]) + __umul64hi(uTH, p.fx_cx2_60[k]) -
                                      p.fx_d2[k]);  // Q59
     const u64 R3 = __umul64hi(R, p.fx_c6[k]);  // Q61 of c rho / 6, and Q63 of R4 = c rho / 24
-    const int E = p.fx_e[k];
+    const int es = p.fx_es[k];
 #pragma unroll
     for (int pr = 0; pr < kPairs; ++pr) {
       if (pair_shell(pr) != k) continue;
       const long long a = fx_hop_dot(pair_cx(pr), pair_cy(pr), mx, my);  // Q62
       const long long sa = a >> 63;                                      // 0 or -1
       const u64 A = (u64)((a ^ sa) - sa);
-      const u64 b = umulhi_t(A, A);                                      // Q60
-      const long long t = R2 + (long long)umulhi_t(b, R3);              // Q59: R2 + b R4
+      const u64 b = umulhi_t63(A, A);                                    // Q60; A < 1.7 2^62
+      const long long bR3 = (long long)umulhi_t63(b, R3);                // b < 2.9 2^60, R3 < 2^61
+      const long long t = R2 + bR3;                                      // Q59: R2 + b R4
       const long long even = R0 + mulhi_su_t(t, b);                      // Q55
-      const long long s = R1 + (long long)umulhi_t(b, R3);              // Q57
+      const long long s = R1 + bR3;                                      // Q57
       const long long oa = mulhi_su_rn(s, A);                            // Q55: |a| (R1 + b R3)
       const long long odd = (oa ^ sa) - sa;                              // the sign of a
-      out.put(1 + 2 * pr, fma(keep, f[1 + 2 * pr], fx_to_double(even + odd, E, k)));
-      out.put(2 + 2 * pr, fma(keep, f[2 + 2 * pr], fx_to_double(even - odd, E, k)));
+      const double gp = fx_convert<ANY>(k, even + odd, es, low);
+      const double gm = fx_convert<ANY>(k, even - odd, es, low);
+      out.put(1 + 2 * pr, fma(keep, f.get(1 + 2 * pr), gp));
+      out.put(2 + 2 * pr, fma(keep, f.get(2 + 2 * pr), gm));
     }
   }
+  return low > 0;
 }
 
 // BGK collision of one site, f <- f - (f - f^eq(rho, u_bar, T_bar)) / tau with
 // u_bar = u + tau g, T_bar = T - tau^2 g^2 / D (Eq. MASTERSHIFT3, Eq. discrete).
 // The equilibrium is evaluated per pair as even +- odd parts with per-shell
 // coefficients (see ShellConsts), pre-scaled by omega rho w_shell.
-template <class O>
-__device__ __forceinline__ void collide_site_fp64(const double (&f)[kQ], const StepParams& p, double rho, double ux,
+template <class F, class P, class O>
+__device__ __forceinline__ void collide_site_fp64(const F& f, const P& p, double rho, double ux,
                                                   double uy, double T, const O& out) {
   const double ubx = ux;
   const double uby = uy + p.uy_shift;
@@ -499,7 +531,7 @@ __device__ __forceinline__ void collide_site_fp64(const double (&f)[kQ], const S
   const double keep = p.one_minus_omega;
   {
     const double C0 = A0 + th * (c_shell.alpha[0] + q * c_shell.beta[0] + th * c_shell.gamma[0]);
-    out.put(0, fma(keep, f[0], wr * c_shell.w[0] * C0));
+    out.put(0, fma(keep, f.get(0), wr * c_shell.w[0] * C0));
   }
 #pragma unroll
   for (int k = 1; k < kShells; ++k) {
@@ -516,29 +548,40 @@ __device__ __forceinline__ void collide_site_fp64(const double (&f)[kQ], const S
       const double b = a * a;
       const double even = P0 + b * (P2 + b * P4);
       const double odd = a * (P1 + b * P3);
-      out.put(1 + 2 * pr, fma(keep, f[1 + 2 * pr], even + odd));
-      out.put(2 + 2 * pr, fma(keep, f[2 + 2 * pr], even - odd));
+      out.put(1 + 2 * pr, fma(keep, f.get(1 + 2 * pr), even + odd));
+      out.put(2 + 2 * pr, fma(keep, f.get(2 + 2 * pr), even - odd));
     }
   }
 }
 
 // One site's collision: moments as exact integer sums, then the fixed-point
 // form inside its ranges, else the FP64 form; the relaxed populations to out.
-template <class O>
-__device__ __forceinline__ void collide_site_to(double (&f)[kQ], const StepParams& p, const O& out) {
+// The common path ends before the rest, which starts again from the
+// populations, so that it keeps nothing alive for it.
+template <class F, class P, class O>
+__device__ __forceinline__ void collide_site_to(const F& f, const P& p, const O& out) {
   long long r, jx, jy, e;
   int emax;
-  FxSite fs;
-  const bool sums = site_sums(f, r, jx, jy, e, emax);
-  if (sums && fx_site_from_sums(r, jx, jy, e, emax, p, fs)) {
-    collide_site_fx(f, p, fs, out);
-    return;
+  {
+    FxSite v;
+    if (site_sums<false>(f, r, jx, jy, e, emax) && fx_site_from_sums(r, jx, jy, e, emax, p, v) &&
+        collide_site_fx<false>(f, p, v, out))
+      return;
   }
   double rho, ux, uy, T;
-  if (sums)
+  if (site_sums<true>(f, r, jx, jy, e, emax)) {
+    FxSite v;
+    if (fx_site_from_sums(r, jx, jy, e, emax, p, v)) {
+      collide_site_fx<true>(f, p, v, out);
+      return;
+    }
     moments_from_sums(r, jx, jy, e, emax, rho, ux, uy, T);
-  else
-    site_moments_fp64(f, rho, ux, uy, T);
+  } else {
+    double g[kQ];
+#pragma unroll
+    for (int l = 0; l < kQ; ++l) g[l] = f.get(l);
+    site_moments_fp64(g, rho, ux, uy, T);
+  }
   collide_site_fp64(f, p, rho, ux, uy, T, out);
 }
 
@@ -656,43 +699,146 @@ __global__ void __launch_bounds__(128) bc_kernel(const double* __restrict__ src,
 template <bool OFF>
 __device__ __forceinline__ void store_images(double* __restrict__ dst, const StepParams& p, int x, int y) {
   if (x >= kHx && x < p.Lx - kHx && (!p.periodic_y || (y >= kHx && y < p.Ly - kHx))) return;
-  const double* s = dst + site_index(p, x, y);
-  double f[kQ];
+  const char* const s = (const char*)(dst + site_index(p, x, y));
 #pragma unroll
-  for (int l = 0; l < kQ; ++l)
-    f[l] = OFF ? *(const double*)((const char*)s + p.plane_off[l]) : s[l * p.plane];
-  int xs[3] = {x, 0, 0}, ys[3] = {y, 0, 0};
-  int nx = 1, ny = 1;
-  if (x < kHx) xs[nx++] = x + p.Lx;
-  if (x >= p.Lx - kHx) xs[nx++] = x - p.Lx;
-  if (p.periodic_y) {
-    if (y < kHx) ys[ny++] = y + p.Ly;
-    if (y >= p.Ly - kHx) ys[ny++] = y - p.Ly;
-  }
-  for (int a = 0; a < nx; ++a)
-    for (int b = 0; b < ny; ++b) {
-      if (a == 0 && b == 0) continue;  // the site's own element
-      double* d = dst + site_index(p, xs[a], ys[b]);
+  for (int part = 0; part < 2; ++part) {  // half of the populations at a time: 96 registers hold no more
+    constexpr int kHalf = (kQ + 1) / 2;
+    double f[kHalf];
 #pragma unroll
-      for (int l = 0; l < kQ; ++l) {
-        if (OFF)
-          *(double*)((char*)d + p.plane_off[l]) = f[l];
-        else
-          d[l * p.plane] = f[l];
-      }
+    for (int k = 0; k < kHalf; ++k) {
+      const int l = part * kHalf + k;
+      if (l < kQ) f[k] = *(const double*)(s + (OFF ? p.plane_off[l] : l * p.plane * 8));
     }
+#pragma unroll 1
+    for (int a = -1; a <= 1; ++a)
+#pragma unroll 1
+      for (int b = p.periodic_y ? -1 : 0; b <= (p.periodic_y ? 1 : 0); ++b) {
+        const int xi = x + a * p.Lx, yi = y + b * p.Ly;  // an image inside the halo
+        if ((a == 0 && b == 0) || xi < -kHx || xi >= p.Lx + kHx || yi < -kHx || yi >= p.Ly + kHx) continue;
+        char* const d = (char*)(dst + site_index(p, xi, yi));
+#pragma unroll
+        for (int k = 0; k < kHalf; ++k) {
+          const int l = part * kHalf + k;
+          if (l < kQ) *(double*)(d + (OFF ? p.plane_off[l] : l * p.plane * 8)) = f[k];
+        }
+      }
+  }
 }
 
-__global__ void __launch_bounds__(kBlockY, D2Q37_SITE_MIN_BLOCKS) collide_kernel(double* __restrict__ buf, StepParams p) {
+// ---- populations staged in shared memory by bulk copies --------------------
+//
+// The blocks of the site kernels (one column x kStageRows rows) fetch their 37
+// rows with one bulk copy each (cp.async.bulk, completion on an mbarrier)
+// instead of 37 loads a thread.  The loads then need no registers, no address
+// arithmetic and no issue slots of the threads, and the populations are read
+// from shared memory twice, for the moment sums and for the relaxation, so
+// that 24 warps per SM are resident with 80 registers (and a few spills)
+// instead of 16 with 128.  Measured on the 2048 x 8192 fused step: 2.70 ms with
+// the populations in registers, 2.42 ms this way (5 blocks of 128, 96
+// registers: 2.56; 2 of 256, 128 registers: 2.86; 2 of 384: 2.64; 3 of 192:
+// 2.61).  Persistent blocks that fetch the next tile into the slots the
+// relaxation has finished with wait less for memory but run more instructions,
+// and one warp per block lets the warps' code drift apart: both were slower.
+constexpr int kStageRows = 256;
+constexpr int kStageBlocks = 3;
+// A slot holds one population's rows from a 16-byte boundary of the frame: one
+// row early when its c_y is odd.
+constexpr int kSlot = (kStageRows + 2) * 8;
+constexpr int kStageBytes = kQ * kSlot + 16;  // and the barrier
+constexpr int kWaitLimit = 1 << 20;           // polls of the barrier, each of some microseconds at most
+
+__host__ __device__ constexpr int odd_hops() {
+  int n = 0;
+  for (int l = 0; l < kQ; ++l) n += vel_cy(l) & 1;
+  return n;
+}
+
+// One thread's row of the staged populations.  The reads are volatile, so
+// that the compiler does not keep the first reading in registers.
+template <bool PULL>
+struct RowPopsOf {
+  unsigned a;  // shared address of the row in slot 0; 0: the copies did not land
+  static __device__ __forceinline__ constexpr int at(int l) { return l * kSlot + (PULL ? vel_cy(l) & 1 : 0) * 8; }
+  __device__ __forceinline__ double get(int l) const {
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a + at(l)));
+    return v;
+  }
+};
+using RowPops = RowPopsOf<true>;
+
+__device__ __forceinline__ bool mbar_wait(unsigned bar) {
+  for (int i = 0; i < kWaitLimit; ++i) {
+    int ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.b32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+// 3-bit fields of c + 3 of the populations, 21 to a word.
+__host__ __device__ constexpr unsigned long long hop_fields(int (*c)(int), int first) {
+  unsigned long long w = 0;
+  for (int l = first; l < kQ && l < first + 21; ++l) w |= (unsigned long long)(c(l) + 3) << (3 * (l - first));
+  return w;
+}
+
+// Copy `rows` rows from `site` (16-byte aligned) of every population into the
+// block's slots, pulled (PULL) or in place, and wait for them.  g: the
+// lattice's plane and NY.  The hops come from packed fields and the copies are
+// spread over the warps: each is started by one lane after the other, and the
+// offsets read from the constant bank with an index per lane take as long.
+template <bool PULL, class G>
+__device__ __forceinline__ RowPopsOf<PULL> stage_rows(unsigned char* stage, const char* site, const G& g, int rows) {
+  const unsigned slots = (unsigned)__cvta_generic_to_shared(stage);
+  const unsigned bar = slots + kQ * kSlot;
+  constexpr int n_odd = PULL ? odd_hops() : 0;
+  const int even = (rows * 8 + 15) & ~15, odd = (rows * 8 + 23) & ~15;
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((kQ - n_odd) * even + n_odd * odd)
+                 : "memory");
+  }
+  __syncthreads();  // the barrier is ready
+  constexpr int per_warp = (kQ + kStageRows / 32 - 1) / (kStageRows / 32);
+  const int lane = threadIdx.x & 31, l = (threadIdx.x >> 5) * per_warp + lane;
+  if (lane < per_warp && l < kQ) {
+    const char* from = site + l * (g.plane * 8);
+    if (PULL) {
+      constexpr unsigned long long x0 = hop_fields(vel_cx, 0), x1 = hop_fields(vel_cx, 21);
+      constexpr unsigned long long y0 = hop_fields(vel_cy, 0), y1 = hop_fields(vel_cy, 21);
+      const int k = 3 * (l < 21 ? l : l - 21);
+      const int cx = (int)((l < 21 ? x0 : x1) >> k & 7) - 3, cy = (int)((l < 21 ? y0 : y1) >> k & 7) - 3;
+      from -= ((long long)cx * g.NY + cy) * 8;
+    }
+    const unsigned long long at = (unsigned long long)from;
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     slots + l * kSlot),
+                 "l"(at & ~15ull), "r"((at & 8) ? odd : even), "r"(bar)
+                 : "memory");
+  }
+  if (mbar_wait(bar)) return {slots + threadIdx.x * 8};
+  // never seen: tell the host (lbm_synchronize returns LBM_ETIMEOUT), give the
+  // copies in flight the same time again and leave the tile unwritten
+  if (threadIdx.x == 0) *(volatile unsigned*)c_shell.late = 1u;
+  mbar_wait(bar);
+  return {0u};
+}
+
+__global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(double* __restrict__ buf, StepParams p) {
+  extern __shared__ __align__(128) unsigned char stage[];
   const int x = blockIdx.x;
-  const int y = blockIdx.y * kBlockY + threadIdx.x;
-  if (y >= p.Ly) return;
-  double* const b = buf + site_index(p, x, y);
-  double f[kQ];
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) f[l] = *(const double*)((const char*)b + p.plane_off[l]);
-  // in place: every population is read above before its pair is written back
-  collide_site_to(f, p, ToPlanes{(char*)b, p});
+  const int y0 = blockIdx.y * kStageRows;
+  const int y = y0 + threadIdx.x;
+  const long long i0 = site_index(p, x, y0);
+  const RowPopsOf<false> f = stage_rows<false>(stage, (const char*)(buf + i0), p, min(kStageRows, p.Ly - y0));
+  if (f.a == 0 || y >= p.Ly) return;
+  collide_site_to(f, p, ToPlanes{(char*)(buf + i0) + threadIdx.x * 8u, p});
   store_images<true>(buf, p, x, y);
 }
 
@@ -721,23 +867,28 @@ __device__ __forceinline__ void fused_site(const double* __restrict__ src, doubl
   }
   // each pair straight to the site's planes, then the halo images, if any
   if constexpr (OFF)
-    collide_site_to(f, px, ToPlanes{(char*)(dst + i), p});
+    collide_site_to(RegPops{f}, px, ToPlanes{(char*)(dst + i), p});
   else
-    collide_site_to(f, px, ToPlanesStride{dst + i, p.plane});
+    collide_site_to(RegPops{f}, px, ToPlanesStride{dst + i, p.plane});
   store_images<OFF>(dst, p, x, y);
 }
 
-__global__ void __launch_bounds__(kBlockY, D2Q37_SITE_MIN_BLOCKS) fused_kernel(const double* __restrict__ src, double* __restrict__ dst,
-                                                        StepParams p) {
+__global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const double* __restrict__ src,
+                                                                        double* __restrict__ dst, StepParams p) {
+  extern __shared__ __align__(128) unsigned char stage[];
   const int x = blockIdx.x;
-  const int y = blockIdx.y * kBlockY + threadIdx.x;
+  const int y0 = blockIdx.y * kStageRows;
+  const int y = y0 + threadIdx.x;
   // the wall-band kernel, launched next with programmatic stream
   // serialization, reads and writes nothing this kernel writes: it may start
   // once every block of this one has started, and fill the tail
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (y >= p.Ly) return;
+  const long long i0 = site_index(p, x, y0);
+  const RowPops f = stage_rows<true>(stage, (const char*)(src + i0), p, min(kStageRows, p.Ly - y0));
+  if (f.a == 0 || y >= p.Ly) return;
   if (!p.periodic_y && (y < 3 || y >= p.Ly - 3)) return;  // wall_band_kernel's
-  fused_site<true, false>(src, dst, p, p, x, y);
+  collide_site_to(f, p, ToPlanes{(char*)(dst + i0) + threadIdx.x * 8u, p});
+  store_images<true>(dst, p, x, y);
 }
 
 // The fused step of the six wall-band rows of every column (y = 0..2 and
@@ -778,7 +929,7 @@ __global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* __r
 #pragma unroll
     for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(sp + p.pull_off[l]);
     apply_wall(f, p.fw[wall], wall, r, ((s0 + s1) + s2) * p.inv_denom[wall]);
-    collide_site_to(f, p, ToPlanes{(char*)(dst + i), p});
+    collide_site_to(RegPops{f}, p, ToPlanes{(char*)(dst + i), p});
     store_images<true>(dst, p, x, y);
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -895,7 +1046,7 @@ __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? 
     double* dst = (double*)g.buf[c ^ 1];
 #pragma unroll
     for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(s + off[l]);
-    collide_site_to(f, L.common, SharedPlanes{(char*)(dst + i), off + kQ});
+    collide_site_to(RegPops{f}, L.common, SharedPlanes{(char*)(dst + i), off + kQ});
     split_images(dst, g, x, i);
     return;
   }
@@ -923,7 +1074,7 @@ __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? 
   for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(s + g.pull_off[l]);
   apply_wall(f, tab[g.entry].p.fw[wall], wall, r, ((s0 + s1) + s2) * g.inv_denom[wall]);
   double* dst = (double*)g.buf[c ^ 1];
-  collide_site_to(f, L.common, GeoPlanes{(char*)(dst + i), g});
+  collide_site_to(RegPops{f}, L.common, GeoPlanes{(char*)(dst + i), g});
   split_images(dst, g, x, i);
 }
 
@@ -976,6 +1127,8 @@ __global__ void __launch_bounds__(kBlockY) init_equilibrium32_kernel(float* __re
 
 dim3 site_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kBlockY - 1) / kBlockY); }
 
+dim3 stage_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kStageRows - 1) / kStageRows); }
+
 // (column, wall) groups of the wall-band kernel: 2 Lx, ten per warp
 int wall_grid(const StepParams& p) {
   constexpr int per_block = kWallGroupsPerWarp * (kWallBlock / 32);
@@ -986,7 +1139,12 @@ int done(int n) { return cudaGetLastError() == cudaSuccess ? n : -1; }
 
 }  // namespace
 
-cudaError_t upload_shell_consts(const ShellConsts& c) { return cudaMemcpyToSymbol(c_shell, &c, sizeof(c)); }
+cudaError_t upload_shell_consts(const ShellConsts& c) {
+  cudaError_t e = cudaFuncSetAttribute(fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(collide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
+  return e == cudaSuccess ? cudaMemcpyToSymbol(c_shell, &c, sizeof(c)) : e;
+}
+
 
 int launch_wrap(double* buf, const StepParams& p, cudaStream_t stream) {
   const long long n = (long long)kQ * 6 * (p.periodic_y ? p.Ly + 2 * kHx : p.Ly) +
@@ -1008,12 +1166,12 @@ int launch_bc(const double* src, double* dst, const StepParams& p, cudaStream_t 
 }
 
 int launch_collide(double* buf, const StepParams& p, cudaStream_t stream) {
-  collide_kernel<<<site_grid(p), kBlockY, 0, stream>>>(buf, p);
+  collide_kernel<<<stage_grid(p), kStageRows, kStageBytes, stream>>>(buf, p);
   return done(1);
 }
 
 int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap) {
-  fused_kernel<<<site_grid(p), kBlockY, 0, stream>>>(src, dst, p);
+  fused_kernel<<<stage_grid(p), kStageRows, kStageBytes, stream>>>(src, dst, p);
   if (p.periodic_y) return done(1);
   if (!overlap) {
     wall_band_kernel<<<wall_grid(p), kWallBlock, 0, stream>>>(src, dst, p);

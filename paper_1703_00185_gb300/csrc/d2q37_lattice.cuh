@@ -97,6 +97,7 @@ struct ShellConsts {
   double s2;
   double w[kShells];
   double alpha[kShells], beta[kShells], gamma[kShells], delta[kShells], eps[kShells];
+  unsigned* late;  // mapped host memory: set by a kernel whose bulk copies did not land in time
 };
 
 // FP32 deviation storage: populations are stored as d_l = f_l - w_l in FP32,
@@ -140,7 +141,7 @@ struct StepParams {
   float wall_e32[2][2];   // (hi, lo): sum_M fwmw32 - sum_O w + sum_M w (M missing, O leaving pairs)
   float wall_inv32[2][2]; // (hi, lo): 1 / sum_M fw32
   // Fixed-point equilibrium constants of the FP64 step: per shell k,
-  // omega w_k = c_k 2^fx_e[k] with c_k in [0.5, 1); as unsigned integers, each
+  // omega w_k = c_k 2^E_k with c_k in [0.5, 1); as unsigned integers, each
   // at the scale that puts its product straight into the format it feeds:
   // c 2^60, 2^62, 2^64; c x2 2^59, 2^60; c x2^2 2^55; (c/6) 2^64, which is
   // also (c/24) 2^66 (x2 = s^2 |c_l|^2).
@@ -151,7 +152,7 @@ struct StepParams {
   // value enters with its sign bit flipped (x + 2^63), less a rounding
   // correction
   unsigned long long fx_d0[kShells], fx_d1[kShells], fx_d2[kShells];
-  int fx_e[kShells];
+  int fx_es[kShells];         // (E_k - 55) 2^20, the exponent of a result
   unsigned long long fx_s62;  // s 2^62
   unsigned long long fx_s63, fx_s2_63;  // s 2^63, s^2 2^63
   long long fx_uy_shift;      // tau g_y 2^64
