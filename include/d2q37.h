@@ -110,9 +110,9 @@ int lbm_create_ext(int Lx, int Ly, const lbm_params* p, void* dev_buf, size_t by
  * Results"): cold T_top fluid over hot T_bot fluid, interface
  * y_i(x) = Ly/2 + (Ly/64) sin(2 pi (x + 1/2) / Lx), T scaled by
  * 1 + 1e-3 (2U - 1), U = (splitmix64(seed + x Ly + y) >> 11) 2^-53;
- * rho = 1/T, u = 0, populations at equilibrium.  The temperature field is
- * built on the host (host-side scratch of 8 Lx Ly bytes) and uploaded; this
- * call synchronises the handle's stream. */
+ * rho = 1/T, u = 0, populations at equilibrium.  The interface is evaluated
+ * on the host (its C library's sine), the rest on the device; this call
+ * synchronises the handle's stream. */
 int lbm_init_rayleigh_taylor(lbm_t* h, uint64_t seed);
 
 /* Upload / download all physical populations, host [37][Lx][Ly] FP64 in this

@@ -298,11 +298,6 @@ int k_fields(lbm_t* h, const void* b, double* rho, double* u, double* T) {
                           : launch_fields((const double*)b, rho, u, T, h->sp, h->stream);
 }
 
-int k_init(lbm_t* h, void* b, const double* T) {
-  return is_fp32(h->prec) ? launch_init_equilibrium32((float*)b, T, h->sp, h->stream)
-                          : launch_init_equilibrium((double*)b, T, h->sp, h->stream);
-}
-
 int setup_handle(lbm_t* h, int Lx, int Ly, const lbm_params* p, void* mem, cudaStream_t stream) {
   h->Lx = Lx;
   h->Ly = Ly;
@@ -324,15 +319,6 @@ int setup_handle(lbm_t* h, int Lx, int Ly, const lbm_params* p, void* mem, cudaS
   int rc = check(cudaMemsetAsync(base, 0, 2 * bb, stream));
   if (rc == LBM_OK) rc = check(cudaStreamSynchronize(stream));
   return rc;
-}
-
-// SplitMix64 (Steele, Lea & Flood, OOPSLA 2014): the finaliser applied to
-// state v + 0x9e3779b97f4a7c15.
-uint64_t splitmix64(uint64_t v) {
-  uint64_t z = v + 0x9e3779b97f4a7c15ULL;
-  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
-  z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
-  return z ^ (z >> 31);
 }
 
 int step_once(lbm_t* h, int phases, bool fused) {
@@ -525,22 +511,21 @@ int lbm_init_rayleigh_taylor(lbm_t* h, uint64_t seed) {
   const TraceRange trace("lbm_init_rayleigh_taylor");
   if (!h) return LBM_EINVAL;
   const int Lx = h->Lx, Ly = h->Ly;
-  std::vector<double> T((size_t)Lx * Ly);
-  const double Tt = h->prm.T_top, Tb = h->prm.T_bot;
+  // the interface of every column here, with this machine's sine; the sites'
+  // temperatures on the device, where they are needed.  Only physical sites are
+  // written: the halo rows of a walled lattice are zero since the handle was
+  // set up, and pbc fills the other halos
+  std::vector<double> yi((size_t)Lx);
   for (int x = 0; x < Lx; ++x) {
     const double arg = (2.0 * M_PI * ((double)x + 0.5)) / (double)Lx;
-    const double yi = 0.5 * (double)Ly + ((double)Ly / 64.0) * std::sin(arg);
-    for (int y = 0; y < Ly; ++y) {
-      const double T0 = ((double)y + 0.5 < yi) ? Tb : Tt;
-      const uint64_t r = splitmix64(seed + (uint64_t)x * (uint64_t)Ly + (uint64_t)y);
-      const double U = (double)(r >> 11) * 0x1.0p-53;
-      T[(size_t)x * Ly + y] = T0 * (1.0 + 1e-3 * (2.0 * U - 1.0));
-    }
+    yi[x] = 0.5 * (double)Ly + ((double)Ly / 64.0) * std::sin(arg);
   }
-  int rc = check(cudaMemcpyAsync(h->scratch, T.data(), T.size() * sizeof(double), cudaMemcpyHostToDevice,
-                                 h->stream));
-  if (!rc) rc = check(cudaMemsetAsync(h->buf[h->cur], 0, buffer_bytes(Lx, Ly, h->prec), h->stream));
-  if (!rc) rc = run_kernel(h, LBM_KIND_INIT, [&] { return k_init(h, h->buf[h->cur], h->scratch); });
+  int rc = check(cudaMemcpyAsync(h->scratch, yi.data(), yi.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+  if (!rc)
+    rc = run_kernel(h, LBM_KIND_INIT, [&] {
+      return launch_init_rayleigh_taylor(h->buf[h->cur], is_fp32(h->prec), h->scratch, h->prm.T_top, h->prm.T_bot, seed,
+                                         h->sp, h->stream);
+    });
   if (!rc) rc = check(cudaStreamSynchronize(h->stream));
   if (!rc) {
     h->have_state = true;

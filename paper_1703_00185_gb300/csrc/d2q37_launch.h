@@ -20,9 +20,12 @@ int launch_collide(double* buf, const StepParams& p, cudaStream_t stream);
 // dependent of the sites kernel and starts in its tail; false: after it.
 int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap = true);
 int launch_fields(const double* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream);
-int launch_init_equilibrium(double* buf, const double* T, const StepParams& p, cudaStream_t stream);
+// Rayleigh-Taylor initial state, FP64 or FP32 deviations; yi: device, the
+// interface of every column.
+int launch_init_rayleigh_taylor(void* buf, bool fp32, const double* yi, double T_top, double T_bot,
+                                unsigned long long seed, const StepParams& p, cudaStream_t stream);
 
-// FP32 deviation storage (d2q37_kernels_fp32.cu; init in d2q37_kernels.cu).
+// FP32 deviation storage (d2q37_kernels_fp32.cu).
 // wide_fp64 selects FP64 (true) or double-float (false) for the wide terms.
 cudaError_t upload_shell_consts32(const ShellConsts32& c);
 int launch_wrap32(float* buf, const StepParams& p, cudaStream_t stream);
@@ -31,7 +34,6 @@ int launch_bc32(const float* src, float* dst, const StepParams& p, cudaStream_t 
 int launch_collide32(float* buf, const StepParams& p, bool wide_fp64, cudaStream_t stream);
 int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_fp64, cudaStream_t stream);
 int launch_fields32(const float* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream);
-int launch_init_equilibrium32(float* buf, const double* T, const StepParams& p, cudaStream_t stream);
 // Batched fused step over a table of n lattices (BatchEntry, device memory),
 // tiles of block_y rows; block_y in {64, 128, 256}; grid = number of blocks
 // of the grid-stride loop.  *_blocks_per_sm: resident blocks per SM.
