@@ -25,6 +25,7 @@ struct lbm_t {
   void* owned;      // cudaMalloc'ed block, NULL for lbm_create_ext
   cudaStream_t stream;
   bool owns_stream;
+  bool shares_device;  // other streams step other lattices at the same time (a job of a server)
   bool have_state;
   bool halo_valid;  // halo columns (and rows, if y is periodic) mirror the current state
   int64_t launches;

@@ -700,8 +700,16 @@ template <bool OFF>
 __device__ __forceinline__ void store_images(double* __restrict__ dst, const StepParams& p, int x, int y) {
   if (x >= kHx && x < p.Lx - kHx && (!p.periodic_y || (y >= kHx && y < p.Ly - kHx))) return;
   const char* const s = (const char*)(dst + site_index(p, x, y));
+  int xs[3] = {x, 0, 0}, ys[3] = {y, 0, 0};
+  int nx = 1, ny = 1;
+  if (x < kHx) xs[nx++] = x + p.Lx;
+  if (x >= p.Lx - kHx) xs[nx++] = x - p.Lx;
+  if (p.periodic_y) {
+    if (y < kHx) ys[ny++] = y + p.Ly;
+    if (y >= p.Ly - kHx) ys[ny++] = y - p.Ly;
+  }
 #pragma unroll
-  for (int part = 0; part < 2; ++part) {  // half of the populations at a time: 96 registers hold no more
+  for (int part = 0; part < 2; ++part) {  // half of the populations at a time: 80 registers hold no more
     constexpr int kHalf = (kQ + 1) / 2;
     double f[kHalf];
 #pragma unroll
@@ -710,18 +718,16 @@ __device__ __forceinline__ void store_images(double* __restrict__ dst, const Ste
       if (l < kQ) f[k] = *(const double*)(s + (OFF ? p.plane_off[l] : l * p.plane * 8));
     }
 #pragma unroll 1
-    for (int a = -1; a <= 1; ++a)
-#pragma unroll 1
-      for (int b = p.periodic_y ? -1 : 0; b <= (p.periodic_y ? 1 : 0); ++b) {
-        const int xi = x + a * p.Lx, yi = y + b * p.Ly;  // an image inside the halo
-        if ((a == 0 && b == 0) || xi < -kHx || xi >= p.Lx + kHx || yi < -kHx || yi >= p.Ly + kHx) continue;
-        char* const d = (char*)(dst + site_index(p, xi, yi));
+    for (int ab = 1; ab < nx * ny; ++ab) {  // 0: the site's own element
+      const int a = ab / ny, b = ab - a * ny;
+      char* const d = (char*)(dst + site_index(p, a == 0 ? xs[0] : a == 1 ? xs[1] : xs[2],
+                                               b == 0 ? ys[0] : b == 1 ? ys[1] : ys[2]));
 #pragma unroll
-        for (int k = 0; k < kHalf; ++k) {
-          const int l = part * kHalf + k;
-          if (l < kQ) *(double*)(d + (OFF ? p.plane_off[l] : l * p.plane * 8)) = f[k];
-        }
+      for (int k = 0; k < kHalf; ++k) {
+        const int l = part * kHalf + k;
+        if (l < kQ) *(double*)(d + (OFF ? p.plane_off[l] : l * p.plane * 8)) = f[k];
       }
+    }
   }
 }
 
@@ -787,8 +793,22 @@ __host__ __device__ constexpr unsigned long long hop_fields(int (*c)(int), int f
   return w;
 }
 
-// Copy `rows` rows from `site` (16-byte aligned) of every population into the
-// block's slots, pulled (PULL) or in place, and wait for them.  g: the
+// The block's barrier, for the copies of `rows` rows of every population.
+__device__ __forceinline__ void stage_init(unsigned char* stage, bool pull, int rows) {
+  const unsigned bar = (unsigned)__cvta_generic_to_shared(stage) + kQ * kSlot;
+  const int n_odd = pull ? odd_hops() : 0;
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                 "r"((kQ - n_odd) * ((rows * 8 + 15) & ~15) + n_odd * ((rows * 8 + 23) & ~15))
+                 : "memory");
+  }
+  __syncthreads();
+}
+
+// After stage_init: copy `rows` rows from `site` (16-byte aligned) of every
+// population into the block's slots, pulled (PULL) or in place, and wait for them.  g: the
 // lattice's plane and NY.  The hops come from packed fields and the copies are
 // spread over the warps: each is started by one lane after the other, and the
 // offsets read from the constant bank with an index per lane take as long.
@@ -796,15 +816,7 @@ template <bool PULL, class G>
 __device__ __forceinline__ RowPopsOf<PULL> stage_rows(unsigned char* stage, const char* site, const G& g, int rows) {
   const unsigned slots = (unsigned)__cvta_generic_to_shared(stage);
   const unsigned bar = slots + kQ * kSlot;
-  constexpr int n_odd = PULL ? odd_hops() : 0;
   const int even = (rows * 8 + 15) & ~15, odd = (rows * 8 + 23) & ~15;
-  if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((kQ - n_odd) * even + n_odd * odd)
-                 : "memory");
-  }
-  __syncthreads();  // the barrier is ready
   constexpr int per_warp = (kQ + kStageRows / 32 - 1) / (kStageRows / 32);
   const int lane = threadIdx.x & 31, l = (threadIdx.x >> 5) * per_warp + lane;
   if (lane < per_warp && l < kQ) {
@@ -836,6 +848,7 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(doubl
   const int y0 = blockIdx.y * kStageRows;
   const int y = y0 + threadIdx.x;
   const long long i0 = site_index(p, x, y0);
+  stage_init(stage, false, min(kStageRows, p.Ly - y0));
   const RowPopsOf<false> f = stage_rows<false>(stage, (const char*)(buf + i0), p, min(kStageRows, p.Ly - y0));
   if (f.a == 0 || y >= p.Ly) return;
   collide_site_to(f, p, ToPlanes{(char*)(buf + i0) + threadIdx.x * 8u, p});
@@ -879,9 +892,14 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const d
   const int x = blockIdx.x;
   const int y0 = blockIdx.y * kStageRows;
   const int y = y0 + threadIdx.x;
-  // the wall-band kernel, launched next with programmatic stream
-  // serialization, reads and writes nothing this kernel writes: it may start
-  // once every block of this one has started, and fill the tail
+  stage_init(stage, true, min(kStageRows, p.Ly - y0));
+  // launched with programmatic stream serialization this kernel starts in the
+  // tail of the one before it (the previous step's): wait for that grid to
+  // complete before the first access
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // the wall-band kernel, launched next the same way, reads and writes nothing
+  // this kernel writes, and the previous step is complete here: it may start
+  // once every block of this one has come this far, and fill the tail
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const long long i0 = site_index(p, x, y0);
   const RowPops f = stage_rows<true>(stage, (const char*)(src + i0), p, min(kStageRows, p.Ly - y0));
@@ -889,6 +907,28 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const d
   if (!p.periodic_y && (y < 3 || y >= p.Ly - 3)) return;  // wall_band_kernel's
   collide_site_to(f, p, ToPlanes{(char*)(dst + i0) + threadIdx.x * 8u, p});
   store_images<true>(dst, p, x, y);
+}
+
+// The same for a lattice so small that all its warps are resident with every
+// register of an SM shared by 8 of them: the populations straight into
+// registers.  What counts there is the length of one site's chain, not room for
+// other warps.  Microseconds a step, before (2 blocks of 256 rows, 128
+// registers, no chaining) / now, blocks of 128 rows: 256 x 128 16.0 / 13.9, 130 x
+// 257 15.3 / 14.8, 64 x 64 15.5 / 14.2; 64 or 32 rows 15.0, 15.4 on the first.
+// Without walls (periodic y, edge rows with halo images in every column)
+// blocks of 32 rows: 130 x 257 13.2 / 11.0, 128 rows 16.2.
+constexpr int kFewWarps = 8;  // resident per SM at up to 255 registers
+
+template <int ROWS>
+__global__ void __launch_bounds__(ROWS, kFewWarps * 32 / ROWS) fused_few_kernel(const double* __restrict__ src,
+                                                                                double* __restrict__ dst, StepParams p) {
+  const int x = blockIdx.x;
+  const int y = blockIdx.y * ROWS + threadIdx.x;
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // as fused_kernel
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (y >= p.Ly) return;
+  if (!p.periodic_y && (y < 3 || y >= p.Ly - 3)) return;  // wall_band_kernel's
+  fused_site<true, false>(src, dst, p, p, x, y);
 }
 
 // The fused step of the six wall-band rows of every column (y = 0..2 and
@@ -911,6 +951,8 @@ constexpr int kWallGroupsPerWarp = 10;
 
 __global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* __restrict__ src,
                                                               double* __restrict__ dst, StepParams p) {
+  // the next step's sites kernel may start in this one's tail (it waits for it)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31;
   const int g = (blockIdx.x * (kWallBlock / 32) + (threadIdx.x >> 5)) * kWallGroupsPerWarp + lane / 3;
   const int r = lane - 3 * (lane / 3);  // row from the wall
@@ -1183,23 +1225,53 @@ int launch_collide(double* buf, const StepParams& p, cudaStream_t stream) {
   return done(1);
 }
 
-int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap) {
-  fused_kernel<<<stage_grid(p), kStageRows, kStageBytes, stream>>>(src, dst, p);
-  if (p.periodic_y) return done(1);
-  if (!overlap) {
-    wall_band_kernel<<<wall_grid(p), kWallBlock, 0, stream>>>(src, dst, p);
-    return done(2);
-  }
+// SMs of the current device (looked up once; the library is for one kind of GPU).
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
+               ? v
+               : 152;
+  }();
+  return n;
+}
+
+// Launch as a programmatic dependent of the kernel before it in the stream.
+template <class... A>
+cudaError_t launch_dependent(void (*kernel)(A...), dim3 grid, int block, int smem, cudaStream_t stream, A... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(wall_grid(p));
-  cfg.blockDim = dim3(kWallBlock);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, wall_band_kernel, src, dst, p) != cudaSuccess) return -1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap, bool chain) {
+  // few sites, and no other stream's grids to share the SMs with (those gain
+  // from the warps that the staged form leaves room for)
+  const bool few = chain && (long long)p.Lx * ((p.Ly + 31) / 32) <= (long long)kFewWarps * sm_count();
+  void (*const sites)(const double*, double*, StepParams) =
+      !few ? fused_kernel : p.periodic_y ? fused_few_kernel<32> : fused_few_kernel<128>;
+  const int rows = !few ? kStageRows : p.periodic_y ? 32 : 128, smem = few ? 0 : kStageBytes;
+  const dim3 grid(p.Lx, (p.Ly + rows - 1) / rows);
+  if (chain) {
+    if (launch_dependent(sites, grid, rows, smem, stream, src, dst, p) != cudaSuccess) return -1;
+  } else {
+    sites<<<grid, rows, smem, stream>>>(src, dst, p);
+  }
+  if (p.periodic_y) return done(1);
+  if (!overlap) {
+    wall_band_kernel<<<wall_grid(p), kWallBlock, 0, stream>>>(src, dst, p);
+    return done(2);
+  }
+  if (launch_dependent(wall_band_kernel, dim3(wall_grid(p)), kWallBlock, 0, stream, src, dst, p) != cudaSuccess) return -1;
   return done(2);
 }
 

@@ -477,6 +477,10 @@ template <class W>
 __global__ void __launch_bounds__(kBlockY, D2Q37_FP32_MIN_BLOCKS) fused32_kernel(const float* __restrict__ src,
                                                                                  float* __restrict__ dst,
                                                                                  StepParams p) {
+  // launched with programmatic stream serialization (chain), this grid starts
+  // in the tail of the previous step's and waits here for it to complete
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int x = blockIdx.x;
   const int y = blockIdx.y * kBlockY + threadIdx.x;
   if (y >= p.Ly) return;
@@ -654,12 +658,18 @@ int launch_collide32(float* buf, const StepParams& p, bool wide_fp64, cudaStream
   return done(1);
 }
 
-int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_fp64, cudaStream_t stream) {
-  if (wide_fp64)
-    fused32_kernel<WideF64><<<site_grid(p), kBlockY, 0, stream>>>(src, dst, p);
-  else
-    fused32_kernel<WideDF><<<site_grid(p), kBlockY, 0, stream>>>(src, dst, p);
-  return done(1);
+int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_fp64, cudaStream_t stream, bool chain) {
+  void (*const kernel)(const float*, float*, StepParams) = wide_fp64 ? fused32_kernel<WideF64> : fused32_kernel<WideDF>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = site_grid(p);
+  cfg.blockDim = dim3(kBlockY);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, src, dst, p) == cudaSuccess ? done(1) : -1;
 }
 
 template <class W, int BY>

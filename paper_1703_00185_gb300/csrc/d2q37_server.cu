@@ -146,6 +146,7 @@ int admit(lbm_server_t* s) {
     j->stream = (int)(std::min_element(s->stream_sites, s->stream_sites + kStreams) - s->stream_sites);
     cudaStream_t st = s->stream[j->stream];
     int rc = lbm_create_ext(j->Lx, j->Ly, &j->prm, s->pool_mem + off, need, st, &j->h);
+    if (!rc) j->h->shares_device = true;
     if (!rc) rc = lbm_init_rayleigh_taylor(j->h, j->seed);
     if (!rc) rc = handle_prepare_halos(j->h, st);
     if (rc) {
