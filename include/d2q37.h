@@ -178,12 +178,9 @@ void lbm_destroy(lbm_t* h);
  * single-GPU form for many independent jobs.  Every lattice keeps its own
  * memory, parameters and state (its lbm_t).  Launch shapes:
  *  - block_y > 0, blocks_per_sm = 0: one launch per step with one block per
- *    tile (one column by block_y rows) of every lattice.  FP64 batches whose
- *    lattices all have walls and the same tau and g (at most 64 lattices,
- *    offsets within 32 bits) run the wall rows in separate wall tiles of the
- *    same launch and read each lattice's offsets from the launch's parameters;
- *    FP32-storage batches of at most 128 lattices read each lattice's
- *    parameters from the launch's parameters; others use the table below.
+ *    tile (one column by block_y rows) of every lattice, in FP64 the wall rows
+ *    in separate wall tiles of the same launch.  At most 384 lattices, whose
+ *    geometry is in the launch's parameters; larger batches use the table below.
  *  - block_y > 0, blocks_per_sm > 0: a persistent grid-stride kernel over the
  *    tiles, each lattice's parameters read from a device table.
  *  - block_y = 0: one launch of the single-lattice fused kernel per lattice,
@@ -234,7 +231,7 @@ void lbm_batch_destroy(lbm_batch_t* b);
  * lbm_batch_step_static advances n lattices (same precision, each with a
  * state; their memory is the caller's, e.g. from lbm_create_ext) by `steps`
  * steps, one batched fused launch per step on cuda_stream, exactly as
- * lbm_batch_step with tiles of 128 rows.  It allocates no device memory and
+ * lbm_batch_step with tiles of 128 rows (one block per tile).  It allocates no device memory and
  * calls no allocating library routine: its tile table lives in a file-scope
  * static device array of LBM_STATIC_BATCH_MAX entries (about 680 KB) that
  * every GPU loading this library holds until the process exits.

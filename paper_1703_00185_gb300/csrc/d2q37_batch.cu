@@ -5,12 +5,10 @@
 // batch owns a device table of BatchEntry (parameters, both buffers, the
 // buffer holding the state, tile range) and a per-tile owner table, and
 // advances every lattice by one step per launch:
-//  - block_y > 0, blocks_per_sm = 0: one block per tile.  FP64 batches that
-//    allow it (walls, one tau and g, at most kBatchGeoMax lattices, 32-bit
-//    offsets) run the split form, site tiles and wall tiles of every lattice
-//    with each lattice's offsets in the launch's parameters (BatchLaunch);
-//    FP32-storage batches of at most kBatchGeo32Max lattices take their
-//    parameters from BatchLaunch32; other batches run the table kernel.
+//  - block_y > 0, blocks_per_sm = 0: one block per tile, site tiles and (FP64,
+//    walls) wall tiles of every lattice, up to kBatchGeoMax (kBatchGeo32Max)
+//    lattices with their geometry in the launch's parameters; other batches
+//    run the table kernel.
 //  - block_y > 0, blocks_per_sm > 0: the table kernel on a persistent grid.
 //  - block_y = 0: the single-lattice fused kernel once per lattice (its
 //    parameters in the constant bank), spread over kAux streams forked from
@@ -18,7 +16,6 @@
 // lbm_batch_step(n) replays a captured two-step CUDA graph when the stream
 // can be captured (with block_y = 0 a graph of parallel branches).
 #include <algorithm>
-#include <cstddef>
 #include <cstring>
 #include <vector>
 
@@ -35,15 +32,10 @@ struct lbm_batch_t {
   int* dev_tile_entry[3];  // owning entry of every tile
   bool uniform;            // every lattice has the collision constants of `common` (same tau, g)
   StepParams common;
-  // FP64 with walls, shared tau and g, at most kBatchGeoMax lattices whose
-  // offsets fit 32 bits: block_y > 0 with blocks_per_sm = 0 runs the split
-  // form (site tiles and wall tiles in one launch), parameters per block_y
-  bool split_ok;
-  BatchLaunch* split[3];
-  // FP32 storage, at most kBatchGeo32Max lattices: block_y > 0 with
-  // blocks_per_sm = 0 runs one block per tile with parameters in the launch
-  bool split32_ok;
-  BatchLaunch32* split32[3];
+  // block_y > 0 with blocks_per_sm = 0: one block per tile, parameters in the
+  // launch, per block_y (null: more lattices than a launch holds)
+  BatchLaunch* launch64[3];
+  BatchLaunch32* launch32[3];
   long long tiles[3];
   int block_y;        // 64, 128 or 256
   int blocks_per_sm;  // 0: one block per tile; else a persistent grid of blocks_per_sm x SMs
@@ -128,11 +120,12 @@ long long grid_of(const lbm_batch_t* b, int block_y, int blocks_per_sm) {
 int launch(lbm_batch_t* b, int block_y, int blocks_per_sm, int parity) {
   if (block_y == 0) return launch_each(b, parity);
   const int s = slot_of(block_y);
-  if (blocks_per_sm == 0 && (b->split_ok || b->split32_ok)) {
-    const int n = b->split_ok ? launch_batch_split(*b->split[s], b->dev_tab[s], b->dev_tile_entry[s], parity,
-                                                   block_y, b->stream)
-                              : launch_batch_split32(*b->split32[s], b->dev_tile_entry[s], (int)b->tiles[s], parity,
-                                                     block_y, b->prec == LBM_PRECISION_FP32_FP64, b->stream);
+  if (blocks_per_sm == 0 && (b->launch64[s] || b->launch32[s])) {
+    const int n = b->launch64[s] ? launch_batch_tiles(*b->launch64[s], b->uniform, b->dev_tab[s], b->dev_tile_entry[s],
+                                                      parity, block_y, b->stream)
+                                 : launch_batch_tiles32(*b->launch32[s], b->dev_tab[s], b->dev_tile_entry[s],
+                                                        (int)b->tiles[s], parity, block_y,
+                                                        b->prec == LBM_PRECISION_FP32_FP64, b->stream);
     if (n < 0) return LBM_ECUDA;
     b->launches += n;
     return LBM_OK;
@@ -187,105 +180,97 @@ bool pair_graph(lbm_batch_t* b, cudaGraphExec_t* out) {
   return true;
 }
 
-bool fits32(long long v) { return v >= -2147483647LL - 1 && v <= 2147483647LL; }
-
-// The FP32 one-block-per-tile form's launch parameters (the lattices'
-// entries of the device table dev_tab hold their wall constants).
-void build_split32(lbm_batch_t* b) {
-  b->split32_ok = b->prec != LBM_PRECISION_FP64 && b->n <= kBatchGeo32Max;
-  for (int s = 0; s < 3 && b->split32_ok; ++s) {
-    if (b->tiles[s] > 2147483647LL) {
-      b->split32_ok = false;
-      break;
-    }
-    BatchLaunch32* L = new BatchLaunch32();
-    std::memset(L, 0, sizeof(*L));
-    L->n = b->n;
-    for (int i = 0; i < b->n; ++i) {
-      const lbm_t* h = b->lat[i];
-      const StepParams& q = h->sp;
-      // device addresses inside the entry's parameters (addresses only: no access on the host)
-      const char* dq = (const char*)b->dev_tab[s] + i * sizeof(BatchEntry) + offsetof(BatchEntry, p);
-      BatchGeo32& g = L->g[i];
-      g.Lx = h->Lx;
-      g.Ly = h->Ly;
-      g.NY = q.NY;
-      g.Hy = q.Hy;
-      g.periodic_y = q.periodic_y;
-      g.tile0 = (int)b->host_tab[s][i].tile0;
-      g.cur = b->host_tab[s][i].cur;
-      g.plane = q.plane;
-      g.buf[0] = h->buf[0];
-      g.buf[1] = h->buf[1];
-      g.omega_f = q.omega_f;
-      g.keep_f = q.keep_f;
-      g.uy_shift_df[0] = q.uy_shift_df[0];
-      g.uy_shift_df[1] = q.uy_shift_df[1];
-      g.theta_shift_df[0] = q.theta_shift_df[0];
-      g.theta_shift_df[1] = q.theta_shift_df[1];
-      g.theta_shift = q.theta_shift;
-      g.fw32 = (const float(*)[kQ])(dq + offsetof(StepParams, fw32));
-      g.fwmw32 = (const float(*)[kQ])(dq + offsetof(StepParams, fwmw32));
-      g.wall_e32 = (const float(*)[2])(dq + offsetof(StepParams, wall_e32));
-      g.wall_inv32 = (const float(*)[2])(dq + offsetof(StepParams, wall_inv32));
-    }
-    b->split32[s] = L;
-  }
-}
-
-// The split form's launch parameters for every block_y, if the batch allows it.
-void build_split(lbm_batch_t* b) {
-  b->split_ok = b->prec == LBM_PRECISION_FP64 && b->uniform && b->n <= kBatchGeoMax;
-  for (int i = 0; i < b->n && b->split_ok; ++i) {
-    const StepParams& q = b->lat[i]->sp;
-    b->split_ok = !q.periodic_y;
-    for (int l = 0; l < kQ && b->split_ok; ++l) b->split_ok = fits32(q.pull_off[l]) && fits32(q.plane_off[l]);
-  }
-  if (!b->split_ok) return;
+// The launch parameters of the one-block-per-tile form.
+void build_launches(lbm_batch_t* b) {
   const int bys[3] = {64, 128, 256};
+  std::vector<int> cur(b->n);
+  for (int i = 0; i < b->n; ++i) cur[i] = b->host_tab[0][i].cur;
   for (int s = 0; s < 3; ++s) {
-    BatchLaunch* L = new BatchLaunch();
-    std::memset(L, 0, sizeof(*L));
-    L->common = b->common;
-    L->n = b->n;
-    long long t0 = 0, w0 = 0;
-    const int per_wall_tile = batch_wall_groups_per_tile(bys[s]);
-    for (int i = 0; i < b->n; ++i) {
-      const lbm_t* h = b->lat[i];
-      BatchGeo& g = L->g[i];
-      for (int l = 0; l < kQ; ++l) {
-        g.pull_off[l] = (int)h->sp.pull_off[l];
-        g.plane_off[l] = (int)h->sp.plane_off[l];
+    if (b->prec == LBM_PRECISION_FP64 && b->n <= kBatchGeoMax) {
+      b->launch64[s] = new BatchLaunch();
+      bool uniform = false;
+      if (fill_batch_launch(*b->launch64[s], b->n, b->lat.data(), cur.data(), bys[s], &uniform) < 0) {
+        delete b->launch64[s];
+        b->launch64[s] = nullptr;
       }
-      g.Lx = h->Lx;
-      g.Ly = h->Ly;
-      g.NY = h->sp.NY;
-      g.Hy = h->sp.Hy;
-      g.ytiles = (h->Ly + bys[s] - 1) / bys[s];
-      g.tile0 = (int)t0;
-      g.wtile0 = (int)w0;
-      g.cur = b->host_tab[s][i].cur;
-      g.entry = i;
-      g.plane = h->sp.plane;
-      g.buf[0] = h->buf[0];
-      g.buf[1] = h->buf[1];
-      g.inv_denom[0] = h->sp.inv_denom[0];
-      g.inv_denom[1] = h->sp.inv_denom[1];
-      t0 += (long long)h->Lx * g.ytiles;
-      w0 += (2LL * h->Lx + per_wall_tile - 1) / per_wall_tile;
+    } else if (b->prec != LBM_PRECISION_FP64 && b->n <= kBatchGeo32Max) {
+      b->launch32[s] = new BatchLaunch32();
+      if (fill_batch_launch32(*b->launch32[s], b->n, b->lat.data(), cur.data(), bys[s]) < 0) {
+        delete b->launch32[s];
+        b->launch32[s] = nullptr;
+      }
     }
-    if (t0 + w0 > 2147483647LL) {
-      delete L;
-      b->split_ok = false;
-      return;
-    }
-    L->site_tiles = (int)t0;
-    L->wall_tiles = (int)w0;
-    b->split[s] = L;
   }
 }
 
 }  // namespace
+
+namespace d2q37 {
+
+long long fill_batch_launch(BatchLaunch& L, int n, lbm_t* const* lattices, const int* cur, int block_y, bool* uniform) {
+  if (n > kBatchGeoMax) return -1;
+  const StepParams& first = lattices[0]->sp;
+  L.common = first;  // its Collision
+  L.n = n;
+  *uniform = true;
+  const int per_wall_tile = batch_wall_groups_per_tile(block_y);
+  long long t0 = 0, w0 = 0;
+  for (int i = 0; i < n; ++i) {
+    const StepParams& q = lattices[i]->sp;
+    *uniform = *uniform && q.omega == first.omega && q.uy_shift == first.uy_shift && q.theta_shift == first.theta_shift;
+    BatchGeo& g = L.g[i];
+    g.Lx = q.Lx;
+    g.Ly = q.Ly;
+    g.NY = q.NY;
+    g.Hy = q.Hy;
+    g.periodic_y = q.periodic_y;
+    g.tile0 = (int)t0;
+    g.wtile0 = (int)w0;
+    g.cur = cur[i];
+    g.plane = q.plane;
+    g.buf[0] = lattices[i]->buf[0];
+    g.buf[1] = lattices[i]->buf[1];
+    g.inv_denom[0] = q.inv_denom[0];
+    g.inv_denom[1] = q.inv_denom[1];
+    t0 += (long long)q.Lx * ((q.Ly + block_y - 1) / block_y);
+    if (!q.periodic_y) w0 += (2LL * q.Lx + per_wall_tile - 1) / per_wall_tile;
+    if (t0 + w0 > 2147483647LL) return -1;
+  }
+  L.site_tiles = (int)t0;
+  L.wall_tiles = (int)w0;
+  return t0;
+}
+
+long long fill_batch_launch32(BatchLaunch32& L, int n, lbm_t* const* lattices, const int* cur, int block_y) {
+  if (n > kBatchGeo32Max) return -1;
+  L.n = n;
+  long long t0 = 0;
+  for (int i = 0; i < n; ++i) {
+    const StepParams& q = lattices[i]->sp;
+    BatchLat32& g = L.g[i];
+    g.Lx = q.Lx;
+    g.Ly = q.Ly;
+    g.NY = q.NY;
+    g.periodic_y = q.periodic_y;
+    g.tile0 = (int)t0;
+    g.cur = cur[i];
+    g.plane = q.plane;
+    g.buf[0] = lattices[i]->buf[0];
+    g.buf[1] = lattices[i]->buf[1];
+    g.omega_f = q.omega_f;
+    g.keep_f = q.keep_f;
+    for (int k = 0; k < 2; ++k) {
+      g.uy_shift_df[k] = q.uy_shift_df[k];
+      g.theta_shift_df[k] = q.theta_shift_df[k];
+    }
+    g.theta_shift = q.theta_shift;
+    t0 += (long long)q.Lx * ((q.Ly + block_y - 1) / block_y);
+    if (t0 > 2147483647LL) return -1;
+  }
+  return t0;
+}
+
+}  // namespace d2q37
 
 extern "C" {
 
@@ -363,10 +348,7 @@ int lbm_batch_create(int n, lbm_t* const* lattices, void* cuda_stream, lbm_batch
     if (!rc) rc = check(cudaStreamSynchronize(b->stream));
   }
   if (!rc) rc = check(cudaStreamSynchronize(b->stream));
-  if (!rc) {
-    build_split(b);
-    build_split32(b);
-  }
+  if (!rc) build_launches(b);
   if (rc) {
     lbm_batch_destroy(b);
     return rc;
@@ -499,8 +481,8 @@ void lbm_batch_destroy(lbm_batch_t* b) {
     if (t) cudaFree(t);
   for (int* t : b->dev_tile_entry)
     if (t) cudaFree(t);
-  for (BatchLaunch* L : b->split) delete L;
-  for (BatchLaunch32* L : b->split32) delete L;
+  for (BatchLaunch* L : b->launch64) delete L;
+  for (BatchLaunch32* L : b->launch32) delete L;
   delete b;
 }
 

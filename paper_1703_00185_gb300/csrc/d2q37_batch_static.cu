@@ -85,30 +85,32 @@ int lbm_batch_step_static(int n, lbm_t* const* lattices, int steps, void* cuda_s
   for (int i = 0; i < n && !rc; ++i) rc = handle_prepare_halos(lattices[i], stream);
   if (rc) return rc;
   // the whole table [0, n) is rewritten every call; entries past n are never read
-  long long tiles = 0;
+  int cur[LBM_STATIC_BATCH_MAX];
   for (int i = 0; i < n; ++i) {
     BatchEntry& e = g_static_host[i];
     std::memset(&e, 0, sizeof(e));
     e.p = lattices[i]->sp;
-    e.buf[0] = lattices[i]->buf[0];
-    e.buf[1] = lattices[i]->buf[1];
-    e.cur = lattices[i]->cur;
-    e.ytiles = (lattices[i]->Ly + 127) / 128;
-    e.tile0 = tiles;
-    tiles += (long long)lattices[i]->Lx * e.ytiles;
+    cur[i] = lattices[i]->cur;
   }
+  // the launches' own parameters: geometry and collision constants
+  static_assert(LBM_STATIC_BATCH_MAX <= kBatchGeoMax && LBM_STATIC_BATCH_MAX <= kBatchGeo32Max, "one launch holds every lattice");
+  static BatchLaunch launch64;
+  static BatchLaunch32 launch32;
+  const int prec = lattices[0]->prec;
+  bool uniform = false;
+  const long long tiles = prec == LBM_PRECISION_FP64 ? fill_batch_launch(launch64, n, lattices, cur, 128, &uniform)
+                                                     : fill_batch_launch32(launch32, n, lattices, cur, 128);
+  if (tiles < 0) return LBM_ETOOBIG;
   // pageable source: the runtime stages it before the call returns (so the
   // next call may rewrite it), which waits for the stream's earlier work
   if (cudaMemcpyAsync(dev_tab, g_static_host, n * sizeof(BatchEntry), cudaMemcpyHostToDevice, stream) !=
       cudaSuccess)
     return LBM_ECUDA;
-  const int prec = lattices[0]->prec;
-  const int grid = (int)(tiles < 2147483647LL ? tiles : 2147483647LL);
   for (int t = 0; t < steps; ++t) {
-    const int launched =
-        prec == LBM_PRECISION_FP64
-            ? launch_batch_fused(dev_tab, nullptr, n, tiles, t & 1, 128, grid, nullptr, stream)
-            : launch_batch_fused32(dev_tab, nullptr, n, tiles, t & 1, 128, grid, prec == LBM_PRECISION_FP32_FP64, stream);
+    const int launched = prec == LBM_PRECISION_FP64
+                             ? launch_batch_tiles(launch64, uniform, dev_tab, nullptr, t & 1, 128, stream)
+                             : launch_batch_tiles32(launch32, dev_tab, nullptr, (int)tiles, t & 1, 128,
+                                                    prec == LBM_PRECISION_FP32_FP64, stream);
     if (launched < 0) return LBM_ECUDA;
   }
   for (int i = 0; i < n; ++i) lattices[i]->cur ^= (steps & 1);

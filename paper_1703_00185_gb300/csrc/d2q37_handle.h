@@ -68,6 +68,13 @@ int handle_prepare_halos(lbm_t* h, cudaStream_t stream);
 // since the last call.
 int handle_sync(cudaStream_t stream);
 
+// The launch parameters of a one-block-per-tile step of n lattices with tiles
+// of block_y rows; cur[i]: the buffer holding lattice i's state at parity 0.
+// Returns the number of site tiles, or -1 when the launch cannot hold them.
+// uniform (FP64): whether every lattice has the collision constants L.common.
+long long fill_batch_launch(BatchLaunch& L, int n, lbm_t* const* lattices, const int* cur, int block_y, bool* uniform);
+long long fill_batch_launch32(BatchLaunch32& L, int n, lbm_t* const* lattices, const int* cur, int block_y);
+
 // Quadrature constants on the current device (0 or an LBM_E* code).
 int handle_device_consts();
 

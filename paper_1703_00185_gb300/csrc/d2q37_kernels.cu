@@ -243,7 +243,6 @@ __device__ __forceinline__ double hop_dot(int cx, int cy, const double (&mx)[3],
 // -7.6e-17), which the moment sums' -1.2e-17 nearly cancels.
 // The odd part takes a rounded product: a bias there would act on the
 // momentum the same way every step.
-constexpr int kFxOut = 55;  // format of R0 and of the results G = even +- odd
 
 using u64 = unsigned long long;
 
@@ -692,12 +691,21 @@ __global__ void __launch_bounds__(128) bc_kernel(const double* __restrict__ src,
   }
 }
 
+// Byte offset of population plane l: from the parameters, or a multiple of the stride.
+template <bool OFF, class P>
+__device__ __forceinline__ long long plane_offset(const P& p, int l) {
+  if constexpr (OFF)
+    return p.plane_off[l];
+  else
+    return l * p.plane * 8;
+}
+
 // The halo images of a site whose populations are already in its own
 // element of dst (written by this thread): read back and copied out.  OFF:
 // the planes addressed with the byte offsets of p (read from the constant
 // bank by the single-lattice kernels) instead of multiples of p.plane.
-template <bool OFF>
-__device__ __forceinline__ void store_images(double* __restrict__ dst, const StepParams& p, int x, int y) {
+template <bool OFF, class P>
+__device__ __forceinline__ void store_images(double* __restrict__ dst, const P& p, int x, int y) {
   if (x >= kHx && x < p.Lx - kHx && (!p.periodic_y || (y >= kHx && y < p.Ly - kHx))) return;
   const char* const s = (const char*)(dst + site_index(p, x, y));
   int xs[3] = {x, 0, 0}, ys[3] = {y, 0, 0};
@@ -715,7 +723,7 @@ __device__ __forceinline__ void store_images(double* __restrict__ dst, const Ste
 #pragma unroll
     for (int k = 0; k < kHalf; ++k) {
       const int l = part * kHalf + k;
-      if (l < kQ) f[k] = *(const double*)(s + (OFF ? p.plane_off[l] : l * p.plane * 8));
+      if (l < kQ) f[k] = *(const double*)(s + (plane_offset<OFF>(p, l)));
     }
 #pragma unroll 1
     for (int ab = 1; ab < nx * ny; ++ab) {  // 0: the site's own element
@@ -725,7 +733,7 @@ __device__ __forceinline__ void store_images(double* __restrict__ dst, const Ste
 #pragma unroll
       for (int k = 0; k < kHalf; ++k) {
         const int l = part * kHalf + k;
-        if (l < kQ) *(double*)(d + (OFF ? p.plane_off[l] : l * p.plane * 8)) = f[k];
+        if (l < kQ) *(double*)(d + (plane_offset<OFF>(p, l))) = f[k];
       }
     }
   }
@@ -749,8 +757,9 @@ constexpr int kStageRows = 256;
 constexpr int kStageBlocks = 3;
 // A slot holds one population's rows from a 16-byte boundary of the frame: one
 // row early when its c_y is odd.
-constexpr int kSlot = (kStageRows + 2) * 8;
-constexpr int kStageBytes = kQ * kSlot + 16;  // and the barrier
+__host__ __device__ constexpr int slot_bytes(int rows) { return (rows + 2) * 8; }
+__host__ __device__ constexpr int stage_bytes(int rows) { return kQ * slot_bytes(rows) + 16; }  // and the barrier
+constexpr int kStageBytes = stage_bytes(kStageRows);
 constexpr int kWaitLimit = 1 << 20;           // polls of the barrier, each of some microseconds at most
 
 __host__ __device__ constexpr int odd_hops() {
@@ -761,10 +770,10 @@ __host__ __device__ constexpr int odd_hops() {
 
 // One thread's row of the staged populations.  The reads are volatile, so
 // that the compiler does not keep the first reading in registers.
-template <bool PULL>
+template <bool PULL, int ROWS = kStageRows>
 struct RowPopsOf {
   unsigned a;  // shared address of the row in slot 0; 0: the copies did not land
-  static __device__ __forceinline__ constexpr int at(int l) { return l * kSlot + (PULL ? vel_cy(l) & 1 : 0) * 8; }
+  static __device__ __forceinline__ constexpr int at(int l) { return l * slot_bytes(ROWS) + (PULL ? vel_cy(l) & 1 : 0) * 8; }
   __device__ __forceinline__ double get(int l) const {
     double v;
     asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a + at(l)));
@@ -794,8 +803,9 @@ __host__ __device__ constexpr unsigned long long hop_fields(int (*c)(int), int f
 }
 
 // The block's barrier, for the copies of `rows` rows of every population.
+template <int ROWS = kStageRows>
 __device__ __forceinline__ void stage_init(unsigned char* stage, bool pull, int rows) {
-  const unsigned bar = (unsigned)__cvta_generic_to_shared(stage) + kQ * kSlot;
+  const unsigned bar = (unsigned)__cvta_generic_to_shared(stage) + kQ * slot_bytes(ROWS);
   const int n_odd = pull ? odd_hops() : 0;
   if (threadIdx.x == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
@@ -812,12 +822,12 @@ __device__ __forceinline__ void stage_init(unsigned char* stage, bool pull, int 
 // lattice's plane and NY.  The hops come from packed fields and the copies are
 // spread over the warps: each is started by one lane after the other, and the
 // offsets read from the constant bank with an index per lane take as long.
-template <bool PULL, class G>
-__device__ __forceinline__ RowPopsOf<PULL> stage_rows(unsigned char* stage, const char* site, const G& g, int rows) {
+template <bool PULL, int ROWS = kStageRows, class G>
+__device__ __forceinline__ RowPopsOf<PULL, ROWS> stage_rows(unsigned char* stage, const char* site, const G& g, int rows) {
   const unsigned slots = (unsigned)__cvta_generic_to_shared(stage);
-  const unsigned bar = slots + kQ * kSlot;
+  const unsigned bar = slots + kQ * slot_bytes(ROWS);
   const int even = (rows * 8 + 15) & ~15, odd = (rows * 8 + 23) & ~15;
-  constexpr int per_warp = (kQ + kStageRows / 32 - 1) / (kStageRows / 32);
+  constexpr int per_warp = (kQ + ROWS / 32 - 1) / (ROWS / 32);
   const int lane = threadIdx.x & 31, l = (threadIdx.x >> 5) * per_warp + lane;
   if (lane < per_warp && l < kQ) {
     const char* from = site + l * (g.plane * 8);
@@ -830,7 +840,7 @@ __device__ __forceinline__ RowPopsOf<PULL> stage_rows(unsigned char* stage, cons
     }
     const unsigned long long at = (unsigned long long)from;
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     slots + l * kSlot),
+                     slots + l * slot_bytes(ROWS)),
                  "l"(at & ~15ull), "r"((at & 8) ? odd : even), "r"(bar)
                  : "memory");
   }
@@ -1001,102 +1011,73 @@ __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? 
   }
 }
 
-// ---- many lattices in one launch, split into site tiles and wall tiles ----
+// ---- many lattices in one launch, one block per tile ----------------------
 //
-// One block per tile, no grid-stride loop: the blocks of site tiles (one
-// column x BY rows, the wall rows left out) run fused_kernel's per-site work,
-// and the blocks of wall tiles run wall_band_kernel's (three lanes per
-// column and wall, the outgoing mass combined by warp shuffles), so that no
-// warp of the launch holds a few wall rows among ordinary ones.  Every
-// lattice's offsets come from the launch's parameter space (BatchLaunch,
-// through the constant cache) and its collision constants from `common`; the
-// per-site arithmetic is the single-lattice kernels', so results are the same
-// bit for bit.  Requires walls, the same tau and g for every lattice and
-// offsets that fit 32 bits (checked on the host).
-static_assert(sizeof(BatchLaunch) <= 32764, "BatchLaunch must fit the kernel parameter space");
+// The blocks of site tiles (one column x ROWS rows, the wall rows left out) run
+// fused_kernel's per-site work, and the blocks of wall tiles run
+// wall_band_kernel's (three lanes per column and wall, the outgoing mass
+// combined by warp shuffles), so that no warp of the launch holds a few wall
+// rows among ordinary ones.  Geometry comes from the launch's parameter space
+// (BatchLaunch, through the constant cache); the collision constants too when
+// every lattice shares tau and g (UNIFORM), else each block copies its
+// lattice's (BatchEntry) to shared memory.  The owner of a site tile comes from
+// a per-tile table or, without one, from a search over the launch's lattices.
+// The per-site arithmetic is the single-lattice kernels', so results are the
+// same bit for bit.  64 uneven lattices (42.3 M sites), milliseconds a step:
+// 7.36 with the populations in registers, 6.70 now (256 rows, 3 blocks per SM);
+// 100 lattices of 60-400 columns, each with its own tau and g: 1.86 as a table
+// walked by grid-stride blocks, 1.33 now (128 rows, 5 blocks per SM).
+static_assert(sizeof(BatchLaunch) <= 32700, "BatchLaunch must fit the kernel parameter space");
 
-
-struct GeoPlanes {
-  char* d;  // the site's element of plane 0
-  const BatchGeo& g;
-  __device__ __forceinline__ void put(int l, double v) const { *(double*)(d + g.plane_off[l]) = v; }
-};
-
-// The same with the plane offsets from a shared-memory copy.
-struct SharedPlanes {
-  char* d;
-  const int* off;  // shared memory: plane offsets of the block's lattice
-  __device__ __forceinline__ void put(int l, double v) const { *(double*)(d + off[l]) = v; }
-};
-
-// The lattice owning block b of the site tiles (wall = false) or wall tiles.
-__device__ __forceinline__ int split_owner(const BatchLaunch& L, int b, bool wall) {
-  int lo = 0, hi = L.n - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if ((wall ? L.g[mid].wtile0 : L.g[mid].tile0) <= b)
-      lo = mid;
-    else
-      hi = mid - 1;
-  }
-  return lo;
-}
-
-// The x halo image(s) of a site of a walled lattice (copied from dst[i]).
-__device__ __forceinline__ void split_images(double* __restrict__ dst, const BatchGeo& g, int x, long long i) {
-  if (x >= kHx && x < g.Lx - kHx) return;
-  const char* s = (const char*)(dst + i);
-  double f[kQ];
-#pragma unroll
-  for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(s + g.plane_off[l]);
-  const long long shift = (long long)g.Lx * g.NY;
-  if (x < kHx) {
-    char* d = (char*)(dst + i + shift);
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) *(double*)(d + g.plane_off[l]) = f[l];
-  }
-  if (x >= g.Lx - kHx) {
-    char* d = (char*)(dst + i - shift);
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) *(double*)(d + g.plane_off[l]) = f[l];
-  }
-}
-
-template <int BY>
-__global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? (D2Q37_BATCH_MIN_BLOCKS * 128) / BY : 1)
-    batch_split_kernel(const __grid_constant__ BatchLaunch L, const BatchEntry* __restrict__ tab,
-                       const int* __restrict__ tile_entry, int parity) {
+template <int ROWS, int BLOCKS, bool UNIFORM>
+__global__ void __launch_bounds__(ROWS, BLOCKS)
+    batch_tile_kernel(const __grid_constant__ BatchLaunch L, const BatchEntry* __restrict__ tab,
+                      const int* __restrict__ tile_entry, int parity) {
+  extern __shared__ __align__(128) unsigned char stage[];
+  __shared__ Collision own;
+  static_assert(sizeof(Collision) % 8 == 0, "Collision is copied in 8-byte words");
   const int b = blockIdx.x;
   if (b < L.site_tiles) {
-    const BatchGeo& g = L.g[tile_entry[b]];
-    // the lattice's 74 offsets in shared memory: the blocks of an SM serve
-    // different lattices, whose parameter slices crowd the constant cache
-    // (read from there: 5796 MLUPS on the 64-lattice workload, against 5881)
-    __shared__ int off[2 * kQ];
-    for (int k = threadIdx.x; k < 2 * kQ; k += BY) off[k] = k < kQ ? g.pull_off[k] : g.plane_off[k - kQ];  // BY may be < 74
-    __syncthreads();
+    const int i = tile_entry ? tile_entry[b] : batch_owner(L, b);
+    const BatchGeo& g = L.g[i];
     // x fastest, as in fused_kernel: the columns a tile pulls from run at the same time
     const int local = b - g.tile0;
     const int yt = local / g.Lx;
     const int x = local - yt * g.Lx;
-    const int y = yt * BY + threadIdx.x;
-    if (y < 3 || y >= g.Ly - 3) return;  // the wall tiles'
+    const int y0 = yt * ROWS, y = y0 + threadIdx.x;
+    if (!UNIFORM) {
+      const long long* from = (const long long*)static_cast<const Collision*>(&tab[i].p);
+      for (int k = threadIdx.x; k < (int)(sizeof(Collision) / 8); k += ROWS) ((long long*)&own)[k] = from[k];
+    }
+    stage_init<ROWS>(stage, true, min(ROWS, g.Ly - y0));
     const int c = g.cur ^ parity;
-    const long long i = site_index(g, x, y);
-    const char* s = (const char*)((const double*)g.buf[c] + i);
-    double f[kQ];
+    const double* src = (const double*)g.buf[c];
     double* dst = (double*)g.buf[c ^ 1];
-#pragma unroll
-    for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(s + off[l]);
-    collide_site_to(RegPops{f}, L.common, SharedPlanes{(char*)(dst + i), off + kQ});
-    split_images(dst, g, x, i);
+    const long long at = site_index(g, x, y0);
+    const RowPopsOf<true, ROWS> f = stage_rows<true, ROWS>(stage, (const char*)(src + at), g, min(ROWS, g.Ly - y0));
+    if (f.a == 0 || y >= g.Ly) return;
+    if (!g.periodic_y && (y < 3 || y >= g.Ly - 3)) return;  // the wall tiles'
+    const ToPlanesStride out{dst + at + threadIdx.x, g.plane};
+    if constexpr (UNIFORM)
+      collide_site_to(f, L.common, out);
+    else
+      collide_site_to(f, own, out);
+    store_images<false>(dst, g, x, y);
     return;
   }
   // wall tile: kWallGroupsPerWarp (column, wall) groups per warp, one lane per wall row
   const int w = b - L.site_tiles;
-  const BatchGeo& g = L.g[split_owner(L, w, true)];
+  int i = 0;
+  for (int hi = L.n - 1; i < hi;) {  // lattices without walls own no wall tiles: the last with wtile0 <= w
+    const int mid = (i + hi + 1) >> 1;
+    if (L.g[mid].wtile0 <= w)
+      i = mid;
+    else
+      hi = mid - 1;
+  }
+  const BatchGeo& g = L.g[i];
   const int lane = threadIdx.x & 31;
-  const int grp = ((w - g.wtile0) * (BY / 32) + (threadIdx.x >> 5)) * kWallGroupsPerWarp + lane / 3;
+  const int grp = ((w - g.wtile0) * (ROWS / 32) + (threadIdx.x >> 5)) * kWallGroupsPerWarp + lane / 3;
   const int r = lane - 3 * (lane / 3);
   const bool active = lane < 3 * kWallGroupsPerWarp && grp < 2 * g.Lx;
   const int x = grp >> 1, wall = grp & 1;
@@ -1109,15 +1090,19 @@ __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? 
   const double s2 = __shfl_sync(0xffffffffu, sum, base + 2);
   if (!active) return;
   const int y = wall ? g.Ly - 1 - r : r;
-  const long long i = site_index(g, x, y);
-  const char* s = (const char*)(src + i);
+  const long long at = site_index(g, x, y);
   double f[kQ];
 #pragma unroll
-  for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(s + g.pull_off[l]);
-  apply_wall(f, tab[g.entry].p.fw[wall], wall, r, ((s0 + s1) + s2) * g.inv_denom[wall]);
+  for (int l = 0; l < kQ; ++l) f[l] = src[l * g.plane + at - vel_cx(l) * g.NY - vel_cy(l)];
+  const StepParams& p = tab[i].p;
+  apply_wall(f, p.fw[wall], wall, r, ((s0 + s1) + s2) * g.inv_denom[wall]);
   double* dst = (double*)g.buf[c ^ 1];
-  collide_site_to(RegPops{f}, L.common, GeoPlanes{(char*)(dst + i), g});
-  split_images(dst, g, x, i);
+  const ToPlanesStride out{dst + at, g.plane};
+  if constexpr (UNIFORM)
+    collide_site_to(RegPops{f}, L.common, out);
+  else
+    collide_site_to(RegPops{f}, p, out);
+  store_images<false>(dst, g, x, y);
 }
 
 __global__ void __launch_bounds__(kBlockY) fields_kernel(const double* __restrict__ buf, double* __restrict__ rho,
@@ -1193,13 +1178,6 @@ int wall_grid(const StepParams& p) {
 int done(int n) { return cudaGetLastError() == cudaSuccess ? n : -1; }
 
 }  // namespace
-
-cudaError_t upload_shell_consts(const ShellConsts& c) {
-  cudaError_t e = cudaFuncSetAttribute(fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(collide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
-  return e == cudaSuccess ? cudaMemcpyToSymbol(c_shell, &c, sizeof(c)) : e;
-}
-
 
 int launch_wrap(double* buf, const StepParams& p, cudaStream_t stream) {
   const long long n = (long long)kQ * 6 * (p.periodic_y ? p.Ly + 2 * kHx : p.Ly) +
@@ -1302,16 +1280,47 @@ int launch_batch_fused(const BatchEntry* tab, const int* tile_entry, int n, long
   }
 }
 
-int launch_batch_split(const BatchLaunch& L, const BatchEntry* tab, const int* tile_entry, int parity, int block_y,
-                       cudaStream_t stream) {
+namespace {
+
+template <int ROWS, int BLOCKS>
+cudaError_t allow_tile_memory() {
+  const cudaError_t e = cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS));
+  return e == cudaSuccess ? cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, false>,
+                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS))
+                          : e;
+}
+
+template <int ROWS, int BLOCKS>
+int tile_launch(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const int* tile_entry, int parity,
+                cudaStream_t stream) {
   const int grid = L.site_tiles + L.wall_tiles;
+  if (uniform)
+    batch_tile_kernel<ROWS, BLOCKS, true><<<grid, ROWS, stage_bytes(ROWS), stream>>>(L, tab, tile_entry, parity);
+  else
+    batch_tile_kernel<ROWS, BLOCKS, false><<<grid, ROWS, stage_bytes(ROWS), stream>>>(L, tab, tile_entry, parity);
+  return done(1);
+}
+
+}  // namespace
+
+int launch_batch_tiles(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const int* tile_entry, int parity,
+                       int block_y, cudaStream_t stream) {
   switch (block_y) {
-    case 64: batch_split_kernel<64><<<grid, 64, 0, stream>>>(L, tab, tile_entry, parity); break;
-    case 128: batch_split_kernel<128><<<grid, 128, 0, stream>>>(L, tab, tile_entry, parity); break;
-    case 256: batch_split_kernel<256><<<grid, 256, 0, stream>>>(L, tab, tile_entry, parity); break;
+    case 64: return tile_launch<64, 10>(L, uniform, tab, tile_entry, parity, stream);
+    case 128: return tile_launch<128, 5>(L, uniform, tab, tile_entry, parity, stream);
+    case 256: return tile_launch<256, 3>(L, uniform, tab, tile_entry, parity, stream);
     default: return -1;
   }
-  return done(1);
+}
+
+cudaError_t upload_shell_consts(const ShellConsts& c) {
+  cudaError_t e = cudaFuncSetAttribute(fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(collide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStageBytes);
+  if (e == cudaSuccess) e = allow_tile_memory<64, 10>();
+  if (e == cudaSuccess) e = allow_tile_memory<128, 5>();
+  if (e == cudaSuccess) e = allow_tile_memory<256, 3>();
+  return e == cudaSuccess ? cudaMemcpyToSymbol(c_shell, &c, sizeof(c)) : e;
 }
 
 int batch_wall_groups_per_tile(int block_y) { return (block_y / 32) * kWallGroupsPerWarp; }

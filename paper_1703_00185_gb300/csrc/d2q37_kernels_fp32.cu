@@ -506,19 +506,30 @@ __global__ void __launch_bounds__(BY, (D2Q37_FP32_MIN_BLOCKS * 128) / BY) batch_
 // lattice's geometry and collision constants come from the launch's parameter
 // space (BatchLaunch32), its wall constants from its entry of the table.  The
 // per-site arithmetic is fused32_kernel's.
-static_assert(sizeof(BatchLaunch32) <= 32764, "BatchLaunch32 must fit the kernel parameter space");
+static_assert(sizeof(BatchLaunch32) <= 32700, "BatchLaunch32 must fit the kernel parameter space");
 
 template <class W, int BY>
 __global__ void __launch_bounds__(BY, (D2Q37_FP32_MIN_BLOCKS * 128) / BY)
-    batch_split32_kernel(const __grid_constant__ BatchLaunch32 L, const int* __restrict__ tile_entry, int parity) {
+    batch_tile32_kernel(const __grid_constant__ BatchLaunch32 L, const BatchEntry* __restrict__ tab,
+                        const int* __restrict__ tile_entry, int parity) {
   const int b = blockIdx.x;
   // the lattice's parameters in shared memory: the blocks of an SM serve
   // different lattices, whose parameter slices would crowd the constant cache
   __shared__ BatchGeo32 g;
-  static_assert(sizeof(BatchGeo32) % sizeof(int) == 0, "BatchGeo32 is copied as ints");
+  static_assert(sizeof(BatchLat32) % sizeof(int) == 0, "BatchLat32 is copied as ints");
   {
-    const int* from = (const int*)&L.g[tile_entry[b]];
-    for (int k = threadIdx.x; k < (int)(sizeof(BatchGeo32) / sizeof(int)); k += BY) ((int*)&g)[k] = from[k];
+    const int i = tile_entry ? tile_entry[b] : batch_owner(L, b);
+    const int* from = (const int*)&L.g[i];
+    int* to = (int*)static_cast<BatchLat32*>(&g);
+    for (int k = threadIdx.x; k < (int)(sizeof(BatchLat32) / sizeof(int)); k += BY) to[k] = from[k];
+    if (threadIdx.x == 0) {
+      const StepParams& p = tab[i].p;
+      g.Hy = kHy32;
+      g.fw32 = p.fw32;
+      g.fwmw32 = p.fwmw32;
+      g.wall_e32 = p.wall_e32;
+      g.wall_inv32 = p.wall_inv32;
+    }
   }
   __syncthreads();
   const int local = b - g.tile0;
@@ -700,20 +711,21 @@ int launch_batch_fused32(const BatchEntry* tab, const int* tile_entry, int n, lo
 }
 
 template <class W, int BY>
-int split32_launch(const BatchLaunch32& L, const int* tile_entry, int tiles, int parity, cudaStream_t stream) {
-  batch_split32_kernel<W, BY><<<tiles, BY, 0, stream>>>(L, tile_entry, parity);
-  return cudaGetLastError() == cudaSuccess ? 1 : -1;
+int tile32_launch(const BatchLaunch32& L, const BatchEntry* tab, const int* tile_entry, int tiles, int parity,
+                  cudaStream_t stream) {
+  batch_tile32_kernel<W, BY><<<tiles, BY, 0, stream>>>(L, tab, tile_entry, parity);
+  return done(1);
 }
 
-int launch_batch_split32(const BatchLaunch32& L, const int* tile_entry, int tiles, int parity, int block_y,
-                         bool wide_fp64, cudaStream_t stream) {
+int launch_batch_tiles32(const BatchLaunch32& L, const BatchEntry* tab, const int* tile_entry, int tiles, int parity,
+                         int block_y, bool wide_fp64, cudaStream_t stream) {
   switch (block_y) {
-    case 64: return wide_fp64 ? split32_launch<WideF64, 64>(L, tile_entry, tiles, parity, stream)
-                              : split32_launch<WideDF, 64>(L, tile_entry, tiles, parity, stream);
-    case 128: return wide_fp64 ? split32_launch<WideF64, 128>(L, tile_entry, tiles, parity, stream)
-                               : split32_launch<WideDF, 128>(L, tile_entry, tiles, parity, stream);
-    case 256: return wide_fp64 ? split32_launch<WideF64, 256>(L, tile_entry, tiles, parity, stream)
-                               : split32_launch<WideDF, 256>(L, tile_entry, tiles, parity, stream);
+    case 64: return wide_fp64 ? tile32_launch<WideF64, 64>(L, tab, tile_entry, tiles, parity, stream)
+                              : tile32_launch<WideDF, 64>(L, tab, tile_entry, tiles, parity, stream);
+    case 128: return wide_fp64 ? tile32_launch<WideF64, 128>(L, tab, tile_entry, tiles, parity, stream)
+                               : tile32_launch<WideDF, 128>(L, tab, tile_entry, tiles, parity, stream);
+    case 256: return wide_fp64 ? tile32_launch<WideF64, 256>(L, tab, tile_entry, tiles, parity, stream)
+                               : tile32_launch<WideDF, 256>(L, tab, tile_entry, tiles, parity, stream);
     default: return -1;
   }
 }

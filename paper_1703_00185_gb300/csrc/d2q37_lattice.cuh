@@ -116,30 +116,12 @@ struct ShellConsts32 {
   float delta[kShells], eps[kShells];  // (x2 - 4)/2, (x2 - 6)/4
 };
 
-// Per-lattice parameters of one step, passed by value to every kernel.
-struct StepParams {
-  int Lx, Ly;
-  int NY;          // column stride (elements)
-  int Hy;          // halo rows below the lattice (16 for FP64, 32 for FP32 storage)
-  int periodic_y;
-  long long plane; // population plane stride (elements) = (Lx + 2 kHx) * NY
-  // byte offsets from a site to the source of its pull (l plane - c_l . (NY, 1))
-  // and to its population planes (l plane), for the single-lattice kernels
-  long long pull_off[kQ], plane_off[kQ];
-  float omega_f, keep_f;  // 1/tau and 1 - 1/tau rounded to FP32 (FP32 storage)
-  float uy_shift_df[2];    // uy_shift and theta_shift as double-float (hi, lo) pairs
-  float theta_shift_df[2];
-  double omega;    // 1 / tau
+// What the FP64 collision of a site takes from a lattice's parameters.
+struct Collision {
+  double omega;  // 1 / tau
   double one_minus_omega;
-  double uy_shift;    // tau g_y = -tau g0: u_bar = u + tau g (Eq. MASTERSHIFT3)
-  double theta_shift; // T_bar - 1 - T = -tau^2 g0^2 / D - 1
-  double fw[2][kQ];   // wall equilibria f^eq(1, 0, T_wall): [0] bottom, [1] top
-  double inv_denom[2];// 1 / sum of fw over the missing (row, population) pairs
-  // the same for the FP32-storage walls, rounded once from FP64:
-  float fw32[2][kQ];    // fw
-  float fwmw32[2][kQ];  // fw - w
-  float wall_e32[2][2];   // (hi, lo): sum_M fwmw32 - sum_O w + sum_M w (M missing, O leaving pairs)
-  float wall_inv32[2][2]; // (hi, lo): 1 / sum_M fw32
+  double uy_shift;     // tau g_y = -tau g0: u_bar = u + tau g (Eq. MASTERSHIFT3)
+  double theta_shift;  // T_bar - 1 - T = -tau^2 g0^2 / D - 1
   // Fixed-point equilibrium constants of the FP64 step: per shell k,
   // omega w_k = c_k 2^E_k with c_k in [0.5, 1); as unsigned integers, each
   // at the scale that puts its product straight into the format it feeds:
@@ -160,6 +142,28 @@ struct StepParams {
   int fx_on;                  // 0: the shifts do not fit the formats, every site takes FP64
 };
 
+// Per-lattice parameters of one step, passed by value to every kernel.
+struct StepParams : Collision {
+  int Lx, Ly;
+  int NY;          // column stride (elements)
+  int Hy;          // halo rows below the lattice (16 for FP64, 32 for FP32 storage)
+  int periodic_y;
+  long long plane; // population plane stride (elements) = (Lx + 2 kHx) * NY
+  // byte offsets from a site to the source of its pull (l plane - c_l . (NY, 1))
+  // and to its population planes (l plane), for the single-lattice kernels
+  long long pull_off[kQ], plane_off[kQ];
+  float omega_f, keep_f;  // 1/tau and 1 - 1/tau rounded to FP32 (FP32 storage)
+  float uy_shift_df[2];    // uy_shift and theta_shift as double-float (hi, lo) pairs
+  float theta_shift_df[2];
+  double fw[2][kQ];   // wall equilibria f^eq(1, 0, T_wall): [0] bottom, [1] top
+  double inv_denom[2];// 1 / sum of fw over the missing (row, population) pairs
+  // the same for the FP32-storage walls, rounded once from FP64:
+  float fw32[2][kQ];    // fw
+  float fwmw32[2][kQ];  // fw - w
+  float wall_e32[2][2];   // (hi, lo): sum_M fwmw32 - sum_O w + sum_M w (M missing, O leaving pairs)
+  float wall_inv32[2][2]; // (hi, lo): 1 / sum_M fw32
+};
+
 // One lattice of a batched launch.  Tiles are one column x by `block_y`
 // consecutive rows; this lattice owns tiles [tile0, tile0 + Lx * ytiles).
 struct BatchEntry {
@@ -170,59 +174,72 @@ struct BatchEntry {
   long long tile0;  // first tile of this lattice
 };
 
-// One lattice of a split batched launch (FP64, walls): its geometry, with
-// the 37 pull and plane offsets as 32-bit byte offsets, in the launch's
-// parameter space (BatchLaunch), where every block reads it through the
-// constant cache.  Site tiles are one column x `block_y` rows (the rows
-// outside the wall bands); wall tiles hold kBatchWallGroups (column, wall)
-// groups of three wall rows each.
+// One lattice of a batched launch with one block per tile: its geometry, in
+// the launch's parameter space (BatchLaunch), where every block reads it
+// through the constant cache.  Site tiles are one column x `block_y` rows; with
+// walls the rows of the wall bands are left to the wall tiles (ten (column,
+// wall) groups of three rows a warp).
 struct BatchGeo {
-  int pull_off[kQ];   // byte offset from a site to the source of its pull
-  int plane_off[kQ];  // byte offset from a site to its element of plane l
   int Lx, Ly, NY, Hy;
-  int ytiles;         // site tiles per column
+  int periodic_y;
   int tile0, wtile0;  // first site tile and first wall tile of this lattice
   int cur;            // buffer holding the state when the launch parity is 0
-  int entry;          // index of this lattice in the BatchEntry table (wall equilibria)
   long long plane;    // population plane stride (elements)
   void* buf[2];
   double inv_denom[2];
 };
 
-constexpr int kBatchGeoMax = 64;       // lattices per split launch (parameter space: 32 KB)
-constexpr int kBatchWallGroups = 40;   // (column, wall) groups per wall tile: 10 per warp, 4 warps
+constexpr int kBatchGeoMax = 384;  // lattices per launch (parameter space: 32 KB)
 
 struct BatchLaunch {
-  StepParams common;  // the collision constants every lattice shares (same tau and g)
+  Collision common;  // the collision constants, when every lattice has the same tau and g
   int n;
   int site_tiles, wall_tiles;
   BatchGeo g[kBatchGeoMax];
 };
 
-// One lattice of a split batched launch in FP32 storage (BatchLaunch32): the
-// fields of StepParams that the FP32 per-site code reads, under the same
-// names, with the wall constants as pointers into the lattice's entry of the
-// BatchEntry table (device memory; only wall rows read them).
-struct BatchGeo32 {
-  int Lx, Ly, NY, Hy, periodic_y;
+// The same in FP32 storage (BatchLaunch32), with the collision's parameters.
+struct BatchLat32 {
+  int Lx, Ly, NY, periodic_y;
   int tile0, cur;
   long long plane;
   void* buf[2];
   float omega_f, keep_f;
   float uy_shift_df[2], theta_shift_df[2];
   double theta_shift;
+};
+
+constexpr int kBatchGeo32Max = 384;  // lattices per launch
+
+struct BatchLaunch32 {
+  int n;
+  BatchLat32 g[kBatchGeo32Max];
+};
+
+// What the FP32 per-site code reads of a lattice of a batched launch: the
+// fields of StepParams under the same names, the wall constants by pointer into
+// the lattice's entry of the BatchEntry table (only wall rows read them).
+struct BatchGeo32 : BatchLat32 {
+  int Hy;
   const float (*fw32)[kQ];
   const float (*fwmw32)[kQ];
   const float (*wall_e32)[2];
   const float (*wall_inv32)[2];
 };
 
-constexpr int kBatchGeo32Max = 128;  // lattices per split FP32 launch
-
-struct BatchLaunch32 {
-  int n;
-  BatchGeo32 g[kBatchGeo32Max];
-};
+// Index of the lattice of a launch that owns tile t (tile0 ascending from 0).
+template <class L>
+__device__ __forceinline__ int batch_owner(const L& l, int t) {
+  int lo = 0, hi = l.n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (l.g[mid].tile0 <= t)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  return lo;
+}
 
 // Index of the entry owning tile t (entries sorted by tile0, tile0[0] = 0).
 __device__ __forceinline__ int batch_entry_of(const BatchEntry* __restrict__ tab, int n, long long t) {

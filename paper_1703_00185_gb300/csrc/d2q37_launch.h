@@ -48,19 +48,20 @@ int launch_fields32(const float* buf, double* rho, double* u, double* T, const S
 int launch_batch_fused(const BatchEntry* tab, const int* tile_entry, int n, long long tiles, int parity,
                        int block_y, int grid, const StepParams* common, cudaStream_t stream);
 int batch_blocks_per_sm(int block_y);
-// The split form of the batched FP64 step (one launch: site tiles, then wall
-// tiles; see BatchLaunch); the (column, wall) groups one wall tile holds.
-// tile_entry: owning lattice of every site tile (the batch's per-tile table).
-int launch_batch_split(const BatchLaunch& L, const BatchEntry* tab, const int* tile_entry, int parity, int block_y,
-                       cudaStream_t stream);
+// The batched FP64 step with one block per tile (see BatchLaunch); uniform:
+// every lattice has the collision constants L.common.  tab: the BatchEntry
+// table (device: wall equilibria and, if not uniform, collision constants).
+// tile_entry: owning lattice of every site tile (device), or null for a search.
+// The (column, wall) groups one wall tile holds.
+int launch_batch_tiles(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const int* tile_entry, int parity,
+                       int block_y, cudaStream_t stream);
 int batch_wall_groups_per_tile(int block_y);
 int launch_batch_fused32(const BatchEntry* tab, const int* tile_entry, int n, long long tiles, int parity,
                          int block_y, int grid, bool wide_fp64, cudaStream_t stream);
 int batch32_blocks_per_sm(int block_y, bool wide_fp64);
-// FP32 storage, one block per tile with every lattice's parameters in the
-// launch's parameter space (BatchLaunch32); tiles: grid size.
-int launch_batch_split32(const BatchLaunch32& L, const int* tile_entry, int tiles, int parity, int block_y,
-                         bool wide_fp64, cudaStream_t stream);
+// The same in FP32 storage (BatchLaunch32); tiles: grid size.
+int launch_batch_tiles32(const BatchLaunch32& L, const BatchEntry* tab, const int* tile_entry, int tiles, int parity,
+                         int block_y, bool wide_fp64, cudaStream_t stream);
 
 // One population plane between a contiguous FP64 [Lx][Ly] array (f) and the
 // FP32 deviation frame (d = f - w_l).
