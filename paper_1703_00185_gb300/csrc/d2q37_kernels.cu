@@ -605,7 +605,7 @@ __device__ __forceinline__ double wall_row_outgoing(const double* __restrict__ s
 #pragma unroll
   for (int l = 0; l < kQ; ++l) {
     const int cy = vel_cy(l);
-    if (wall ? (cy > r) : (cy < -r)) s += src[l * p.plane + i];
+    if (wall ? (cy > r) : (cy < -r)) s += __ldcg(src + (l * p.plane + i));
   }
   return s;
 }
@@ -949,6 +949,8 @@ __global__ void __launch_bounds__(ROWS, kFewWarps * 32 / ROWS) fused_few_kernel(
 // 30 and 31 idle); every lane sums the populations of its own row that leave
 // through the wall, and the group's three row sums meet by warp shuffles, so
 // the column's outgoing mass is read once instead of once per wall site.
+// Its loads of the source go to L2 (ld.global.cg): no line that this SM's L1
+// may hold from an earlier step.
 // When it is launched as a programmatic dependent of fused_kernel it may run
 // while that kernel's last blocks still run; every thread then waits for the
 // sites kernel to complete (griddepcontrol.wait: the prerequisite grid has
@@ -979,7 +981,7 @@ __global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* __r
     double f[kQ];
     const char* sp = (const char*)(src + i);
 #pragma unroll
-    for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(sp + p.pull_off[l]);
+    for (int l = 0; l < kQ; ++l) f[l] = __ldcg((const double*)(sp + p.pull_off[l]));
     apply_wall(f, p.fw[wall], wall, r, ((s0 + s1) + s2) * p.inv_denom[wall]);
     collide_site_to(RegPops{f}, p, ToPlanes{(char*)(dst + i), p});
     store_images<true>(dst, p, x, y);
