@@ -1,5 +1,6 @@
 // C ABI of the D2Q37 library (declared in include/d2q37.h): handle life
 // cycle, device memory layout, step scheduling and host<->device transfers.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -166,7 +167,9 @@ size_t buffer_bytes(int Lx, int Ly, int prec) {
   return align256((size_t)kQ * (size_t)(Lx + 2 * kHx) * (size_t)frame_ny(Ly, prec) * elem_bytes(prec));
 }
 
-size_t scratch_bytes(int Lx, int Ly) { return align256((size_t)4 * Lx * Ly * sizeof(double)); }
+constexpr int kScratchPlanes = 4;  // FP64 planes of Lx x Ly the scratch holds
+
+size_t scratch_bytes(int Lx, int Ly) { return align256((size_t)kScratchPlanes * Lx * Ly * sizeof(double)); }
 
 void fill_step_params(lbm_t* h) {
   StepParams& sp = h->sp;
@@ -544,24 +547,26 @@ int lbm_set_populations(lbm_t* h, const double* f) {
   if (!h || !f) return LBM_EINVAL;
   char* d = (char*)h->buf[h->cur];
   const size_t n = (size_t)h->Lx * h->Ly;
-  for (int l = 0; l < kQ; ++l) {
-    if (!is_fp32(h->prec)) {
+  if (!is_fp32(h->prec)) {
+    for (int l = 0; l < kQ; ++l)
       if (cudaMemcpy2DAsync(d + plane_offset_bytes(h, l), h->NY * sizeof(double), f + (size_t)l * n,
                             h->Ly * sizeof(double), h->Ly * sizeof(double), h->Lx, cudaMemcpyHostToDevice,
                             h->stream) != cudaSuccess)
         return LBM_ECUDA;
-      continue;
+  } else {
+    // FP32 storage: FP64 planes staged in scratch, converted to deviations on the device
+    for (int l = 0; l < kQ; l += kScratchPlanes) {
+      const int m = std::min(kScratchPlanes, kQ - l);
+      if (cudaMemcpyAsync(h->scratch, f + (size_t)l * n, m * n * sizeof(double), cudaMemcpyHostToDevice, h->stream) !=
+          cudaSuccess)
+        return LBM_ECUDA;
+      const int rc = run_kernel(h, LBM_KIND_CONVERT, [&] {
+        return launch_planes_to_frame32((float*)h->buf[h->cur], h->scratch, l, m, h->sp, h->stream);
+      });
+      if (rc) return rc;
     }
-    // FP32 storage: stage the FP64 plane in scratch, convert to deviations on the device
-    if (cudaMemcpyAsync(h->scratch, f + (size_t)l * n, n * sizeof(double), cudaMemcpyHostToDevice, h->stream) !=
-        cudaSuccess)
-      return LBM_ECUDA;
-    const int rc = run_kernel(h, LBM_KIND_CONVERT, [&] {
-      return launch_plane_to_frame32((float*)h->buf[h->cur], h->scratch, l, h->sp, h->stream);
-    });
-    if (rc) return rc;
+    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LBM_ECUDA;
   }
-  if (is_fp32(h->prec) && cudaStreamSynchronize(h->stream) != cudaSuccess) return LBM_ECUDA;
   h->have_state = true;
   h->halo_valid = false;
   return LBM_OK;
@@ -572,21 +577,23 @@ int lbm_get_populations(lbm_t* h, double* f) {
   if (!h->have_state) return LBM_ESTATE;
   const char* d = (const char*)h->buf[h->cur];
   const size_t n = (size_t)h->Lx * h->Ly;
-  for (int l = 0; l < kQ; ++l) {
-    if (!is_fp32(h->prec)) {
+  if (!is_fp32(h->prec)) {
+    for (int l = 0; l < kQ; ++l)
       if (cudaMemcpy2DAsync(f + (size_t)l * n, h->Ly * sizeof(double), d + plane_offset_bytes(h, l),
                             h->NY * sizeof(double), h->Ly * sizeof(double), h->Lx, cudaMemcpyDeviceToHost,
                             h->stream) != cudaSuccess)
         return LBM_ECUDA;
-      continue;
+  } else {
+    for (int l = 0; l < kQ; l += kScratchPlanes) {
+      const int m = std::min(kScratchPlanes, kQ - l);
+      const int rc = run_kernel(h, LBM_KIND_CONVERT, [&] {
+        return launch_frame32_to_planes(h->scratch, (const float*)h->buf[h->cur], l, m, h->sp, h->stream);
+      });
+      if (rc) return rc;
+      if (cudaMemcpyAsync(f + (size_t)l * n, h->scratch, m * n * sizeof(double), cudaMemcpyDeviceToHost, h->stream) !=
+          cudaSuccess)
+        return LBM_ECUDA;
     }
-    const int rc = run_kernel(h, LBM_KIND_CONVERT, [&] {
-      return launch_frame32_to_plane(h->scratch, (const float*)h->buf[h->cur], l, h->sp, h->stream);
-    });
-    if (rc) return rc;
-    if (cudaMemcpyAsync(f + (size_t)l * n, h->scratch, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream) !=
-        cudaSuccess)
-      return LBM_ECUDA;
   }
   return check(cudaStreamSynchronize(h->stream));
 }

@@ -637,23 +637,28 @@ __global__ void __launch_bounds__(kBlockY) fields32_kernel(const float* __restri
   T[o] = t;
 }
 
-__global__ void __launch_bounds__(kBlockY) plane_to_frame32_kernel(float* __restrict__ frame,
-                                                                   const double* __restrict__ plane, int l,
-                                                                   StepParams p) {
-  const int x = blockIdx.x;
+// Populations l0 .. l0 + gridDim.z - 1 between contiguous FP64 planes and the
+// FP32 deviation frame.  Several planes a launch: with one, the copies over the
+// host link waited for 37 kernels each way (512 x 1024 up and down, 4 steps:
+// 2.63 ms; 2.06 ms with four).
+__global__ void __launch_bounds__(kBlockY) planes_to_frame32_kernel(float* __restrict__ frame,
+                                                                    const double* __restrict__ planes, int l0,
+                                                                    StepParams p) {
+  const int x = blockIdx.x, l = l0 + blockIdx.z;
   const int y = blockIdx.y * kBlockY + threadIdx.x;
   if (y >= p.Ly) return;
   frame[l * p.plane + site_index(p, x, y)] =
-      (float)(plane[(long long)x * p.Ly + y] - c_shell32.w64[vel_shell(l)]);
+      (float)(planes[((long long)blockIdx.z * p.Lx + x) * p.Ly + y] - c_shell32.w64[vel_shell(l)]);
 }
 
-__global__ void __launch_bounds__(kBlockY) frame32_to_plane_kernel(double* __restrict__ plane,
-                                                                   const float* __restrict__ frame, int l,
-                                                                   StepParams p) {
-  const int x = blockIdx.x;
+__global__ void __launch_bounds__(kBlockY) frame32_to_planes_kernel(double* __restrict__ planes,
+                                                                    const float* __restrict__ frame, int l0,
+                                                                    StepParams p) {
+  const int x = blockIdx.x, l = l0 + blockIdx.z;
   const int y = blockIdx.y * kBlockY + threadIdx.x;
   if (y >= p.Ly) return;
-  plane[(long long)x * p.Ly + y] = c_shell32.w64[vel_shell(l)] + (double)frame[l * p.plane + site_index(p, x, y)];
+  planes[((long long)blockIdx.z * p.Lx + x) * p.Ly + y] =
+      c_shell32.w64[vel_shell(l)] + (double)frame[l * p.plane + site_index(p, x, y)];
 }
 
 dim3 site_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kBlockY - 1) / kBlockY); }
@@ -662,13 +667,19 @@ int done(int n) { return cudaGetLastError() == cudaSuccess ? n : -1; }
 
 }  // namespace
 
-int launch_plane_to_frame32(float* frame, const double* plane, int l, const StepParams& p, cudaStream_t stream) {
-  plane_to_frame32_kernel<<<site_grid(p), kBlockY, 0, stream>>>(frame, plane, l, p);
+int launch_planes_to_frame32(float* frame, const double* planes, int l0, int count, const StepParams& p,
+                             cudaStream_t stream) {
+  dim3 grid = site_grid(p);
+  grid.z = count;
+  planes_to_frame32_kernel<<<grid, kBlockY, 0, stream>>>(frame, planes, l0, p);
   return done(1);
 }
 
-int launch_frame32_to_plane(double* plane, const float* frame, int l, const StepParams& p, cudaStream_t stream) {
-  frame32_to_plane_kernel<<<site_grid(p), kBlockY, 0, stream>>>(plane, frame, l, p);
+int launch_frame32_to_planes(double* planes, const float* frame, int l0, int count, const StepParams& p,
+                             cudaStream_t stream) {
+  dim3 grid = site_grid(p);
+  grid.z = count;
+  frame32_to_planes_kernel<<<grid, kBlockY, 0, stream>>>(planes, frame, l0, p);
   return done(1);
 }
 

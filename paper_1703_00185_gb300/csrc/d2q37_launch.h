@@ -63,9 +63,11 @@ int batch32_blocks_per_sm(int block_y, bool wide_fp64);
 int launch_batch_tiles32(const BatchLaunch32& L, const BatchEntry* tab, const int* tile_entry, int tiles, int parity,
                          int block_y, bool wide_fp64, cudaStream_t stream);
 
-// One population plane between a contiguous FP64 [Lx][Ly] array (f) and the
-// FP32 deviation frame (d = f - w_l).
-int launch_plane_to_frame32(float* frame, const double* plane, int l, const StepParams& p, cudaStream_t stream);
-int launch_frame32_to_plane(double* plane, const float* frame, int l, const StepParams& p, cudaStream_t stream);
+// Populations l0 .. l0 + count - 1 between contiguous FP64 [count][Lx][Ly]
+// planes and the FP32 deviation frame (d = f - w_l).
+int launch_planes_to_frame32(float* frame, const double* planes, int l0, int count, const StepParams& p,
+                             cudaStream_t stream);
+int launch_frame32_to_planes(double* planes, const float* frame, int l0, int count, const StepParams& p,
+                             cudaStream_t stream);
 
 }  // namespace d2q37
