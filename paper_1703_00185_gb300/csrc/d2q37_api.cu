@@ -303,8 +303,9 @@ int k_fused(lbm_t* h, const void* s, void* d) {
 }
 
 int k_fields(lbm_t* h, const void* b, double* rho, double* u, double* T) {
-  return is_fp32(h->prec) ? launch_fields32((const float*)b, rho, u, T, h->sp, h->stream)
-                          : launch_fields((const double*)b, rho, u, T, h->sp, h->stream);
+  const bool chain = !h->timing && !h->shares_device;  // as k_fused
+  return is_fp32(h->prec) ? launch_fields32((const float*)b, rho, u, T, h->sp, h->stream, chain)
+                          : launch_fields((const double*)b, rho, u, T, h->sp, h->stream, chain);
 }
 
 int setup_handle(lbm_t* h, int Lx, int Ly, const lbm_params* p, void* mem, cudaStream_t stream) {

@@ -21,6 +21,8 @@
 // (the paper's 1-D blocks along y, Sec. "The propagate and bc Kernels").
 // Every warp reads 32 consecutive doubles of each population plane, so each
 // gather is a coalesced 256-byte row shifted by at most 3 elements.
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "d2q37_launch.h"
@@ -1110,6 +1112,7 @@ __global__ void __launch_bounds__(ROWS, BLOCKS)
 __global__ void __launch_bounds__(kBlockY) fields_kernel(const double* __restrict__ buf, double* __restrict__ rho,
                                                          double* __restrict__ u, double* __restrict__ T,
                                                          StepParams p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // chained to the step before it (see fused_kernel)
   const int x = blockIdx.x;
   const int y = blockIdx.y * kBlockY + threadIdx.x;
   if (y >= p.Ly) return;
@@ -1217,9 +1220,10 @@ int sm_count() {
   return n;
 }
 
-// Launch as a programmatic dependent of the kernel before it in the stream.
+// Launch; dependent: as a programmatic dependent of the kernel before it in the stream.
 template <class... A>
-cudaError_t launch_dependent(void (*kernel)(A...), dim3 grid, int block, int smem, cudaStream_t stream, A... args) {
+bool launch_pdl(void (*kernel)(A...), dim3 grid, int block, int smem, cudaStream_t stream, bool dependent,
+                std::common_type_t<A>... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
@@ -1229,8 +1233,8 @@ cudaError_t launch_dependent(void (*kernel)(A...), dim3 grid, int block, int sme
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess;
 }
 
 int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap, bool chain) {
@@ -1241,17 +1245,9 @@ int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream
       !few ? fused_kernel : p.periodic_y ? fused_few_kernel<32> : fused_few_kernel<128>;
   const int rows = !few ? kStageRows : p.periodic_y ? 32 : 128, smem = few ? 0 : kStageBytes;
   const dim3 grid(p.Lx, (p.Ly + rows - 1) / rows);
-  if (chain) {
-    if (launch_dependent(sites, grid, rows, smem, stream, src, dst, p) != cudaSuccess) return -1;
-  } else {
-    sites<<<grid, rows, smem, stream>>>(src, dst, p);
-  }
+  if (!launch_pdl(sites, grid, rows, smem, stream, chain, src, dst, p)) return -1;
   if (p.periodic_y) return done(1);
-  if (!overlap) {
-    wall_band_kernel<<<wall_grid(p), kWallBlock, 0, stream>>>(src, dst, p);
-    return done(2);
-  }
-  if (launch_dependent(wall_band_kernel, dim3(wall_grid(p)), kWallBlock, 0, stream, src, dst, p) != cudaSuccess) return -1;
+  if (!launch_pdl(wall_band_kernel, dim3(wall_grid(p)), kWallBlock, 0, stream, overlap, src, dst, p)) return -1;
   return done(2);
 }
 
@@ -1336,9 +1332,9 @@ int batch_blocks_per_sm(int block_y) {
   }
 }
 
-int launch_fields(const double* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream) {
-  fields_kernel<<<site_grid(p), kBlockY, 0, stream>>>(buf, rho, u, T, p);
-  return done(1);
+int launch_fields(const double* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream,
+                  bool chain) {
+  return launch_pdl(fields_kernel, site_grid(p), kBlockY, 0, stream, chain, buf, rho, u, T, p) ? done(1) : -1;
 }
 
 int launch_init_rayleigh_taylor(void* buf, bool fp32, const double* yi, double T_top, double T_bot,

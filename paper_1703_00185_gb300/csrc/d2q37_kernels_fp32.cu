@@ -11,6 +11,8 @@
 //     in FP32, with d' = (1 - omega) d + omega w (rho P - 1).
 // Layout and step sequence are those of the FP64 kernels (d2q37_kernels.cu)
 // with 32 halo rows so FP32 columns stay 128-byte aligned.
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "d2q37_launch.h"
@@ -620,6 +622,7 @@ __global__ void __launch_bounds__(kBlockY, D2Q37_FP32_MIN_BLOCKS) collide32_kern
 __global__ void __launch_bounds__(kBlockY) fields32_kernel(const float* __restrict__ buf, double* __restrict__ rho,
                                                            double* __restrict__ u, double* __restrict__ T,
                                                            StepParams p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // chained to the step before it
   const int x = blockIdx.x;
   const int y = blockIdx.y * kBlockY + threadIdx.x;
   if (y >= p.Ly) return;
@@ -712,18 +715,28 @@ int launch_collide32(float* buf, const StepParams& p, bool wide_fp64, cudaStream
   return done(1);
 }
 
-int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_fp64, cudaStream_t stream, bool chain) {
-  void (*const kernel)(const float*, float*, StepParams) = wide_fp64 ? fused32_kernel<WideF64> : fused32_kernel<WideDF>;
+namespace {
+
+// Launch; dependent: as a programmatic dependent of the kernel before it in the stream.
+template <class... A>
+int launch_pdl32(void (*kernel)(A...), dim3 grid, cudaStream_t stream, bool dependent, std::common_type_t<A>... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = site_grid(p);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(kBlockY);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = chain ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, src, dst, p) == cudaSuccess ? done(1) : -1;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? done(1) : -1;
+}
+
+}  // namespace
+
+int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_fp64, cudaStream_t stream, bool chain) {
+  return launch_pdl32(wide_fp64 ? fused32_kernel<WideF64> : fused32_kernel<WideDF>, site_grid(p), stream, chain, src, dst,
+                      p);
 }
 
 template <class W, int BY>
@@ -782,9 +795,9 @@ int batch32_blocks_per_sm(int block_y, bool wide_fp64) {
   }
 }
 
-int launch_fields32(const float* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream) {
-  fields32_kernel<<<site_grid(p), kBlockY, 0, stream>>>(buf, rho, u, T, p);
-  return done(1);
+int launch_fields32(const float* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream,
+                    bool chain) {
+  return launch_pdl32(fields32_kernel, site_grid(p), stream, chain, buf, rho, u, T, p);
 }
 
 }  // namespace d2q37

@@ -22,7 +22,8 @@ int launch_collide(double* buf, const StepParams& p, cudaStream_t stream);
 // kernel precedes it in the stream (it waits for it before its first access).
 int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap = true,
                  bool chain = false);
-int launch_fields(const double* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream);
+int launch_fields(const double* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream,
+                  bool chain = false);
 // Rayleigh-Taylor initial state, FP64 or FP32 deviations; yi: device, the
 // interface of every column.
 int launch_init_rayleigh_taylor(void* buf, bool fp32, const double* yi, double T_top, double T_bot,
@@ -37,7 +38,8 @@ int launch_bc32(const float* src, float* dst, const StepParams& p, cudaStream_t 
 int launch_collide32(float* buf, const StepParams& p, bool wide_fp64, cudaStream_t stream);
 int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_fp64, cudaStream_t stream,
                    bool chain = false);
-int launch_fields32(const float* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream);
+int launch_fields32(const float* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream,
+                    bool chain = false);
 // Batched fused step over a table of n lattices (BatchEntry, device memory),
 // tiles of block_y rows; block_y in {64, 128, 256}; grid = number of blocks
 // of the grid-stride loop.  *_blocks_per_sm: resident blocks per SM.
