@@ -215,8 +215,10 @@ long long fill_batch_launch(BatchLaunch& L, int n, lbm_t* const* lattices, const
   *uniform = true;
   const int per_wall_tile = batch_wall_groups_per_tile(block_y);
   long long t0 = 0, w0 = 0;
+  L.site_warps = 0;
   for (int i = 0; i < n; ++i) {
     const StepParams& q = lattices[i]->sp;
+    L.site_warps += (long long)q.Lx * ((q.Ly + 31) / 32);
     *uniform = *uniform && q.omega == first.omega && q.uy_shift == first.uy_shift && q.theta_shift == first.theta_shift;
     BatchGeo& g = L.g[i];
     g.Lx = q.Lx;

@@ -1033,7 +1033,7 @@ __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? 
 // walked by grid-stride blocks, 1.33 now (128 rows, 5 blocks per SM).
 static_assert(sizeof(BatchLaunch) <= 32700, "BatchLaunch must fit the kernel parameter space");
 
-template <int ROWS, int BLOCKS, bool UNIFORM>
+template <int ROWS, int BLOCKS, bool UNIFORM, bool STAGED>
 __global__ void __launch_bounds__(ROWS, BLOCKS)
     batch_tile_kernel(const __grid_constant__ BatchLaunch L, const BatchEntry* __restrict__ tab,
                       const int* __restrict__ tile_entry, int parity) {
@@ -1053,20 +1053,39 @@ __global__ void __launch_bounds__(ROWS, BLOCKS)
       const long long* from = (const long long*)static_cast<const Collision*>(&tab[i].p);
       for (int k = threadIdx.x; k < (int)(sizeof(Collision) / 8); k += ROWS) ((long long*)&own)[k] = from[k];
     }
-    stage_init<ROWS>(stage, true, min(ROWS, g.Ly - y0));
-    const int c = g.cur ^ parity;
-    const double* src = (const double*)g.buf[c];
-    double* dst = (double*)g.buf[c ^ 1];
-    const long long at = site_index(g, x, y0);
-    const RowPopsOf<true, ROWS> f = stage_rows<true, ROWS>(stage, (const char*)(src + at), g, min(ROWS, g.Ly - y0));
-    if (f.a == 0 || y >= g.Ly) return;
-    if (!g.periodic_y && (y < 3 || y >= g.Ly - 3)) return;  // the wall tiles'
-    const ToPlanesStride out{dst + at + threadIdx.x, g.plane};
-    if constexpr (UNIFORM)
-      collide_site_to(f, L.common, out);
-    else
-      collide_site_to(f, own, out);
-    store_images<false>(dst, g, x, y);
+    if constexpr (STAGED) {
+      stage_init<ROWS>(stage, true, min(ROWS, g.Ly - y0));
+      const int c = g.cur ^ parity;
+      const double* src = (const double*)g.buf[c];
+      double* dst = (double*)g.buf[c ^ 1];
+      const long long at = site_index(g, x, y0);
+      const RowPopsOf<true, ROWS> f = stage_rows<true, ROWS>(stage, (const char*)(src + at), g, min(ROWS, g.Ly - y0));
+      if (f.a == 0 || y >= g.Ly) return;
+      if (!g.periodic_y && (y < 3 || y >= g.Ly - 3)) return;  // the wall tiles'
+      const ToPlanesStride out{dst + at + threadIdx.x, g.plane};
+      if constexpr (UNIFORM)
+        collide_site_to(f, L.common, out);
+      else
+        collide_site_to(f, own, out);
+      store_images<false>(dst, g, x, y);
+    } else {
+      if (!UNIFORM) __syncthreads();
+      if (y >= g.Ly) return;
+      if (!g.periodic_y && (y < 3 || y >= g.Ly - 3)) return;
+      const int c = g.cur ^ parity;
+      const double* src = (const double*)g.buf[c];
+      double* dst = (double*)g.buf[c ^ 1];
+      const long long at = site_index(g, x, y);
+      double f[kQ];
+#pragma unroll
+      for (int l = 0; l < kQ; ++l) f[l] = src[l * g.plane + at - vel_cx(l) * g.NY - vel_cy(l)];
+      const ToPlanesStride out{dst + at, g.plane};
+      if constexpr (UNIFORM)
+        collide_site_to(RegPops{f}, L.common, out);
+      else
+        collide_site_to(RegPops{f}, own, out);
+      store_images<false>(dst, g, x, y);
+    }
     return;
   }
   // wall tile: kWallGroupsPerWarp (column, wall) groups per warp, one lane per wall row
@@ -1174,6 +1193,18 @@ dim3 site_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kBlockY - 1) / k
 
 dim3 stage_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kStageRows - 1) / kStageRows); }
 
+// SMs of the current device (looked up once; the library is for one kind of GPU).
+int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
+               ? v
+               : 152;
+  }();
+  return n;
+}
+
 // (column, wall) groups of the wall-band kernel: 2 Lx, ten per warp
 int wall_grid(const StepParams& p) {
   constexpr int per_block = kWallGroupsPerWarp * (kWallBlock / 32);
@@ -1206,18 +1237,6 @@ int launch_bc(const double* src, double* dst, const StepParams& p, cudaStream_t 
 int launch_collide(double* buf, const StepParams& p, cudaStream_t stream) {
   collide_kernel<<<stage_grid(p), kStageRows, kStageBytes, stream>>>(buf, p);
   return done(1);
-}
-
-// SMs of the current device (looked up once; the library is for one kind of GPU).
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    return cudaGetDevice(&dev) == cudaSuccess &&
-                   cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
-               ? v
-               : 152;
-  }();
-  return n;
 }
 
 // Launch; dependent: as a programmatic dependent of the kernel before it in the stream.
@@ -1282,21 +1301,32 @@ namespace {
 
 template <int ROWS, int BLOCKS>
 cudaError_t allow_tile_memory() {
-  const cudaError_t e = cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, true>,
+  const cudaError_t e = cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, true, true>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS));
-  return e == cudaSuccess ? cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, false>,
+  return e == cudaSuccess ? cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, false, true>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS))
                           : e;
 }
 
+// Up to this many warps of sites per SM (some waves) the register form (128
+// registers, 16 warps per SM) is the faster one: a wave is one site's chain
+// long, and the bulk copies add theirs.  Microseconds a step in registers /
+// staged, 128 rows: 3 lattices of up to 40 x 80 17.6 / 21.7, 10 of 60 x 120 18.6
+// / 23.0, 10 of 200 x 400 (30 warps per SM) 51 / 59, 60 of 120 x 240 (100)
+// 159 / 162; 64 of up to 1024 x 2048 (8700) 7360 / 6700.
+constexpr int kBatchFewWarps = 200;
+
 template <int ROWS, int BLOCKS>
 int tile_launch(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const int* tile_entry, int parity,
                 cudaStream_t stream) {
+  constexpr int kRegBlocks = 4 * 128 / ROWS;
   const int grid = L.site_tiles + L.wall_tiles;
-  if (uniform)
-    batch_tile_kernel<ROWS, BLOCKS, true><<<grid, ROWS, stage_bytes(ROWS), stream>>>(L, tab, tile_entry, parity);
-  else
-    batch_tile_kernel<ROWS, BLOCKS, false><<<grid, ROWS, stage_bytes(ROWS), stream>>>(L, tab, tile_entry, parity);
+  const bool staged = L.site_warps > (long long)kBatchFewWarps * sm_count();
+  void (*const kernel)(BatchLaunch, const BatchEntry*, const int*, int) =
+      staged ? (uniform ? batch_tile_kernel<ROWS, BLOCKS, true, true> : batch_tile_kernel<ROWS, BLOCKS, false, true>)
+             : (uniform ? batch_tile_kernel<ROWS, kRegBlocks, true, false>
+                        : batch_tile_kernel<ROWS, kRegBlocks, false, false>);
+  kernel<<<grid, ROWS, staged ? stage_bytes(ROWS) : 0, stream>>>(L, tab, tile_entry, parity);
   return done(1);
 }
 

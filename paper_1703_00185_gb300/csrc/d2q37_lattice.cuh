@@ -195,6 +195,7 @@ struct BatchLaunch {
   Collision common;  // the collision constants, when every lattice has the same tau and g
   int n;
   int site_tiles, wall_tiles;
+  long long site_warps;  // warps of 32 rows, over all lattices
   BatchGeo g[kBatchGeoMax];
 };
 
