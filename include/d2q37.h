@@ -40,7 +40,7 @@ extern "C" {
 #define LBM_EINVAL (-1)   /* bad argument: NULL, Lx < 3, Ly < 6, tau <= 0.5, bad phase mask */
 #define LBM_ENOMEM (-2)   /* device allocation failed, or caller buffer too small */
 #define LBM_ECUDA (-3)    /* a CUDA call or kernel launch failed */
-#define LBM_ETIMEOUT (-4) /* reserved for bounded device waits */
+#define LBM_ETIMEOUT (-4) /* a bounded device wait ran out since the last synchronisation */
 #define LBM_ESTATE (-5)   /* call out of order, e.g. a step before any initial state */
 #define LBM_ETOOBIG (-6)  /* more lattices than lbm_batch_step_static's fixed table holds */
 
