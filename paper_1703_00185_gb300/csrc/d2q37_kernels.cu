@@ -599,8 +599,7 @@ __device__ __forceinline__ void collide_site_to(const F& f, const P& p, const O&
 // column's wall rows each sum their own row and combine the sums by warp
 // shuffles (wall_band_kernel), so both give the same bits.
 template <class P>  // StepParams or BatchGeo (Ly, NY, Hy, plane)
-__device__ __forceinline__ double wall_row_outgoing(const double* __restrict__ src, const P& p, int x, int wall,
-                                                    int r) {
+__device__ __forceinline__ double wall_row_outgoing(const double* src, const P& p, int x, int wall, int r) {
   const int y = wall ? p.Ly - 1 - r : r;
   const long long i = site_index(p, x, y);
   double s = 0.0;
@@ -612,8 +611,7 @@ __device__ __forceinline__ double wall_row_outgoing(const double* __restrict__ s
   return s;
 }
 
-__device__ __forceinline__ double wall_density(const double* __restrict__ src, const StepParams& p, int x,
-                                               int wall) {
+__device__ __forceinline__ double wall_density(const double* src, const StepParams& p, int x, int wall) {
   const double s0 = wall_row_outgoing(src, p, x, wall, 0);
   const double s1 = wall_row_outgoing(src, p, x, wall, 1);
   const double s2 = wall_row_outgoing(src, p, x, wall, 2);
@@ -871,17 +869,18 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(doubl
 // collide, store with halo images.
 // p: the lattice (geometry, walls); px: the constants of its collision (tau,
 // g: the fixed-point tables, omega, the field shifts), the same object for a
-// single lattice.  OFF: addresses from the byte offsets of p (see store_images).
+// single lattice.  OFF: addresses from the byte offsets of p (see store_images),
+// and loads of the source from L2 (see launch_pdl).
 // WALLS = false: the caller never passes a wall-band site.
 template <bool OFF, bool WALLS = true>
-__device__ __forceinline__ void fused_site(const double* __restrict__ src, double* __restrict__ dst,
-                                           const StepParams& p, const StepParams& px, int x, int y) {
+__device__ __forceinline__ void fused_site(const double* src, double* dst, const StepParams& p, const StepParams& px,
+                                           int x, int y) {
   const long long i = site_index(p, x, y);
   double f[kQ];
   if constexpr (OFF) {
     const char* s = (const char*)(src + i);
 #pragma unroll
-    for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(s + p.pull_off[l]);
+    for (int l = 0; l < kQ; ++l) f[l] = __ldcg((const double*)(s + p.pull_off[l]));
   } else {
 #pragma unroll
     for (int l = 0; l < kQ; ++l) f[l] = src[l * p.plane + i - vel_cx(l) * p.NY - vel_cy(l)];
@@ -898,8 +897,8 @@ __device__ __forceinline__ void fused_site(const double* __restrict__ src, doubl
   store_images<OFF>(dst, p, x, y);
 }
 
-__global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const double* __restrict__ src,
-                                                                        double* __restrict__ dst, StepParams p) {
+__global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const double* src, double* dst,
+                                                                        StepParams p) {
   extern __shared__ __align__(128) unsigned char stage[];
   const int x = blockIdx.x;
   const int y0 = blockIdx.y * kStageRows;
@@ -932,8 +931,8 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const d
 constexpr int kFewWarps = 8;  // resident per SM at up to 255 registers
 
 template <int ROWS>
-__global__ void __launch_bounds__(ROWS, kFewWarps * 32 / ROWS) fused_few_kernel(const double* __restrict__ src,
-                                                                                double* __restrict__ dst, StepParams p) {
+__global__ void __launch_bounds__(ROWS, kFewWarps * 32 / ROWS) fused_few_kernel(const double* src, double* dst,
+                                                                               StepParams p) {
   const int x = blockIdx.x;
   const int y = blockIdx.y * ROWS + threadIdx.x;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // as fused_kernel
@@ -963,8 +962,7 @@ __global__ void __launch_bounds__(ROWS, kFewWarps * 32 / ROWS) fused_few_kernel(
 // wait returns at once.
 constexpr int kWallGroupsPerWarp = 10;
 
-__global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* __restrict__ src,
-                                                              double* __restrict__ dst, StepParams p) {
+__global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* src, double* dst, StepParams p) {
   // the next step's sites kernel may start in this one's tail (it waits for it)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31;
@@ -1128,8 +1126,7 @@ __global__ void __launch_bounds__(ROWS, BLOCKS)
   store_images<false>(dst, g, x, y);
 }
 
-__global__ void __launch_bounds__(kBlockY) fields_kernel(const double* __restrict__ buf, double* __restrict__ rho,
-                                                         double* __restrict__ u, double* __restrict__ T,
+__global__ void __launch_bounds__(kBlockY) fields_kernel(const double* buf, double* rho, double* u, double* T,
                                                          StepParams p) {
   asm volatile("griddepcontrol.wait;" ::: "memory");  // chained to the step before it (see fused_kernel)
   const int x = blockIdx.x;
@@ -1138,7 +1135,7 @@ __global__ void __launch_bounds__(kBlockY) fields_kernel(const double* __restric
   const long long i = site_index(p, x, y);
   double f[kQ];
 #pragma unroll
-  for (int l = 0; l < kQ; ++l) f[l] = buf[l * p.plane + i];
+  for (int l = 0; l < kQ; ++l) f[l] = __ldcg(buf + (l * p.plane + i));  // see launch_pdl
   double r, ux, uy, t;
   site_moments(f, r, ux, uy, t);
   const long long o = (long long)x * p.Ly + y;
@@ -1239,7 +1236,15 @@ int launch_collide(double* buf, const StepParams& p, cudaStream_t stream) {
   return done(1);
 }
 
-// Launch; dependent: as a programmatic dependent of the kernel before it in the stream.
+// Launch; dependent: as a programmatic dependent of the kernel before it in the
+// stream.  Such a grid may be resident while earlier kernels still write what it
+// reads: after its griddepcontrol.wait those writes are visible to its ordinary
+// loads, but not to loads through the read-only path, whose data must not change
+// while the grid lives.  So no pointer of a kernel launched here is const
+// __restrict__ (which lets the compiler take that path, and move a load above
+// the wait), and the loads of populations go to L2: store_images reads row 3 of
+// the edge columns back, and with it the wall rows of the same sector, which
+// wall_band_kernel may be writing, into the L1 of an SM where the next grid waits.
 template <class... A>
 bool launch_pdl(void (*kernel)(A...), dim3 grid, int block, int smem, cudaStream_t stream, bool dependent,
                 std::common_type_t<A>... args) {

@@ -393,8 +393,7 @@ __device__ __forceinline__ void fields_of_site32(const float (&d)[kQ], double& r
 
 // Halo images as in the FP64 store_site.
 template <class P>
-__device__ __forceinline__ void store_site32(float* __restrict__ dst, const P& p, int x, int y,
-                                             const float (&d)[kQ]) {
+__device__ __forceinline__ void store_site32(float* dst, const P& p, int x, int y, const float (&d)[kQ]) {
   if (x >= kHx && x < p.Lx - kHx && (!p.periodic_y || (y >= kHx && y < p.Ly - kHx))) {
     float* q = dst + (int)site_index(p, x, y);  // no halo image: the common case
 #pragma unroll
@@ -431,8 +430,7 @@ __device__ __forceinline__ void store_site32(float* __restrict__ dst, const P& p
 // with E and 1/D carried as (hi, lo) float pairs, so that no rounding of a
 // constant biases the wall's mass the same way every step.
 template <class P>
-__device__ __forceinline__ float wall_rho_minus_1(const float* __restrict__ src, const P& p, int x,
-                                                  int wall) {
+__device__ __forceinline__ float wall_rho_minus_1(const float* src, const P& p, int x, int wall) {
   float out_d = 0.0f;
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
@@ -485,8 +483,7 @@ __global__ void __launch_bounds__(256) wrap32_kernel(float* __restrict__ buf, St
 // One site of the fused step (pull, wall bc on the wall bands, collide,
 // store with halo images).
 template <class W, class P>
-__device__ __forceinline__ void fused_site32(const float* __restrict__ src, float* __restrict__ dst, const P& p,
-                                             int x, int y) {
+__device__ __forceinline__ void fused_site32(const float* src, float* dst, const P& p, int x, int y) {
   // the site's pointer once per thread; each population at an offset that is
   // the same for the whole block (l plane - cx NY - cy)
   const float* q = src + (int)site_index(p, x, y);
@@ -508,8 +505,7 @@ __device__ __forceinline__ void fused_site32(const float* __restrict__ src, floa
 }
 
 template <class W>
-__global__ void __launch_bounds__(kBlockY, D2Q37_FP32_MIN_BLOCKS) fused32_kernel(const float* __restrict__ src,
-                                                                                 float* __restrict__ dst,
+__global__ void __launch_bounds__(kBlockY, D2Q37_FP32_MIN_BLOCKS) fused32_kernel(const float* src, float* dst,
                                                                                  StepParams p) {
   // launched with programmatic stream serialization (chain), this grid starts
   // in the tail of the previous step's and waits here for it to complete
@@ -619,8 +615,7 @@ __global__ void __launch_bounds__(kBlockY, D2Q37_FP32_MIN_BLOCKS) collide32_kern
 }
 
 // Fields in FP64 from the stored deviations.
-__global__ void __launch_bounds__(kBlockY) fields32_kernel(const float* __restrict__ buf, double* __restrict__ rho,
-                                                           double* __restrict__ u, double* __restrict__ T,
+__global__ void __launch_bounds__(kBlockY) fields32_kernel(const float* buf, double* rho, double* u, double* T,
                                                            StepParams p) {
   asm volatile("griddepcontrol.wait;" ::: "memory");  // chained to the step before it
   const int x = blockIdx.x;
@@ -717,7 +712,11 @@ int launch_collide32(float* buf, const StepParams& p, bool wide_fp64, cudaStream
 
 namespace {
 
-// Launch; dependent: as a programmatic dependent of the kernel before it in the stream.
+// Launch; dependent: as a programmatic dependent of the kernel before it in the
+// stream.  No pointer of a kernel launched here is const __restrict__: its grid
+// may be resident while the kernel before it writes what it reads, which the
+// read-only path does not allow; ordinary loads after griddepcontrol.wait see
+// those writes.
 template <class... A>
 int launch_pdl32(void (*kernel)(A...), dim3 grid, cudaStream_t stream, bool dependent, std::common_type_t<A>... args) {
   cudaLaunchConfig_t cfg = {};

@@ -57,3 +57,20 @@ def test_forms_agree_bit_for_bit(Lx, Ly, periodic_y, wild):
         lat.set_populations(f)
         lat.step(5)
         assert np.max(np.abs(lat.populations() - out[0])) <= 1e-15 * 5
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp32-df"])
+@pytest.mark.parametrize("Lx,Ly", [(3, 6), (5, 257), (38, 1024), (130, 257)])
+def test_long_chains_equal_the_serial_schedule(Lx, Ly, precision):
+    """Steps that start in the tail of the one before them, and a read-out behind
+    them, see everything those wrote: 203 steps, with single ones between."""
+    out = []
+    for kernel in ("fused", "fused_serial"):
+        lat = lbm.Lattice(Lx, Ly, kernel=kernel, precision=precision, device="cuda:0")
+        lat.init_rayleigh_taylor(7)
+        got = []
+        for n in (1, 1, 1, 100, 100):
+            lat.step(n)
+            got += list(lat.fields())
+        out.append(got + [lat.populations()])
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
