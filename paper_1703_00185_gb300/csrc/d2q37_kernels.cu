@@ -21,6 +21,7 @@
 // (the paper's 1-D blocks along y, Sec. "The propagate and bc Kernels").
 // Every warp reads 32 consecutive doubles of each population plane, so each
 // gather is a coalesced 256-byte row shifted by at most 3 elements.
+#include <atomic>
 #include <type_traits>
 
 #include <cuda_runtime.h>
@@ -1190,18 +1191,6 @@ dim3 site_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kBlockY - 1) / k
 
 dim3 stage_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kStageRows - 1) / kStageRows); }
 
-// SMs of the current device (looked up once; the library is for one kind of GPU).
-int sm_count() {
-  static const int n = [] {
-    int dev = 0, v = 0;
-    return cudaGetDevice(&dev) == cudaSuccess &&
-                   cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0
-               ? v
-               : 152;
-  }();
-  return n;
-}
-
 // (column, wall) groups of the wall-band kernel: 2 Lx, ten per warp
 int wall_grid(const StepParams& p) {
   constexpr int per_block = kWallGroupsPerWarp * (kWallBlock / 32);
@@ -1211,6 +1200,17 @@ int wall_grid(const StepParams& p) {
 int done(int n) { return cudaGetLastError() == cudaSuccess ? n : -1; }
 
 }  // namespace
+
+// SMs of the current device, looked up once per device.
+int sm_count() {
+  static std::atomic<int> known[256];
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return 152;
+  if ((v = known[dev].load(std::memory_order_relaxed)) > 0) return v;
+  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 152;
+  known[dev].store(v, std::memory_order_relaxed);
+  return v;
+}
 
 int launch_wrap(double* buf, const StepParams& p, cudaStream_t stream) {
   const long long n = (long long)kQ * 6 * (p.periodic_y ? p.Ly + 2 * kHx : p.Ly) +

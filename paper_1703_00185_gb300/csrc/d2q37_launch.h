@@ -12,6 +12,8 @@ namespace d2q37 {
 // Copy the quadrature constants to the current device's constant memory.
 cudaError_t upload_shell_consts(const ShellConsts& c);
 
+int sm_count();  // of the current device
+
 int launch_wrap(double* buf, const StepParams& p, cudaStream_t stream);
 int launch_propagate(const double* src, double* dst, const StepParams& p, cudaStream_t stream);
 int launch_bc(const double* src, double* dst, const StepParams& p, cudaStream_t stream);
