@@ -733,8 +733,18 @@ int launch_pdl32(void (*kernel)(A...), dim3 grid, cudaStream_t stream, bool depe
 
 }  // namespace
 
+// Chained (128 rows x 6 blocks per SM) unless the grid takes between 5/12 and 9/10
+// of the room: there the next step's blocks, waiting where this one leaves room,
+// pile up on some SMs and the step after runs unevenly.  Chained / not, us a step:
+// 110 x 512 periodic (0.48 of the room) double-float 5.2 / 5.7; 130 x 512 (0.57)
+// 7.3 / 6.0, FP64 wide terms 12.0 / 9.8; 190 x 512 (0.83) 7.5 / 6.9; 200 x 512
+// (0.88) 7.5 / 8.0; 285 x 512 (1.25) 10.0 / 10.2; 130 x 257 (0.43, a third of the
+// blocks nearly empty) 5.4 / 5.0.
 int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_fp64, cudaStream_t stream, bool chain) {
-  return launch_pdl32(wide_fp64 ? fused32_kernel<WideF64> : fused32_kernel<WideDF>, site_grid(p), stream, chain, src, dst,
+  const dim3 grid = site_grid(p);
+  const long long blocks = (long long)grid.x * grid.y, room = (long long)D2Q37_FP32_MIN_BLOCKS * sm_count();
+  chain = chain && (blocks * 12 <= room * 5 || blocks * 10 >= room * 9);
+  return launch_pdl32(wide_fp64 ? fused32_kernel<WideF64> : fused32_kernel<WideDF>, grid, stream, chain, src, dst,
                       p);
 }
 
