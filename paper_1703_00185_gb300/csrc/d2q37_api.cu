@@ -299,7 +299,7 @@ int k_fused(lbm_t* h, const void* s, void* d) {
   const bool serial = h->prm.kernel == LBM_KERNEL_FUSED_SERIAL, chain = !serial && !h->timing && !h->shares_device;
   return is_fp32(h->prec) ? launch_fused32((const float*)s, (float*)d, h->sp, h->prec == LBM_PRECISION_FP32_FP64,
                                            h->stream, chain)
-                          : launch_fused((const double*)s, (double*)d, h->sp, h->stream, !serial, chain);
+                          : launch_fused((const double*)s, (double*)d, h->sp, h->stream, !serial, chain, !h->shares_device);
 }
 
 int k_fields(lbm_t* h, const void* b, double* rho, double* u, double* T) {

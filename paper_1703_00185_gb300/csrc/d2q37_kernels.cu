@@ -130,15 +130,13 @@ __device__ __forceinline__ long long fixed_term(double v, unsigned top2, unsigne
   return r;
 }
 
-// The population of the largest magnitude (by its high word).
+// The largest magnitude of the populations' high words: its exponent field is
+// the largest exponent.
 template <class F>
-__device__ __forceinline__ double largest(const F& f) {
-  double m = 0.0;
+__device__ __forceinline__ int largest_high(const F& f) {
+  int m = 0;
 #pragma unroll
-  for (int l = 0; l < kQ; ++l) {
-    const double v = f.get(l);
-    if ((__double2hiint(v) & 0x7FFFFFFF) > (__double2hiint(m) & 0x7FFFFFFF)) m = v;
-  }
+  for (int l = 0; l < kQ; ++l) m = max(m, __double2hiint(f.get(l)) & 0x7FFFFFFF);
   return m;
 }
 
@@ -150,7 +148,7 @@ __device__ __forceinline__ double largest(const F& f) {
 template <bool ANY, class F>
 __device__ __forceinline__ bool site_sums(const F& f, long long& r, long long& jx, long long& jy,
                                           long long& e, int& emax) {
-  const int top = __double2hiint(ANY ? largest(f) : f.get(0));
+  const int top = ANY ? largest_high(f) : __double2hiint(f.get(0));
   emax = top >> 20 & 0x7FF;
   const unsigned top2 = 2u * (unsigned)(top | 0xFFFFF);
   unsigned wrap = 0;
@@ -559,12 +557,15 @@ __device__ __forceinline__ void collide_site_fp64(const F& f, const P& p, double
 // One site's collision: moments as exact integer sums, then the fixed-point
 // form inside its ranges, else the FP64 form; the relaxed populations to out.
 // The common path ends before the rest, which starts again from the
-// populations, so that it keeps nothing alive for it.
-template <class F, class P, class O>
+// populations, so that it keeps nothing alive for it.  SHORT = false leaves the
+// common path out: populations in registers stay alive for the rest, which 128
+// registers do not hold (364 bytes of spills; 142 x 512 periodic 17.5 us a step,
+// without 15.7).
+template <bool SHORT, class F, class P, class O>
 __device__ __forceinline__ void collide_site_to(const F& f, const P& p, const O& out) {
   long long r, jx, jy, e;
   int emax;
-  {
+  if constexpr (SHORT) {
     FxSite v;
     if (site_sums<false>(f, r, jx, jy, e, emax) && fx_site_from_sums(r, jx, jy, e, emax, p, v) &&
         collide_site_fx<false>(f, p, v, out))
@@ -599,7 +600,8 @@ __device__ __forceinline__ void collide_site_to(const F& f, const P& p, const O&
 // whether one thread sums the column (wall_density) or the three threads of a
 // column's wall rows each sum their own row and combine the sums by warp
 // shuffles (wall_band_kernel), so both give the same bits.
-template <class P>  // StepParams or BatchGeo (Ly, NY, Hy, plane)
+// L2: the loads bypass L1 (see launch_pdl).
+template <bool L2, class P>  // P: StepParams or BatchGeo (Ly, NY, Hy, plane)
 __device__ __forceinline__ double wall_row_outgoing(const double* src, const P& p, int x, int wall, int r) {
   const int y = wall ? p.Ly - 1 - r : r;
   const long long i = site_index(p, x, y);
@@ -607,15 +609,15 @@ __device__ __forceinline__ double wall_row_outgoing(const double* src, const P& 
 #pragma unroll
   for (int l = 0; l < kQ; ++l) {
     const int cy = vel_cy(l);
-    if (wall ? (cy > r) : (cy < -r)) s += __ldcg(src + (l * p.plane + i));
+    if (wall ? (cy > r) : (cy < -r)) s += L2 ? __ldcg(src + (l * p.plane + i)) : src[l * p.plane + i];
   }
   return s;
 }
 
 __device__ __forceinline__ double wall_density(const double* src, const StepParams& p, int x, int wall) {
-  const double s0 = wall_row_outgoing(src, p, x, wall, 0);
-  const double s1 = wall_row_outgoing(src, p, x, wall, 1);
-  const double s2 = wall_row_outgoing(src, p, x, wall, 2);
+  const double s0 = wall_row_outgoing<false>(src, p, x, wall, 0);
+  const double s1 = wall_row_outgoing<false>(src, p, x, wall, 1);
+  const double s2 = wall_row_outgoing<false>(src, p, x, wall, 2);
   return ((s0 + s1) + s2) * p.inv_denom[wall];
 }
 
@@ -705,7 +707,9 @@ __device__ __forceinline__ long long plane_offset(const P& p, int l) {
 // element of dst (written by this thread): read back and copied out.  OFF:
 // the planes addressed with the byte offsets of p (read from the constant
 // bank by the single-lattice kernels) instead of multiples of p.plane.
-template <bool OFF, class P>
+// PARTS: the populations copied in one go or in halves (where the kernel's 80 or
+// 96 registers hold no more; a round trip to L2 longer for the edge sites).
+template <bool OFF, int PARTS, class P>
 __device__ __forceinline__ void store_images(double* __restrict__ dst, const P& p, int x, int y) {
   if (x >= kHx && x < p.Lx - kHx && (!p.periodic_y || (y >= kHx && y < p.Ly - kHx))) return;
   const char* const s = (const char*)(dst + site_index(p, x, y));
@@ -718,12 +722,12 @@ __device__ __forceinline__ void store_images(double* __restrict__ dst, const P& 
     if (y >= p.Ly - kHx) ys[ny++] = y - p.Ly;
   }
 #pragma unroll
-  for (int part = 0; part < 2; ++part) {  // half of the populations at a time: 80 registers hold no more
-    constexpr int kHalf = (kQ + 1) / 2;
-    double f[kHalf];
+  for (int part = 0; part < PARTS; ++part) {
+    constexpr int kPart = (kQ + PARTS - 1) / PARTS;
+    double f[kPart];
 #pragma unroll
-    for (int k = 0; k < kHalf; ++k) {
-      const int l = part * kHalf + k;
+    for (int k = 0; k < kPart; ++k) {
+      const int l = part * kPart + k;
       if (l < kQ) f[k] = *(const double*)(s + (plane_offset<OFF>(p, l)));
     }
 #pragma unroll 1
@@ -732,8 +736,8 @@ __device__ __forceinline__ void store_images(double* __restrict__ dst, const P& 
       char* const d = (char*)(dst + site_index(p, a == 0 ? xs[0] : a == 1 ? xs[1] : xs[2],
                                                b == 0 ? ys[0] : b == 1 ? ys[1] : ys[2]));
 #pragma unroll
-      for (int k = 0; k < kHalf; ++k) {
-        const int l = part * kHalf + k;
+      for (int k = 0; k < kPart; ++k) {
+        const int l = part * kPart + k;
         if (l < kQ) *(double*)(d + (plane_offset<OFF>(p, l))) = f[k];
       }
     }
@@ -862,8 +866,8 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(doubl
   stage_init(stage, false, min(kStageRows, p.Ly - y0));
   const RowPopsOf<false> f = stage_rows<false>(stage, (const char*)(buf + i0), p, min(kStageRows, p.Ly - y0));
   if (f.a == 0 || y >= p.Ly) return;
-  collide_site_to(f, p, ToPlanes{(char*)(buf + i0) + threadIdx.x * 8u, p});
-  store_images<true>(buf, p, x, y);
+  collide_site_to<true>(f, p, ToPlanes{(char*)(buf + i0) + threadIdx.x * 8u, p});
+  store_images<true, 2>(buf, p, x, y);
 }
 
 // One site of the fused step: gather (pull), wall bc on the wall bands,
@@ -873,7 +877,7 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(doubl
 // single lattice.  OFF: addresses from the byte offsets of p (see store_images),
 // and loads of the source from L2 (see launch_pdl).
 // WALLS = false: the caller never passes a wall-band site.
-template <bool OFF, bool WALLS = true>
+template <bool OFF, bool WALLS = true, bool SHORT = false>
 __device__ __forceinline__ void fused_site(const double* src, double* dst, const StepParams& p, const StepParams& px,
                                            int x, int y) {
   const long long i = site_index(p, x, y);
@@ -892,10 +896,10 @@ __device__ __forceinline__ void fused_site(const double* src, double* dst, const
   }
   // each pair straight to the site's planes, then the halo images, if any
   if constexpr (OFF)
-    collide_site_to(RegPops{f}, px, ToPlanes{(char*)(dst + i), p});
+    collide_site_to<SHORT>(RegPops{f}, px, ToPlanes{(char*)(dst + i), p});
   else
-    collide_site_to(RegPops{f}, px, ToPlanesStride{dst + i, p.plane});
-  store_images<OFF>(dst, p, x, y);
+    collide_site_to<SHORT>(RegPops{f}, px, ToPlanesStride{dst + i, p.plane});
+  store_images<OFF, OFF ? 1 : 2>(dst, p, x, y);
 }
 
 __global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const double* src, double* dst,
@@ -917,30 +921,38 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) fused_kernel(const d
   const RowPops f = stage_rows<true>(stage, (const char*)(src + i0), p, min(kStageRows, p.Ly - y0));
   if (f.a == 0 || y >= p.Ly) return;
   if (!p.periodic_y && (y < 3 || y >= p.Ly - 3)) return;  // wall_band_kernel's
-  collide_site_to(f, p, ToPlanes{(char*)(dst + i0) + threadIdx.x * 8u, p});
-  store_images<true>(dst, p, x, y);
+  collide_site_to<true>(f, p, ToPlanes{(char*)(dst + i0) + threadIdx.x * 8u, p});
+  store_images<true, 2>(dst, p, x, y);
 }
 
-// The same for a lattice so small that all its warps are resident with every
-// register of an SM shared by 8 of them: the populations straight into
-// registers.  What counts there is the length of one site's chain, not room for
-// other warps.  Microseconds a step, before (2 blocks of 256 rows, 128
-// registers, no chaining) / now, blocks of 128 rows: 256 x 128 16.0 / 13.9, 130 x
-// 257 15.3 / 14.8, 64 x 64 15.5 / 14.2; 64 or 32 rows 15.0, 15.4 on the first.
-// Without walls (periodic y, edge rows with halo images in every column)
-// blocks of 32 rows: 130 x 257 13.2 / 11.0, 128 rows 16.2.
-constexpr int kFewWarps = 8;  // resident per SM at up to 255 registers
-
-template <int ROWS>
-__global__ void __launch_bounds__(ROWS, kFewWarps * 32 / ROWS) fused_few_kernel(const double* src, double* dst,
-                                                                               StepParams p) {
+// The same with the populations straight into registers, WARPS resident warps
+// per SM: for lattices of few sites, where the length of one site's chain counts
+// and not room for other warps, and for columns that fill tiles of 256 rows badly
+// (see SiteForm).
+template <int ROWS, int WARPS>
+__global__ void __launch_bounds__(ROWS, WARPS * 32 / ROWS) fused_reg_kernel(const double* src, double* dst,
+                                                                            StepParams p) {
   const int x = blockIdx.x;
   const int y = blockIdx.y * ROWS + threadIdx.x;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // as fused_kernel
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (y >= p.Ly) return;
   if (!p.periodic_y && (y < 3 || y >= p.Ly - 3)) return;  // wall_band_kernel's
-  fused_site<true, false>(src, dst, p, p, x, y);
+  fused_site<true, false, WARPS == 8>(src, dst, p, p, x, y);
+}
+
+template <int ROWS>
+__global__ void __launch_bounds__(ROWS, 16 * 32 / ROWS) collide_reg_kernel(double* buf, StepParams p) {
+  const int x = blockIdx.x;
+  const int y = blockIdx.y * ROWS + threadIdx.x;
+  if (y >= p.Ly) return;
+  char* const b = (char*)(buf + site_index(p, x, y));
+  double f[kQ];
+#pragma unroll
+  for (int l = 0; l < kQ; ++l) f[l] = *(const double*)(b + p.plane_off[l]);
+  // in place: every population is read above before its pair is written back
+  collide_site_to<false>(RegPops{f}, p, ToPlanes{b, p});
+  store_images<true, 1>(buf, p, x, y);
 }
 
 // The fused step of the six wall-band rows of every column (y = 0..2 and
@@ -971,7 +983,7 @@ __global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* src
   const int r = lane - 3 * (lane / 3);  // row from the wall
   const bool active = lane < 3 * kWallGroupsPerWarp && g < 2 * p.Lx;
   const int x = g >> 1, wall = g & 1;
-  const double s = active ? wall_row_outgoing(src, p, x, wall, r) : 0.0;
+  const double s = active ? wall_row_outgoing<true>(src, p, x, wall, r) : 0.0;
   const int base = lane - r;  // the group's row-0 lane (idle lanes read lanes 30, 31, 32 mod 32)
   const double s0 = __shfl_sync(0xffffffffu, s, base);
   const double s1 = __shfl_sync(0xffffffffu, s, base + 1);
@@ -984,8 +996,8 @@ __global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* src
 #pragma unroll
     for (int l = 0; l < kQ; ++l) f[l] = __ldcg((const double*)(sp + p.pull_off[l]));
     apply_wall(f, p.fw[wall], wall, r, ((s0 + s1) + s2) * p.inv_denom[wall]);
-    collide_site_to(RegPops{f}, p, ToPlanes{(char*)(dst + i), p});
-    store_images<true>(dst, p, x, y);
+    collide_site_to<true>(RegPops{f}, p, ToPlanes{(char*)(dst + i), p});
+    store_images<true, 1>(dst, p, x, y);
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -1063,10 +1075,10 @@ __global__ void __launch_bounds__(ROWS, BLOCKS)
       if (!g.periodic_y && (y < 3 || y >= g.Ly - 3)) return;  // the wall tiles'
       const ToPlanesStride out{dst + at + threadIdx.x, g.plane};
       if constexpr (UNIFORM)
-        collide_site_to(f, L.common, out);
+        collide_site_to<true>(f, L.common, out);
       else
-        collide_site_to(f, own, out);
-      store_images<false>(dst, g, x, y);
+        collide_site_to<true>(f, own, out);
+      store_images<false, 2>(dst, g, x, y);
     } else {
       if (!UNIFORM) __syncthreads();
       if (y >= g.Ly) return;
@@ -1080,10 +1092,10 @@ __global__ void __launch_bounds__(ROWS, BLOCKS)
       for (int l = 0; l < kQ; ++l) f[l] = src[l * g.plane + at - vel_cx(l) * g.NY - vel_cy(l)];
       const ToPlanesStride out{dst + at, g.plane};
       if constexpr (UNIFORM)
-        collide_site_to(RegPops{f}, L.common, out);
+        collide_site_to<false>(RegPops{f}, L.common, out);
       else
-        collide_site_to(RegPops{f}, own, out);
-      store_images<false>(dst, g, x, y);
+        collide_site_to<false>(RegPops{f}, own, out);
+      store_images<false, 1>(dst, g, x, y);
     }
     return;
   }
@@ -1105,7 +1117,7 @@ __global__ void __launch_bounds__(ROWS, BLOCKS)
   const int x = grp >> 1, wall = grp & 1;
   const int c = g.cur ^ parity;
   const double* src = (const double*)g.buf[c];
-  const double sum = active ? wall_row_outgoing(src, g, x, wall, r) : 0.0;
+  const double sum = active ? wall_row_outgoing<false>(src, g, x, wall, r) : 0.0;
   const int base = lane - r;
   const double s0 = __shfl_sync(0xffffffffu, sum, base);
   const double s1 = __shfl_sync(0xffffffffu, sum, base + 1);
@@ -1121,10 +1133,10 @@ __global__ void __launch_bounds__(ROWS, BLOCKS)
   double* dst = (double*)g.buf[c ^ 1];
   const ToPlanesStride out{dst + at, g.plane};
   if constexpr (UNIFORM)
-    collide_site_to(RegPops{f}, L.common, out);
+    collide_site_to<false>(RegPops{f}, L.common, out);
   else
-    collide_site_to(RegPops{f}, p, out);
-  store_images<false>(dst, g, x, y);
+    collide_site_to<false>(RegPops{f}, p, out);
+  store_images<false, 2>(dst, g, x, y);
 }
 
 __global__ void __launch_bounds__(kBlockY) fields_kernel(const double* buf, double* rho, double* u, double* T,
@@ -1189,8 +1201,6 @@ __global__ void __launch_bounds__(kBlockY) init_rayleigh_taylor_kernel(T* __rest
 
 dim3 site_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kBlockY - 1) / kBlockY); }
 
-dim3 stage_grid(const StepParams& p) { return dim3(p.Lx, (p.Ly + kStageRows - 1) / kStageRows); }
-
 // (column, wall) groups of the wall-band kernel: 2 Lx, ten per warp
 int wall_grid(const StepParams& p) {
   constexpr int per_block = kWallGroupsPerWarp * (kWallBlock / 32);
@@ -1231,11 +1241,6 @@ int launch_bc(const double* src, double* dst, const StepParams& p, cudaStream_t 
   return done(1);
 }
 
-int launch_collide(double* buf, const StepParams& p, cudaStream_t stream) {
-  collide_kernel<<<stage_grid(p), kStageRows, kStageBytes, stream>>>(buf, p);
-  return done(1);
-}
-
 // Launch; dependent: as a programmatic dependent of the kernel before it in the
 // stream.  Such a grid may be resident while earlier kernels still write what it
 // reads: after its griddepcontrol.wait those writes are visible to its ordinary
@@ -1261,17 +1266,110 @@ bool launch_pdl(void (*kernel)(A...), dim3 grid, int block, int smem, cudaStream
   return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess;
 }
 
-int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap, bool chain) {
-  // few sites, and no other stream's grids to share the SMs with (those gain
-  // from the warps that the staged form leaves room for)
-  const bool few = chain && (long long)p.Lx * ((p.Ly + 31) / 32) <= (long long)kFewWarps * sm_count();
+// The form of a sites kernel: rows per block and warps per SM of a register form
+// (255 registers with 8 warps, 128 with 16), or the staged one (rows = 0).
+// Microseconds a step, "w" = warps of 32 rows per SM, 512 rows unless stated:
+//                          staged  255 regs  128 regs   before the staged form
+//  walls    38 x 512   4 w   13.7      12.9      13.4
+//           76 x 512   8 w   17.0      21.7      15.9
+//          142 x 512  15 w   22.2      22.6      18.0    19.2
+//          185 x 512  19 w   23.9      30.7      25.0
+//          570 x 512  60 w   64.1      87.3      65.5    68.8
+//  periodic 64 x 64          9.5       8.4       8.5     9.0
+//          142 x 512  15 w   22.3      19.4      15.7    17.0
+//          285 x 512  30 w   30.2      37.3      28.4    30.6
+//          570 x 512  60 w   58.3      77.9      60.0    60.1
+//         1140 x 512 120 w  101.5     143.1     109.8   106.5
+struct SiteForm {
+  int rows, warps;
+};
+constexpr SiteForm kStaged = {0, 0};
+
+// 128 registers: blocks of 32 rows leave the fewest threads idle (512 x 257
+// periodic 28.3 us, of 128 rows 32.9).  Blocks of 128 have fewer warps with edge
+// rows and are fewer to start: 64 x 64 periodic 8.5 / 8.9 us, 60 lattices of 120 x
+// 240 on four streams 347 / 369.
+SiteForm reg_form(int rows) {
+  const bool one = rows > 32 && rows <= 128, full = rows * 10LL >= 9 * 128LL * ((rows + 127) / 128);
+  return {one || full ? 128 : 32, 16};
+}
+
+// Whether a register form's blocks over Lx columns of `rows` rows and `walls`
+// blocks of the wall-band kernel (246 registers) are all resident at once.
+bool form_resident(SiteForm f, int Lx, int rows, int walls) {
+  const long long warps = (long long)Lx * ((rows + f.rows - 1) / f.rows) * (f.rows / 32);
+  return warps + walls * (kWallBlock / 32) * (f.warps / 8) <= (long long)f.warps * sm_count();
+}
+
+// Whether the staged tiles hold so few rows that 128 registers win at any size
+// (their idle warps keep a third of the SM's warps from running): below 0.8 of
+// 256 rows a tile, below a half where the staged tiles are one wave.  Staged / 128
+// registers: 1500 x 300 (0.59) periodic 117 / 94 us, 1000 x 384 (0.75) 81.5 / 78,
+// 1000 x 450 (0.88) 93.3 / 93.8, 400 x 1200 (0.94) 88 / 94; walls 1500 x 300 113 /
+// 98, 600 x 800 (0.78) 101 / 98, 800 x 640 (0.83) 102 / 103; 256 x 196 (0.75,
+// one wave) 17.4 / 21.9.
+bool poor_fill(int Lx, int rows) {
+  const int tiles = (rows + kStageRows - 1) / kStageRows;
+  const bool one_wave = (long long)Lx * tiles <= (long long)kStageBlocks * sm_count();
+  return rows * 10LL < (one_wave ? 5LL : 8LL) * kStageRows * tiles;
+}
+
+// Up to this many warps of rows per SM 128 registers win without walls, where no
+// second kernel waits for room.
+constexpr int kRegWarps = 40;
+bool few_warps(int Lx, int rows) { return (long long)Lx * ((rows + 31) / 32) <= (long long)kRegWarps * sm_count(); }
+
+// alone: no other stream's grids beside this one.  Beside others, walled lattices
+// that do not fill the GPU many times over keep the staged form, which leaves room (a server's burst of 12 jobs 17.5 ms,
+// 19.3 with tiles filled badly in 128 registers; 16 jobs of 200 to 500 columns
+// 54.7, 59.6), and no lattice takes 255 registers.  A walled step that is not
+// chained keeps the staged form too, for the wall-band kernel's room.
+SiteForm fused_form(const StepParams& p, int rows, int walls, bool chain, bool alone) {
+  if (p.periodic_y ? alone : chain)
+    for (const SiteForm f : {SiteForm{rows > 32 ? 128 : 32, 8}, SiteForm{32, 8}})
+      if (form_resident(f, p.Lx, rows, walls)) return f;
+  if (!alone && !p.periodic_y && few_warps(p.Lx, rows)) return kStaged;
+  const SiteForm reg = reg_form(rows);
+  if (poor_fill(p.Lx, rows)) return reg;
+  if (p.periodic_y ? few_warps(p.Lx, rows) : chain && form_resident(reg, p.Lx, rows, walls)) return reg;
+  return kStaged;
+}
+
+int launch_collide(double* buf, const StepParams& p, cudaStream_t stream) {
+  const SiteForm form = poor_fill(p.Lx, p.Ly) || few_warps(p.Lx, p.Ly) ? reg_form(p.Ly) : kStaged;
+  void (*const kernel)(double*, StepParams) =
+      !form.rows ? collide_kernel : form.rows == 128 ? collide_reg_kernel<128> : collide_reg_kernel<32>;
+  const int rows = form.rows ? form.rows : kStageRows;
+  kernel<<<dim3(p.Lx, (p.Ly + rows - 1) / rows), rows, form.rows ? 0 : kStageBytes, stream>>>(buf, p);
+  return done(1);
+}
+
+int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap, bool chain,
+                 bool alone) {
+  // the last three rows of a walled lattice are the wall-band kernel's
+  const int Ly = p.periodic_y ? p.Ly : p.Ly - 3, walls = p.periodic_y ? 0 : wall_grid(p);
+  const SiteForm form = fused_form(p, Ly, walls, chain, alone);
   void (*const sites)(const double*, double*, StepParams) =
-      !few ? fused_kernel : p.periodic_y ? fused_few_kernel<32> : fused_few_kernel<128>;
-  const int rows = !few ? kStageRows : p.periodic_y ? 32 : 128, smem = few ? 0 : kStageBytes;
-  const dim3 grid(p.Lx, (p.Ly + rows - 1) / rows);
-  if (!launch_pdl(sites, grid, rows, smem, stream, chain, src, dst, p)) return -1;
+      !form.rows         ? fused_kernel
+      : form.warps == 8  ? (form.rows == 128 ? fused_reg_kernel<128, 8> : fused_reg_kernel<32, 8>)
+      : form.rows == 128 ? fused_reg_kernel<128, 16>
+                         : fused_reg_kernel<32, 16>;
+  const int rows = form.rows ? form.rows : kStageRows;
+  const dim3 grid(p.Lx, (Ly + rows - 1) / rows);
+  // The next step's blocks wait where this one's leave room.  With 255 registers
+  // that hides the launch.  Between half and all of the room they pile up on some
+  // SMs, and the step after runs unevenly (100 x 512 periodic 15.5 us, not chained
+  // 13.4); with walls and more than one wave they keep the wall-band kernel
+  // from its room (570 x 512 67.4 us, 64.1; 185 x 512, one wave, 23.9, 26.5).
+  const long long used = (long long)grid.x * grid.y * (rows / 32);
+  const long long room = (long long)(form.rows ? form.warps : kStageBlocks * kStageRows / 32) * sm_count();
+  if (form.warps != 8)
+    chain = chain && (p.periodic_y ? used * 12 <= room * 5 || used * 10 >= room * 9
+                      : form.rows  ? form_resident(form, p.Lx, Ly, walls)
+                                   : used * 10 <= room * 9);
+  if (!launch_pdl(sites, grid, rows, form.rows ? 0 : kStageBytes, stream, chain, src, dst, p)) return -1;
   if (p.periodic_y) return done(1);
-  if (!launch_pdl(wall_band_kernel, dim3(wall_grid(p)), kWallBlock, 0, stream, overlap, src, dst, p)) return -1;
+  if (!launch_pdl(wall_band_kernel, dim3(walls), kWallBlock, 0, stream, overlap, src, dst, p)) return -1;
   return done(2);
 }
 

@@ -22,8 +22,9 @@ int launch_collide(double* buf, const StepParams& p, cudaStream_t stream);
 // dependent of the sites kernel and starts in its tail; false: after it.
 // chain: the first kernel is launched as a programmatic dependent of whatever
 // kernel precedes it in the stream (it waits for it before its first access).
+// alone: no other stream's grids are expected beside it.
 int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap = true,
-                 bool chain = false);
+                 bool chain = false, bool alone = false);
 int launch_fields(const double* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream,
                   bool chain = false);
 // Rayleigh-Taylor initial state, FP64 or FP32 deviations; yi: device, the

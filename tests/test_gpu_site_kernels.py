@@ -74,3 +74,33 @@ def test_long_chains_equal_the_serial_schedule(Lx, Ly, precision):
             got += list(lat.fields())
         out.append(got + [lat.populations()])
     assert all(np.array_equal(a, b) for a, b in zip(*out))
+
+
+# (Lx, Ly) on both sides of every rule that picks a form, and blocks whose last one is nearly empty
+FORMS = [(3, 9), (64, 64), (227, 34), (1000, 16), (2000, 35), (76, 512), (100, 512), (142, 515), (152, 515),
+         (130, 257), (130, 260), (256, 196), (400, 100), (500, 516), (470, 262), (460, 191), (40, 1030)]
+
+
+@pytest.mark.parametrize("Lx,Ly", FORMS)
+@pytest.mark.parametrize("periodic_y", [False, True])
+def test_every_form_gives_the_same_bits(Lx, Ly, periodic_y):
+    """One lattice chained, serial, in a batch of one launch per lattice and with
+    separate kernels, each in the form its rule picks, against the batch's table
+    kernel (one register form for every size)."""
+    f = initial(Lx, Ly, False)
+    out = []
+    for kernel, config in (("fused", (128, 1)), ("fused", (0, 0)), ("fused", None), ("fused_serial", None),
+                           ("separate", None)):
+        lat = lbm.Lattice(Lx, Ly, tau=0.9, g0=1e-3, periodic_y=periodic_y, kernel=kernel, device="cuda:0")
+        lat.set_populations(f)
+        if config:
+            b = lbm.Batch([lat])
+            b.set_config(*config)
+            b.step(5)
+            b.synchronize()
+            b.close()
+        else:
+            lat.step(5)
+        out.append(lat.populations())
+    for got in out[1:]:
+        assert np.array_equal(got, out[0])
