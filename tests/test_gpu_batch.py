@@ -63,9 +63,10 @@ def test_batch_equals_alone(precision, config, shared_tau):
 
 @pytest.mark.parametrize("block_y", [64, 128, 256])
 def test_split_single_launch_equals_alone(block_y):
-    """FP64 lattices with walls and one tau and g: one block per tile runs the
-    split form (site tiles and wall tiles in one launch), one kernel per step,
-    and each lattice's result is bit-identical to the lattice stepped alone."""
+    """FP64 lattices with walls and one tau and g: one block per tile, site tiles
+    and wall tiles in one launch, one kernel per step, and each lattice's result
+    is bit-identical to the lattice stepped alone.  (Of a batch this small the
+    populations are kept in registers; test_gpu_batch_tiles.py has a large one.)"""
     alone = make("fp64", periodic_last=False, shared_tau=True)
     batched = make("fp64", periodic_last=False, shared_tau=True)
     for lat in alone:
