@@ -765,6 +765,7 @@ constexpr int kStageBlocks = 3;
 __host__ __device__ constexpr int slot_bytes(int rows) { return (rows + 2) * 8; }
 __host__ __device__ constexpr int stage_bytes(int rows) { return kQ * slot_bytes(rows) + 16; }  // and the barrier
 constexpr int kStageBytes = stage_bytes(kStageRows);
+constexpr int kSharedPerSm = 228 * 1024, kSystemShared = 1024;  // the latter taken from it for every block
 constexpr int kWaitLimit = 1 << 20;           // polls of the barrier, each of some microseconds at most
 
 __host__ __device__ constexpr int odd_hops() {
@@ -1039,15 +1040,19 @@ __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? 
 // a per-tile table or, without one, from a search over the launch's lattices.
 // The per-site arithmetic is the single-lattice kernels', so results are the
 // same bit for bit.  64 uneven lattices (42.3 M sites), milliseconds a step:
-// 7.36 with the populations in registers, 6.70 now (256 rows, 3 blocks per SM);
-// 100 lattices of 60-400 columns, each with its own tau and g: 1.86 as a table
-// walked by grid-stride blocks, 1.33 now (128 rows, 5 blocks per SM).
+// 7.36 with the populations in registers, 6.62 staged (256 rows, 3 blocks per
+// SM); 100 lattices of 60-400 columns, each with its own tau and g: 1.86 as a
+// table walked by grid-stride blocks, 1.33 staged (128 rows, 5 blocks per SM).
+// Tiles of 256 rows with their own constants are never staged (own_staged).
 static_assert(sizeof(BatchLaunch) <= 32700, "BatchLaunch must fit the kernel parameter space");
 
 template <int ROWS, int BLOCKS, bool UNIFORM, bool STAGED>
 __global__ void __launch_bounds__(ROWS, BLOCKS)
     batch_tile_kernel(const __grid_constant__ BatchLaunch L, const BatchEntry* __restrict__ tab,
                       const int* __restrict__ tile_entry, int parity) {
+  static_assert(!STAGED || BLOCKS * (stage_bytes(ROWS) + (UNIFORM ? 0 : (int)sizeof(Collision)) + kSystemShared) <=
+                               kSharedPerSm,
+                "blocks per SM that do not fit its shared memory");
   extern __shared__ __align__(128) unsigned char stage[];
   __shared__ Collision own;
   static_assert(sizeof(Collision) % 8 == 0, "Collision is copied in 8-byte words");
@@ -1402,13 +1407,22 @@ int launch_batch_fused(const BatchEntry* tab, const int* tile_entry, int n, long
 
 namespace {
 
+// Whether BLOCKS staged blocks and their copies of the collision constants fit an
+// SM.  Three of 256 rows do not (352 bytes short); two of them took the same 80
+// registers: 24 lattices of 1024 x 1024 4.69 ms a step, in registers 4.53.
+constexpr bool own_staged(int rows, int blocks) {
+  return blocks * (stage_bytes(rows) + (int)sizeof(Collision) + kSystemShared) <= kSharedPerSm;
+}
+
 template <int ROWS, int BLOCKS>
 cudaError_t allow_tile_memory() {
-  const cudaError_t e = cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, true, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS));
-  return e == cudaSuccess ? cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, false, true>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS))
-                          : e;
+  cudaError_t e = cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, true, true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS));
+  if constexpr (own_staged(ROWS, BLOCKS))
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(batch_tile_kernel<ROWS, BLOCKS, false, true>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, stage_bytes(ROWS));
+  return e;
 }
 
 // Up to this many warps of sites per SM (some waves) the register form (128
@@ -1424,11 +1438,13 @@ int tile_launch(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const
                 cudaStream_t stream) {
   constexpr int kRegBlocks = 4 * 128 / ROWS;
   const int grid = L.site_tiles + L.wall_tiles;
-  const bool staged = L.site_warps > (long long)kBatchFewWarps * sm_count();
-  void (*const kernel)(BatchLaunch, const BatchEntry*, const int*, int) =
-      staged ? (uniform ? batch_tile_kernel<ROWS, BLOCKS, true, true> : batch_tile_kernel<ROWS, BLOCKS, false, true>)
-             : (uniform ? batch_tile_kernel<ROWS, kRegBlocks, true, false>
-                        : batch_tile_kernel<ROWS, kRegBlocks, false, false>);
+  const bool staged =
+      (uniform || own_staged(ROWS, BLOCKS)) && L.site_warps > (long long)kBatchFewWarps * sm_count();
+  void (*kernel)(BatchLaunch, const BatchEntry*, const int*, int) =
+      uniform ? batch_tile_kernel<ROWS, kRegBlocks, true, false> : batch_tile_kernel<ROWS, kRegBlocks, false, false>;
+  if (staged && uniform) kernel = batch_tile_kernel<ROWS, BLOCKS, true, true>;
+  if constexpr (own_staged(ROWS, BLOCKS))
+    if (staged && !uniform) kernel = batch_tile_kernel<ROWS, BLOCKS, false, true>;
   kernel<<<grid, ROWS, staged ? stage_bytes(ROWS) : 0, stream>>>(L, tab, tile_entry, parity);
   return done(1);
 }
