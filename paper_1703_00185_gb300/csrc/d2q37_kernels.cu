@@ -879,8 +879,8 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(doubl
 // and loads of the source from L2 (see launch_pdl).
 // WALLS = false: the caller never passes a wall-band site.
 template <bool OFF, bool WALLS = true, bool SHORT = false>
-__device__ __forceinline__ void fused_site(const double* src, double* dst, const StepParams& p, const StepParams& px,
-                                           int x, int y) {
+__device__ __forceinline__ void fused_site(const double* src, double* __restrict__ dst, const StepParams& p,
+                                           const StepParams& px, int x, int y) {
   const long long i = site_index(p, x, y);
   double f[kQ];
   if constexpr (OFF) {

@@ -393,7 +393,7 @@ __device__ __forceinline__ void fields_of_site32(const float (&d)[kQ], double& r
 
 // Halo images as in the FP64 store_site.
 template <class P>
-__device__ __forceinline__ void store_site32(float* dst, const P& p, int x, int y, const float (&d)[kQ]) {
+__device__ __forceinline__ void store_site32(float* __restrict__ dst, const P& p, int x, int y, const float (&d)[kQ]) {
   if (x >= kHx && x < p.Lx - kHx && (!p.periodic_y || (y >= kHx && y < p.Ly - kHx))) {
     float* q = dst + (int)site_index(p, x, y);  // no halo image: the common case
 #pragma unroll
@@ -482,8 +482,9 @@ __global__ void __launch_bounds__(256) wrap32_kernel(float* __restrict__ buf, St
 
 // One site of the fused step (pull, wall bc on the wall bands, collide,
 // store with halo images).
+// dst aliases nothing: p may be in shared memory, read again after every store otherwise.
 template <class W, class P>
-__device__ __forceinline__ void fused_site32(const float* src, float* dst, const P& p, int x, int y) {
+__device__ __forceinline__ void fused_site32(const float* src, float* __restrict__ dst, const P& p, int x, int y) {
   // the site's pointer once per thread; each population at an offset that is
   // the same for the whole block (l plane - cx NY - cy)
   const float* q = src + (int)site_index(p, x, y);
