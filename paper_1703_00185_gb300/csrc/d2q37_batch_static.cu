@@ -86,11 +86,18 @@ int lbm_batch_step_static(int n, lbm_t* const* lattices, int steps, void* cuda_s
   if (rc) return rc;
   // the whole table [0, n) is rewritten every call; entries past n are never read
   int cur[LBM_STATIC_BATCH_MAX];
+  long long tile0 = 0, warps = 0;  // tiles and warps of 32 rows so far
   for (int i = 0; i < n; ++i) {
     BatchEntry& e = g_static_host[i];
     std::memset(&e, 0, sizeof(e));
     e.p = lattices[i]->sp;
-    cur[i] = lattices[i]->cur;
+    e.buf[0] = lattices[i]->buf[0];
+    e.buf[1] = lattices[i]->buf[1];
+    e.cur = cur[i] = lattices[i]->cur;
+    e.ytiles = (lattices[i]->Ly + 127) / 128;
+    e.tile0 = tile0;
+    tile0 += (long long)lattices[i]->Lx * e.ytiles;
+    warps += (long long)lattices[i]->Lx * ((lattices[i]->Ly + 31) / 32);
   }
   // the launches' own parameters: geometry and collision constants
   static_assert(LBM_STATIC_BATCH_MAX <= kBatchGeoMax && LBM_STATIC_BATCH_MAX <= kBatchGeo32Max, "one launch holds every lattice");
@@ -101,6 +108,13 @@ int lbm_batch_step_static(int n, lbm_t* const* lattices, int steps, void* cuda_s
   const long long tiles = prec == LBM_PRECISION_FP64 ? fill_batch_launch(launch64, n, lattices, cur, 128, &uniform)
                                                      : fill_batch_launch32(launch32, n, lattices, cur, 128);
   if (tiles < 0) return LBM_ETOOBIG;
+  // FP32 steps of few sites go through the table: a launch with 32 KB of parameters
+  // takes the host 1.7 us longer, which shows where each call is followed by host
+  // work for every lattice.  16 steps and a read-out of 10 lattices of 12 to 100
+  // columns (8 warps of sites per SM) 327 us with tiles, 283 through the table; 40
+  // (28) 815, 764; 10 of 12 to 200 (21) 325, 328.  (launch_batch_tiles has a
+  // rule of its own for FP64.)
+  const bool table32 = warps <= 30LL * sm_count();
   // pageable source: the runtime stages it before the call returns (so the
   // next call may rewrite it), which waits for the stream's earlier work
   if (cudaMemcpyAsync(dev_tab, g_static_host, n * sizeof(BatchEntry), cudaMemcpyHostToDevice, stream) !=
@@ -109,6 +123,9 @@ int lbm_batch_step_static(int n, lbm_t* const* lattices, int steps, void* cuda_s
   for (int t = 0; t < steps; ++t) {
     const int launched = prec == LBM_PRECISION_FP64
                              ? launch_batch_tiles(launch64, uniform, dev_tab, nullptr, t & 1, 128, stream)
+                         : table32
+                             ? launch_batch_fused32(dev_tab, nullptr, n, tiles, t & 1, 128, (int)tiles,
+                                                    prec == LBM_PRECISION_FP32_FP64, stream)
                              : launch_batch_tiles32(launch32, dev_tab, nullptr, (int)tiles, t & 1, 128,
                                                     prec == LBM_PRECISION_FP32_FP64, stream);
     if (launched < 0) return LBM_ECUDA;

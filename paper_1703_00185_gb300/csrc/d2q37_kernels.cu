@@ -880,7 +880,7 @@ __global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(doubl
 // WALLS = false: the caller never passes a wall-band site.
 template <bool OFF, bool WALLS = true, bool SHORT = false>
 __device__ __forceinline__ void fused_site(const double* src, double* __restrict__ dst, const StepParams& p,
-                                           const StepParams& px, int x, int y) {
+                                           const Collision& px, int x, int y) {
   const long long i = site_index(p, x, y);
   double f[kQ];
   if constexpr (OFF) {
@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(kWallBlock) wall_band_kernel(const double* src
 template <int BY, bool UNIFORM>
 __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? (D2Q37_BATCH_MIN_BLOCKS * 128) / BY : 1)
     batch_fused_kernel(const BatchEntry* __restrict__ tab, const int* __restrict__ tile_entry, int n, long long tiles,
-                       int parity, StepParams common) {
+                       int parity, Collision common) {
   for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
     // owning lattice: per-tile table when given, else binary search; its
     // parameters are read in place (read-only, cached)
@@ -1023,7 +1023,8 @@ __global__ void __launch_bounds__(BY, (D2Q37_BATCH_MIN_BLOCKS * 128) / BY > 0 ? 
     const int y = (local - x * e.ytiles) * BY + threadIdx.x;
     const int c = e.cur ^ parity;
     if (y < e.p.Ly)
-      fused_site<false>((const double*)e.buf[c], (double*)e.buf[c ^ 1], e.p, UNIFORM ? common : e.p, x, y);
+      fused_site<false>((const double*)e.buf[c], (double*)e.buf[c ^ 1], e.p,
+                        UNIFORM ? common : static_cast<const Collision&>(e.p), x, y);
   }
 }
 
@@ -1380,11 +1381,11 @@ int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream
 
 template <int BY>
 int batch_launch(const BatchEntry* tab, const int* tile_entry, int n, long long tiles, int parity, int grid,
-                 const StepParams* common, cudaStream_t stream) {
+                 const Collision* common, cudaStream_t stream) {
   if (common)
     batch_fused_kernel<BY, true><<<grid, BY, 0, stream>>>(tab, tile_entry, n, tiles, parity, *common);
   else
-    batch_fused_kernel<BY, false><<<grid, BY, 0, stream>>>(tab, tile_entry, n, tiles, parity, StepParams{});
+    batch_fused_kernel<BY, false><<<grid, BY, 0, stream>>>(tab, tile_entry, n, tiles, parity, Collision{});
   return done(1);
 }
 
@@ -1396,7 +1397,7 @@ int batch_occupancy() {
 }
 
 int launch_batch_fused(const BatchEntry* tab, const int* tile_entry, int n, long long tiles, int parity,
-                       int block_y, int grid, const StepParams* common, cudaStream_t stream) {
+                       int block_y, int grid, const Collision* common, cudaStream_t stream) {
   switch (block_y) {
     case 64: return batch_launch<64>(tab, tile_entry, n, tiles, parity, grid, common, stream);
     case 128: return batch_launch<128>(tab, tile_entry, n, tiles, parity, grid, common, stream);
@@ -1428,10 +1429,11 @@ cudaError_t allow_tile_memory() {
 // Up to this many warps of sites per SM (some waves) the register form (128
 // registers, 16 warps per SM) is the faster one: a wave is one site's chain
 // long, and the bulk copies add theirs.  Microseconds a step in registers /
-// staged, 128 rows: 3 lattices of up to 40 x 80 17.6 / 21.7, 10 of 60 x 120 18.6
-// / 23.0, 10 of 200 x 400 (30 warps per SM) 51 / 59, 60 of 120 x 240 (100)
-// 159 / 162; 64 of up to 1024 x 2048 (8700) 7360 / 6700.
-constexpr int kBatchFewWarps = 200;
+// staged, 128 rows, walls: shared tau and g 3 lattices of 40 x 80 (2 warps) 17.0 /
+// 21.1, 10 of 120 x 240 (63) 81.7 / 83.4, 14 (88) 105.5 / 104.7, 20 (126) 139 /
+// 137, 40 of 100 x 97 (105) 121 / 126, 60 of 120 x 240 (379) 372 / 359, 24 of 1024 x 1024 (5174) 4449 / 4084; their own 10 (63)
+// 85 / 93, 20 (126) 145 / 151, 30 (189) 207 / 210, 60 (379) 394 / 384.
+constexpr int kBatchFewWarps = 120, kBatchFewWarpsOwn = 250;
 
 template <int ROWS, int BLOCKS>
 int tile_launch(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const int* tile_entry, int parity,
@@ -1439,7 +1441,8 @@ int tile_launch(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const
   constexpr int kRegBlocks = 4 * 128 / ROWS;
   const int grid = L.site_tiles + L.wall_tiles;
   const bool staged =
-      (uniform || own_staged(ROWS, BLOCKS)) && L.site_warps > (long long)kBatchFewWarps * sm_count();
+      (uniform || own_staged(ROWS, BLOCKS)) &&
+      L.site_warps > (long long)(uniform ? kBatchFewWarps : kBatchFewWarpsOwn) * sm_count();
   void (*kernel)(BatchLaunch, const BatchEntry*, const int*, int) =
       uniform ? batch_tile_kernel<ROWS, kRegBlocks, true, false> : batch_tile_kernel<ROWS, kRegBlocks, false, false>;
   if (staged && uniform) kernel = batch_tile_kernel<ROWS, BLOCKS, true, true>;
@@ -1449,10 +1452,32 @@ int tile_launch(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const
   return done(1);
 }
 
+// With walls and up to 8 warps of sites per SM the table kernel is faster: its wall
+// rows are a few lanes' longer chain in a block of sites, where a wall tile's
+// chain waits for its row sums first.  So it is where the wall tiles alone would
+// start a second or third wave.  Microseconds a step, tiles / table, 128 rows: 2
+// lattices of 16 x 40 18.0 / 13.6, 6 of 40 x 80 (5 warps) 18.0 / 14.8, 5 of 60 x 120
+// (8) 20.9 / 16.6, 6 (9.5) 21.0 / 18.9, 8 (13) 23.6 / 24.0, 3 of 120 x 240 (19) 31.2 /
+// 35.9, 5 (32, two waves and the wall tiles) 50.2 / 44.2; with their own tau and g
+// 18.9 / 14.8, 18.7 / 15.5, 22.9 / 16.7, 22.0 / 18.8, 24.0 / 23.3, 32.1 / 36.3, 53.1 /
+// 46.3 (64 rows 51.7 / 53.1).  Without walls tiles win: 10.7 / 11.5 on the first.
+constexpr int kBatchTableWarps = 8;
+
+bool table_is_faster(const BatchLaunch& L, int block_y) {
+  if (!L.wall_tiles) return false;
+  if (L.site_warps <= (long long)kBatchTableWarps * sm_count()) return true;
+  const long long slots = (long long)(16 * 32 / block_y) * sm_count();
+  const long long sites = (L.site_tiles + slots - 1) / slots, all = (L.site_tiles + L.wall_tiles + slots - 1) / slots;
+  return block_y >= 128 && sites <= 2 && all > sites;
+}
+
 }  // namespace
 
 int launch_batch_tiles(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const int* tile_entry, int parity,
                        int block_y, cudaStream_t stream) {
+  if (table_is_faster(L, block_y))
+    return launch_batch_fused(tab, tile_entry, L.n, L.site_tiles, parity, block_y, L.site_tiles,
+                              uniform ? &L.common : nullptr, stream);
   switch (block_y) {
     case 64: return tile_launch<64, 10>(L, uniform, tab, tile_entry, parity, stream);
     case 128: return tile_launch<128, 5>(L, uniform, tab, tile_entry, parity, stream);

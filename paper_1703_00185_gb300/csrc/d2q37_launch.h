@@ -48,18 +48,19 @@ int launch_fields32(const float* buf, double* rho, double* u, double* T, const S
 // of the grid-stride loop.  *_blocks_per_sm: resident blocks per SM.
 // tile_entry: owning entry of every tile (device, tiles values), or null
 // for a binary search over the table's tile0.  common (FP64): when every
-// lattice shares tau and g, a StepParams holding their collision constants
-// (passed as a kernel argument), else null.
+// lattice shares tau and g, their collision constants (passed as a kernel
+// argument), else null.
 int launch_batch_fused(const BatchEntry* tab, const int* tile_entry, int n, long long tiles, int parity,
-                       int block_y, int grid, const StepParams* common, cudaStream_t stream);
+                       int block_y, int grid, const Collision* common, cudaStream_t stream);
 int batch_blocks_per_sm(int block_y);
 // The batched FP64 step with one block per tile (see BatchLaunch); uniform:
 // every lattice has the collision constants L.common.  tab: the BatchEntry
-// table (device: wall equilibria and, if not uniform, collision constants).
+// table for tiles of block_y rows (device).
 // tile_entry: owning lattice of every site tile (device), or null for a search.
-// The (column, wall) groups one wall tile holds.
+// Small batches run the table kernel instead.
 int launch_batch_tiles(const BatchLaunch& L, bool uniform, const BatchEntry* tab, const int* tile_entry, int parity,
                        int block_y, cudaStream_t stream);
+// The (column, wall) groups one wall tile holds.
 int batch_wall_groups_per_tile(int block_y);
 int launch_batch_fused32(const BatchEntry* tab, const int* tile_entry, int n, long long tiles, int parity,
                          int block_y, int grid, bool wide_fp64, cudaStream_t stream);
