@@ -40,7 +40,10 @@ extern "C" {
 #define LBM_EINVAL (-1)   /* bad argument: NULL, Lx < 3, Ly < 6, tau <= 0.5, bad phase mask */
 #define LBM_ENOMEM (-2)   /* device allocation failed, or caller buffer too small */
 #define LBM_ECUDA (-3)    /* a CUDA call or kernel launch failed */
-#define LBM_ETIMEOUT (-4) /* a bounded device wait ran out since the last synchronisation */
+#define LBM_ETIMEOUT (-4) /* a bounded device wait of this handle's kernels ran out: part of the state is
+                             unwritten.  Returned once, by the first call on the handle that sees it (any
+                             that steps, reads out or synchronises); the handle has no state then, until
+                             lbm_init_rayleigh_taylor or lbm_set_populations */
 #define LBM_ESTATE (-5)   /* call out of order, e.g. a step before any initial state */
 #define LBM_ETOOBIG (-6)  /* more lattices than lbm_batch_step_static's fixed table holds */
 
@@ -139,7 +142,7 @@ int lbm_fields(lbm_t* h, double* rho, double* u, double* T);
 int lbm_fields_device(lbm_t* h, double* rho, double* u, double* T);
 
 /* Wait for all work enqueued on the handle's stream; reports any
- * asynchronous CUDA error as LBM_ECUDA. */
+ * asynchronous CUDA error as LBM_ECUDA, a wait that ran out as LBM_ETIMEOUT. */
 int lbm_synchronize(lbm_t* h);
 
 /* Number of CUDA kernels this handle has enqueued so far, graph replays
@@ -215,6 +218,8 @@ int lbm_batch_get_config(const lbm_batch_t* b, int* block_y, int* blocks_per_sm)
  * Synchronises the batch stream. */
 int lbm_batch_autotune(lbm_batch_t* b, int trial_steps, int* block_y, int* blocks_per_sm, double* best_ms);
 
+/* Wait for the batch stream.  LBM_ETIMEOUT when a wait of any of the lattices ran
+ * out; those lattices have no state then. */
 int lbm_batch_synchronize(lbm_batch_t* b);
 int64_t lbm_batch_launch_count(const lbm_batch_t* b);
 
@@ -284,7 +289,7 @@ typedef struct {
   size_t budget_bytes, bytes_in_use, largest_free_bytes;
 } lbm_server_stats;
 
-/* Allocates the pool (cudaMalloc of hbm_budget_bytes) and 3 streams on the
+/* Allocates the pool (cudaMalloc of hbm_budget_bytes) and 8 streams on the
  * current device.  LBM_ENOMEM if the pool cannot be allocated. */
 int lbm_server_create(size_t hbm_budget_bytes, int max_steps_per_tick, lbm_server_t** out);
 
@@ -305,7 +310,8 @@ int lbm_server_poll(lbm_server_t* s, int64_t* ids, int max_ids, int* n);
 int lbm_server_job_state(const lbm_server_t* s, int64_t id, int* state, int* steps_left);
 
 /* Copy a completed job's fields (layout of lbm_fields) and forget the job.
- * LBM_ESTATE if it has not completed. */
+ * LBM_ESTATE if it has not completed; LBM_ETIMEOUT, and the job forgotten, if
+ * a bounded device wait of its kernels ran out (it has no fields). */
 int lbm_server_fetch(lbm_server_t* s, int64_t id, double* rho, double* u, double* T);
 
 int lbm_server_stats_get(const lbm_server_t* s, lbm_server_stats* out);

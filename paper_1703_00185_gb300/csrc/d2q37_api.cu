@@ -120,18 +120,47 @@ int ensure_device_consts() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 256) return LBM_ECUDA;
   std::lock_guard<std::mutex> lock(g_dev_mutex);
   if (!g_dev_ready[dev]) {
-    if (!g_consts.late) {  // one word for the process, mapped on every device
-      void* w = nullptr;
-      if (cudaHostAlloc(&w, sizeof(unsigned), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess)
-        return LBM_ENOMEM;
-      g_consts.late = (unsigned*)w;
-      *g_consts.late = 0;
-    }
     if (upload_shell_consts(g_consts) != cudaSuccess) return LBM_ECUDA;
     if (upload_shell_consts32(g_consts32) != cudaSuccess) return LBM_ECUDA;
     g_dev_ready[dev] = true;
   }
   return LBM_OK;
+}
+
+// The handles' time-out words: host memory mapped on every device, so that a
+// kernel's store reaches the host without a copy.  Taken with a handle and given
+// back with it; the pages stay, as many as the most handles alive at once need.
+class LateWords {
+ public:
+  unsigned* take() {
+    std::lock_guard<std::mutex> lock(mutex_);
+    if (free_.empty()) {
+      void* page = nullptr;
+      if (cudaHostAlloc(&page, kPage * sizeof(unsigned), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+      }
+      for (int k = kPage; k-- > 0;) free_.push_back((unsigned*)page + k);
+    }
+    unsigned* const w = free_.back();
+    free_.pop_back();
+    *w = 0;
+    return w;
+  }
+  void give(unsigned* w) {
+    std::lock_guard<std::mutex> lock(mutex_);
+    free_.push_back(w);
+  }
+
+ private:
+  static constexpr int kPage = 1024;
+  std::mutex mutex_;
+  std::vector<unsigned*> free_;
+};
+
+LateWords& late_words() {
+  static LateWords* const w = new LateWords();  // never destroyed: handles may outlive static objects
+  return *w;
 }
 
 size_t align256(size_t n) { return (n + 255) & ~size_t(255); }
@@ -180,6 +209,7 @@ void fill_step_params(lbm_t* h) {
   sp.Hy = halo_rows(h->prec);
   sp.periodic_y = h->prm.periodic_y ? 1 : 0;
   sp.plane = (long long)h->NX * h->NY;
+  sp.late = h->late;
   for (int l = 0; l < kQ; ++l) {
     sp.pull_off[l] = (l * sp.plane - kCx[l] * (long long)sp.NY - kCy[l]) * (long long)sizeof(double);
     sp.plane_off[l] = l * sp.plane * (long long)sizeof(double);
@@ -323,6 +353,8 @@ int setup_handle(lbm_t* h, int Lx, int Ly, const lbm_params* p, void* mem, cudaS
   h->scratch = (double*)(base + 2 * bb);
   h->cur = 0;
   h->stream = stream;
+  h->late = late_words().take();
+  if (!h->late) return LBM_ENOMEM;
   fill_step_params(h);
   // halo rows must read as zero (FP64) or as f = w (FP32 deviations): the pull
   // takes the populations a wall replaces from there
@@ -402,6 +434,19 @@ bool fused_graph(lbm_t* h, int steps, cudaGraphExec_t* out) {
   return true;
 }
 
+// Whether the handle has a state to work on.
+int check_state(lbm_t* h) {
+  const int rc = handle_late(h);
+  return rc ? rc : h->have_state ? LBM_OK : LBM_ESTATE;
+}
+
+// A new state: an earlier time-out, if any, is of no consequence.
+void new_state(lbm_t* h) {
+  handle_late(h);
+  h->have_state = true;
+  h->halo_valid = false;
+}
+
 size_t plane_offset_bytes(const lbm_t* h, int l) {
   return ((size_t)l * h->sp.plane + (size_t)kHx * h->NY + h->sp.Hy) * h->elem;
 }
@@ -420,12 +465,16 @@ int handle_prepare_halos(lbm_t* h, cudaStream_t stream) {
   return LBM_OK;
 }
 
-int handle_sync(cudaStream_t stream) {
-  const int rc = check(cudaStreamSynchronize(stream));
-  volatile unsigned* late = g_consts.late;
-  if (rc || !late || !*late) return rc;
-  *late = 0;
+int handle_late(lbm_t* h) {
+  if (!__atomic_load_n(h->late, __ATOMIC_ACQUIRE)) return LBM_OK;
+  __atomic_store_n(h->late, 0u, __ATOMIC_RELEASE);
+  h->have_state = false;
   return LBM_ETIMEOUT;
+}
+
+int handle_sync(lbm_t* h) {
+  const int rc = check(cudaStreamSynchronize(h->stream));
+  return rc ? rc : handle_late(h);
 }
 
 int handle_device_consts() {
@@ -537,10 +586,7 @@ int lbm_init_rayleigh_taylor(lbm_t* h, uint64_t seed) {
                                          h->sp, h->stream);
     });
   if (!rc) rc = check(cudaStreamSynchronize(h->stream));
-  if (!rc) {
-    h->have_state = true;
-    h->halo_valid = false;
-  }
+  if (!rc) new_state(h);
   return rc;
 }
 
@@ -568,14 +614,13 @@ int lbm_set_populations(lbm_t* h, const double* f) {
     }
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LBM_ECUDA;
   }
-  h->have_state = true;
-  h->halo_valid = false;
+  new_state(h);
   return LBM_OK;
 }
 
 int lbm_get_populations(lbm_t* h, double* f) {
   if (!h || !f) return LBM_EINVAL;
-  if (!h->have_state) return LBM_ESTATE;
+  if (const int rc = check_state(h)) return rc;
   const char* d = (const char*)h->buf[h->cur];
   const size_t n = (size_t)h->Lx * h->Ly;
   if (!is_fp32(h->prec)) {
@@ -596,13 +641,13 @@ int lbm_get_populations(lbm_t* h, double* f) {
         return LBM_ECUDA;
     }
   }
-  return check(cudaStreamSynchronize(h->stream));
+  return handle_sync(h);
 }
 
 int lbm_step(lbm_t* h, int n) {
   const TraceRange trace("lbm_step");
   if (!h || n < 0) return LBM_EINVAL;
-  if (!h->have_state) return LBM_ESTATE;
+  if (const int rc = check_state(h)) return rc;
   const bool fused = h->prm.kernel != LBM_KERNEL_SEPARATE;
   int t = 0;
   if (fused && !h->timing && n >= 4) {
@@ -633,7 +678,7 @@ int lbm_step(lbm_t* h, int n) {
 int lbm_run_phases(lbm_t* h, int n, int phases) {
   if (!h || n < 0 || phases <= 0 || phases > LBM_PHASE_ALL) return LBM_EINVAL;
   if ((phases & LBM_PHASE_BC) && !(phases & LBM_PHASE_PROPAGATE)) return LBM_EINVAL;
-  if (!h->have_state) return LBM_ESTATE;
+  if (const int rc = check_state(h)) return rc;
   for (int t = 0; t < n; ++t) {
     const int rc = step_once(h, phases, false);
     if (rc) return rc;
@@ -643,7 +688,7 @@ int lbm_run_phases(lbm_t* h, int n, int phases) {
 
 int lbm_fields_device(lbm_t* h, double* rho, double* u, double* T) {
   if (!h || !rho || !u || !T) return LBM_EINVAL;
-  if (!h->have_state) return LBM_ESTATE;
+  if (const int rc = check_state(h)) return rc;
   return run_kernel(h, LBM_KIND_FIELDS, [&] { return k_fields(h, h->buf[h->cur], rho, u, T); });
 }
 
@@ -656,20 +701,19 @@ int lbm_fields(lbm_t* h, double* rho, double* u, double* T) {
   rc = check(cudaMemcpyAsync(rho, s, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   if (!rc) rc = check(cudaMemcpyAsync(u, s + n, 2 * n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   if (!rc) rc = check(cudaMemcpyAsync(T, s + 3 * n, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  if (!rc) rc = check(cudaStreamSynchronize(h->stream));
-  return rc;
+  return rc ? rc : handle_sync(h);
 }
 
 int lbm_synchronize(lbm_t* h) {
   if (!h) return LBM_EINVAL;
-  return handle_sync(h->stream);
+  return handle_sync(h);
 }
 
 int64_t lbm_launch_count(const lbm_t* h) { return h ? h->launches : 0; }
 
 int lbm_set_timing(lbm_t* h, int enable) {
   if (!h) return LBM_EINVAL;
-  int rc = check(cudaStreamSynchronize(h->stream));
+  int rc = handle_sync(h);
   if (drain_timing(h) != LBM_OK) rc = LBM_ECUDA;
   for (int k = 0; k < LBM_KIND_COUNT; ++k) {
     h->kind_ms[k] = 0.0;
@@ -681,7 +725,7 @@ int lbm_set_timing(lbm_t* h, int enable) {
 
 int lbm_kernel_times(lbm_t* h, double* ms, int64_t* launches) {
   if (!h) return LBM_EINVAL;
-  int rc = check(cudaStreamSynchronize(h->stream));
+  int rc = handle_sync(h);
   if (drain_timing(h) != LBM_OK) rc = LBM_ECUDA;
   for (int k = 0; k < LBM_KIND_COUNT; ++k) {
     if (ms) ms[k] = h->kind_ms[k];
@@ -701,8 +745,12 @@ void lbm_destroy(lbm_t* h) {
     if (g) cudaGraphExecDestroy(g);
   if (h->owns_stream && h->stream) cudaStreamDestroy(h->stream);
   if (h->owned) cudaFree(h->owned);
+  if (h->late) late_words().give(h->late);
   delete h;
 }
+
+// For tests (not in the header): the word that a kernel of this handle stores to.
+unsigned* d2q37_late_word(lbm_t* h) { return h->late; }
 
 const char* lbm_strerror(int code) {
   switch (code) {

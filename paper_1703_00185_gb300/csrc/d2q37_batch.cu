@@ -141,6 +141,15 @@ int launch(lbm_batch_t* b, int block_y, int blocks_per_sm, int parity) {
   return LBM_OK;
 }
 
+// LBM_ETIMEOUT when a lattice's kernel gave up a wait; each such lattice has no
+// state until a new one is set.
+int lattices_late(lbm_batch_t* b) {
+  int rc = LBM_OK;
+  for (lbm_t* h : b->lat)
+    if (handle_late(h)) rc = LBM_ETIMEOUT;
+  return rc;
+}
+
 // Record the parity of the lattices' current buffers in their handles.
 void publish_parity(lbm_batch_t* b) {
   for (int i = 0; i < b->n; ++i) b->lat[i]->cur = b->host_tab[0][i].cur ^ b->parity;
@@ -234,6 +243,7 @@ long long fill_batch_launch(BatchLaunch& L, int n, lbm_t* const* lattices, const
     g.buf[1] = lattices[i]->buf[1];
     g.inv_denom[0] = q.inv_denom[0];
     g.inv_denom[1] = q.inv_denom[1];
+    g.late = q.late;
     t0 += (long long)q.Lx * ((q.Ly + block_y - 1) / block_y);
     if (!q.periodic_y) w0 += (2LL * q.Lx + per_wall_tile - 1) / per_wall_tile;
     if (t0 + w0 > 2147483647LL) return -1;
@@ -308,7 +318,7 @@ int lbm_batch_create(int n, lbm_t* const* lattices, void* cuda_stream, lbm_batch
   }
   // the lattices' own pending work comes first; their halos must mirror the state
   for (int i = 0; i < n && !rc; ++i) {
-    rc = check(cudaStreamSynchronize(lattices[i]->stream));
+    rc = handle_sync(lattices[i]);
     if (!rc) rc = handle_prepare_halos(lattices[i], b->stream);
   }
   const int bys[3] = {64, 128, 256};
@@ -449,6 +459,7 @@ int lbm_batch_autotune(lbm_batch_t* b, int trial_steps, int* block_y, int* block
   b->launches = launches0;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  if (!rc) rc = lattices_late(b);
   if (rc) return rc;
   b->block_y = best_by;
   b->blocks_per_sm = best_bps;
@@ -460,7 +471,8 @@ int lbm_batch_autotune(lbm_batch_t* b, int trial_steps, int* block_y, int* block
 
 int lbm_batch_synchronize(lbm_batch_t* b) {
   if (!b) return LBM_EINVAL;
-  return handle_sync(b->stream);
+  const int rc = check(cudaStreamSynchronize(b->stream));
+  return rc ? rc : lattices_late(b);
 }
 
 int64_t lbm_batch_launch_count(const lbm_batch_t* b) { return b ? b->launches : 0; }

@@ -52,6 +52,7 @@ int lbm_batch_step_static(int n, lbm_t* const* lattices, int steps, void* cuda_s
   if (n > LBM_STATIC_BATCH_MAX) return LBM_ETOOBIG;
   for (int i = 0; i < n; ++i) {
     if (!lattices[i] || lattices[i]->prec != lattices[0]->prec) return LBM_EINVAL;
+    if (const int rc = handle_late(lattices[i])) return rc;
     if (!lattices[i]->have_state) return LBM_ESTATE;
     for (int j = 0; j < i; ++j)
       if (lattices[j] == lattices[i]) return LBM_EINVAL;

@@ -27,6 +27,7 @@ struct lbm_t {
   bool owns_stream;
   bool shares_device;  // other streams step other lattices at the same time (a job of a server)
   bool have_state;
+  unsigned* late;  // this handle's word (StepParams::late), see handle_late
   bool halo_valid;  // halo columns (and rows, if y is periodic) mirror the current state
   int64_t launches;
   cudaGraphExec_t graph2[2];  // two fused steps starting from buffer 0 / 1
@@ -64,9 +65,13 @@ constexpr int kLongGraphSteps = 16;
 // Launch the pbc kernel on `stream` if the handle's halos are stale.
 int handle_prepare_halos(lbm_t* h, cudaStream_t stream);
 
-// Wait for the stream; LBM_ETIMEOUT when a kernel's bounded wait has run out
-// since the last call.
-int handle_sync(cudaStream_t stream);
+// LBM_ETIMEOUT when a bounded wait of a kernel of this handle has run out since
+// the last call: tiles of its populations are unwritten, so it has no state
+// until a new one is set.  Looks at the work completed so far.
+int handle_late(lbm_t* h);
+
+// Wait for the handle's stream, then handle_late.
+int handle_sync(lbm_t* h);
 
 // The launch parameters of a one-block-per-tile step of n lattices with tiles
 // of block_y rows; cur[i]: the buffer holding lattice i's state at parity 0.

@@ -825,7 +825,7 @@ __device__ __forceinline__ void stage_init(unsigned char* stage, bool pull, int 
 
 // After stage_init: copy `rows` rows from `site` (16-byte aligned) of every
 // population into the block's slots, pulled (PULL) or in place, and wait for them.  g: the
-// lattice's plane and NY.  The hops come from packed fields and the copies are
+// lattice's plane, NY and late.  The hops come from packed fields and the copies are
 // spread over the warps: each is started by one lane after the other, and the
 // offsets read from the constant bank with an index per lane take as long.
 template <bool PULL, int ROWS = kStageRows, class G>
@@ -850,12 +850,14 @@ __device__ __forceinline__ RowPopsOf<PULL, ROWS> stage_rows(unsigned char* stage
                  "l"(at & ~15ull), "r"((at & 8) ? odd : even), "r"(bar)
                  : "memory");
   }
-  if (mbar_wait(bar)) return {slots + threadIdx.x * 8};
-  // never seen: tell the host (lbm_synchronize returns LBM_ETIMEOUT), give the
-  // copies in flight the same time again and leave the tile unwritten
-  if (threadIdx.x == 0) *(volatile unsigned*)c_shell.late = 1u;
-  mbar_wait(bar);
-  return {0u};
+  if (!mbar_wait(bar)) {
+    // never seen: every thread that ran out tells the host (the next call on the
+    // handle returns LBM_ETIMEOUT) and gives the copies in flight the same time
+    // again; its row stays unwritten if they do not land then either
+    *(volatile unsigned*)g.late = 1u;
+    if (!mbar_wait(bar)) return {0u};
+  }
+  return {slots + threadIdx.x * 8};
 }
 
 __global__ void __launch_bounds__(kStageRows, kStageBlocks) collide_kernel(double* __restrict__ buf, StepParams p) {

@@ -97,7 +97,6 @@ struct ShellConsts {
   double s2;
   double w[kShells];
   double alpha[kShells], beta[kShells], gamma[kShells], delta[kShells], eps[kShells];
-  unsigned* late;  // mapped host memory: set by a kernel whose bulk copies did not land in time
 };
 
 // FP32 deviation storage: populations are stored as d_l = f_l - w_l in FP32,
@@ -152,6 +151,7 @@ struct StepParams : Collision {
   // byte offsets from a site to the source of its pull (l plane - c_l . (NY, 1))
   // and to its population planes (l plane), for the single-lattice kernels
   long long pull_off[kQ], plane_off[kQ];
+  unsigned* late;  // the handle's word of mapped host memory: set by a kernel whose bulk copies did not land in time
   float omega_f, keep_f;  // 1/tau and 1 - 1/tau rounded to FP32 (FP32 storage)
   float uy_shift_df[2];    // uy_shift and theta_shift as double-float (hi, lo) pairs
   float theta_shift_df[2];
@@ -187,6 +187,7 @@ struct BatchGeo {
   long long plane;    // population plane stride (elements)
   void* buf[2];
   double inv_denom[2];
+  unsigned* late;     // as in StepParams
 };
 
 constexpr int kBatchGeoMax = 384;  // lattices per launch (parameter space: 32 KB)

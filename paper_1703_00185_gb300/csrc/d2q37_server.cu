@@ -42,6 +42,7 @@ struct Job {
   lbm_t* h;
   int stream;  // index into lbm_server_t::stream
   bool draining;        // fields enqueued into the scratch, waiting for done_ev
+  bool late;            // a bounded wait of its kernels ran out: there are no fields
   cudaEvent_t done_ev;  // recorded behind the fields kernel
   std::vector<double> rho, u, T;  // results once done
 };
@@ -172,15 +173,18 @@ int finalize(lbm_server_t* s, bool block) {
       if (e == cudaErrorNotReady && pass == 1 && block) e = cudaEventSynchronize(j->done_ev);
       if (e == cudaErrorNotReady) continue;
       if (e != cudaSuccess) return LBM_ECUDA;
-      const size_t n = (size_t)j->Lx * j->Ly;
-      j->rho.resize(n);
-      j->u.resize(2 * n);
-      j->T.resize(n);
-      const double* sc = j->h->scratch;  // rho, ux, uy, T planes
-      if (cudaMemcpy(j->rho.data(), sc, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
-          cudaMemcpy(j->u.data(), sc + n, 2 * n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
-          cudaMemcpy(j->T.data(), sc + 3 * n, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
-        return LBM_ECUDA;
+      if (handle_late(j->h)) j->late = true;
+      if (!j->late) {
+        const size_t n = (size_t)j->Lx * j->Ly;
+        j->rho.resize(n);
+        j->u.resize(2 * n);
+        j->T.resize(n);
+        const double* sc = j->h->scratch;  // rho, ux, uy, T planes
+        if (cudaMemcpy(j->rho.data(), sc, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
+            cudaMemcpy(j->u.data(), sc + n, 2 * n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess ||
+            cudaMemcpy(j->T.data(), sc + 3 * n, n * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
+          return LBM_ECUDA;
+      }
       s->stream_sites[j->stream] -= (long long)j->Lx * j->Ly;
       release_job_memory(s, j);
       j->state = LBM_JOB_DONE;
@@ -278,16 +282,25 @@ int lbm_server_tick(lbm_server_t* s, int* steps_done) {
     if (k > 0) {
       const int64_t before = j->h->launches;
       rc = lbm_step(j->h, k);
-      if (rc) return rc;
-      s->stats.launches += j->h->launches - before;
-      j->steps_left -= k;
-      s->stats.steps += k;
-      kmax = std::max(kmax, k);
+      if (rc == LBM_ETIMEOUT) {  // this job ends here; the others go on
+        j->late = true;
+        j->steps_left = 0;
+      } else {
+        if (rc) return rc;
+        s->stats.launches += j->h->launches - before;
+        j->steps_left -= k;
+        s->stats.steps += k;
+        kmax = std::max(kmax, k);
+      }
     }
     if (j->steps_left == 0) {
       const size_t n = (size_t)j->Lx * j->Ly;
       double* sc = j->h->scratch;
-      rc = lbm_fields_device(j->h, sc, sc + n, sc + 3 * n);
+      rc = j->late ? LBM_OK : lbm_fields_device(j->h, sc, sc + n, sc + 3 * n);
+      if (rc == LBM_ETIMEOUT) {
+        j->late = true;
+        rc = LBM_OK;
+      }
       if (!rc && cudaEventCreateWithFlags(&j->done_ev, cudaEventDisableTiming) != cudaSuccess) rc = LBM_ECUDA;
       if (!rc && cudaEventRecord(j->done_ev, s->stream[j->stream]) != cudaSuccess) rc = LBM_ECUDA;
       if (rc) return rc;
@@ -331,12 +344,23 @@ int lbm_server_fetch(lbm_server_t* s, int64_t id, double* rho, double* u, double
   if (it == s->jobs.end()) return LBM_EINVAL;
   Job* j = it->second;
   if (j->state != LBM_JOB_DONE) return LBM_ESTATE;
+  if (j->late) {
+    s->jobs.erase(it);
+    delete j;
+    return LBM_ETIMEOUT;
+  }
   std::memcpy(rho, j->rho.data(), j->rho.size() * sizeof(double));
   std::memcpy(u, j->u.data(), j->u.size() * sizeof(double));
   std::memcpy(T, j->T.data(), j->T.size() * sizeof(double));
   s->jobs.erase(it);
   delete j;
   return LBM_OK;
+}
+
+// For tests (not in the header): the handle of an active job, else null.
+lbm_t* d2q37_server_job_handle(lbm_server_t* s, int64_t id) {
+  auto it = s->jobs.find(id);
+  return it == s->jobs.end() ? nullptr : it->second->h;
 }
 
 int lbm_server_stats_get(const lbm_server_t* s, lbm_server_stats* out) {

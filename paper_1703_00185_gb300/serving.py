@@ -12,7 +12,7 @@ import time
 
 import numpy as np
 
-from . import (JOB_DONE, LBMError, PRECISIONS, _check, lbm_default_params, lbm_server_stats,
+from . import (JOB_DONE, LBM_ETIMEOUT, LBMError, PRECISIONS, _check, lbm_default_params, lbm_server_stats,
                load_library)
 
 
@@ -121,8 +121,14 @@ def run_trace(trace, budget_bytes, max_steps_per_tick=16, device=None, keep_resu
         t_now = time.perf_counter() - t0
         for jid in srv.poll():
             tid = by_jid[jid]
+            try:
+                r = srv.fetch(jid)
+            except LBMError as e:
+                if e.code != LBM_ETIMEOUT:
+                    raise
+                rejected.append(tid)
+                continue
             done_at[tid] = t_now
-            r = srv.fetch(jid)
             if keep_results:
                 results[tid] = r
     st = srv.stats()
