@@ -1,6 +1,6 @@
 """Build the sm_103a shared library in-tree with nvcc (no cmake, no torch JIT).
 
-Three translation units compile in parallel, then link into
+The translation units compile in parallel, then link into
 ``paper_1703_00185_gb300/libd2q37_gb300.so``.  Host code is compiled with
 ``-ffp-contract=off`` so the host-side initial-state recipe rounds the same
 way on every machine.
@@ -16,7 +16,7 @@ OBJ_DIR = os.path.join(HERE, "_build")
 LIB_NAME = "libd2q37_gb300.so"
 LIB_PATH = os.path.join(HERE, LIB_NAME)
 SOURCES = ["d2q37_kernels.cu", "d2q37_kernels_fp32.cu", "d2q37_api.cu", "d2q37_batch.cu", "d2q37_batch_static.cu", "d2q37_server.cu", "quadrature_dd.cu"]
-HEADERS = ["d2q37_lattice.cuh", "d2q37_launch.h", "d2q37_handle.h", "dfloat.cuh"]
+HEADERS = ["d2q37_lattice.cuh", "d2q37_launch.h", "d2q37_handle.h", "dfloat.cuh", "f32_convert.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

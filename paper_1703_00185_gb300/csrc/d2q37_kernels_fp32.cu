@@ -17,6 +17,7 @@
 
 #include "d2q37_launch.h"
 #include "dfloat.cuh"
+#include "f32_convert.cuh"
 
 namespace d2q37 {
 
@@ -41,33 +42,13 @@ __device__ __forceinline__ long long site_index(const P& p, int x, int y) {
 
 // ---- the wide type: FP64 or double-float, behind one set of names ----------
 
-// Conversions between FP64 and FP32 by integer operations, with the results of
-// the instructions to the last bit except that FP32 subnormals are zero: on
-// GB300 a conversion takes the FP64 pipe as long as an FMA does (16 clocks a
-// warp and SM), and that pipe bounds the FP64 wide terms.  1024 x 8192 step
-// 0.98 ms with the conversion instructions, 0.64 ms this way.  No branches: the
-// compiler contracts the FP64 products and sums around them into FMAs only
-// within a block of code.
-
-// round to nearest even
-__device__ __forceinline__ float f64_to_f32(double v) {
-  const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-  const unsigned ah = hi & 0x7FFFFFFFu;
-  // bits 29 .. 60: the exponent's low bits and the 23 bits kept; re-biased by -896
-  const unsigned x = __funnelshift_l(lo, hi, 3);
-  const unsigned up = (lo << 3) + (x & 1u) > 0x80000000u;  // above a half, or a half and odd
-  unsigned r = (x + 0x40000000u + up) & 0x7FFFFFFFu;
-  r = ah < (897u << 20) ? 0u : r;
-  r = ah >= (1151u << 20) ? (ah > 0x7FF00000u ? 0x7FFFFFFFu : 0x7F800000u) : r;
-  return __int_as_float((int)(r | (hi & 0x80000000u)));
+__device__ __forceinline__ float f64_to_f32(double v) {  // see f32_convert.cuh
+  return __uint_as_float(f32_bits((unsigned)__double2hiint(v), (unsigned)__double2loint(v)));
 }
 
 __device__ __forceinline__ double f32_to_f64(float v) {
-  const unsigned b = (unsigned)__float_as_int(v), ab = b & 0x7FFFFFFFu;
-  unsigned h = (ab >> 3) + (896u << 20);
-  h = ab < (1u << 23) ? 0u : h;
-  h = ab >= 0x7F800000u ? 0x7FF00000u | (ab >> 3) : h;
-  return __hiloint2double((int)(h | (b & 0x80000000u)), ab < (1u << 23) ? 0 : (int)(b << 29));
+  const unsigned b = __float_as_uint(v);
+  return __hiloint2double((int)f64_high(b), (int)f64_low(b));
 }
 
 struct WideF64 {
