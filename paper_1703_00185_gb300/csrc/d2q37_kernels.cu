@@ -22,7 +22,6 @@
 // Every warp reads 32 consecutive doubles of each population plane, so each
 // gather is a coalesced 256-byte row shifted by at most 3 elements.
 #include <atomic>
-#include <type_traits>
 
 #include <cuda_runtime.h>
 
@@ -1247,31 +1246,6 @@ int launch_propagate(const double* src, double* dst, const StepParams& p, cudaSt
 int launch_bc(const double* src, double* dst, const StepParams& p, cudaStream_t stream) {
   bc_kernel<<<(2 * p.Lx + 127) / 128, 128, 0, stream>>>(src, dst, p);
   return done(1);
-}
-
-// Launch; dependent: as a programmatic dependent of the kernel before it in the
-// stream.  Such a grid may be resident while earlier kernels still write what it
-// reads: after its griddepcontrol.wait those writes are visible to its ordinary
-// loads, but not to loads through the read-only path, whose data must not change
-// while the grid lives.  So no pointer of a kernel launched here is const
-// __restrict__ (which lets the compiler take that path, and move a load above
-// the wait), and the loads of populations go to L2: store_images reads row 3 of
-// the edge columns back, and with it the wall rows of the same sector, which
-// wall_band_kernel may be writing, into the L1 of an SM where the next grid waits.
-template <class... A>
-bool launch_pdl(void (*kernel)(A...), dim3 grid, int block, int smem, cudaStream_t stream, bool dependent,
-                std::common_type_t<A>... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess;
 }
 
 // The form of a sites kernel: rows per block and warps per SM of a register form

@@ -11,8 +11,6 @@
 //     in FP32, with d' = (1 - omega) d + omega w (rho P - 1).
 // Layout and step sequence are those of the FP64 kernels (d2q37_kernels.cu)
 // with 32 halo rows so FP32 columns stay 128-byte aligned.
-#include <type_traits>
-
 #include <cuda_runtime.h>
 
 #include "d2q37_launch.h"
@@ -692,29 +690,6 @@ int launch_collide32(float* buf, const StepParams& p, bool wide_fp64, cudaStream
   return done(1);
 }
 
-namespace {
-
-// Launch; dependent: as a programmatic dependent of the kernel before it in the
-// stream.  No pointer of a kernel launched here is const __restrict__: its grid
-// may be resident while the kernel before it writes what it reads, which the
-// read-only path does not allow; ordinary loads after griddepcontrol.wait see
-// those writes.
-template <class... A>
-int launch_pdl32(void (*kernel)(A...), dim3 grid, cudaStream_t stream, bool dependent, std::common_type_t<A>... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(kBlockY);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? done(1) : -1;
-}
-
-}  // namespace
-
 // Chained (128 rows x 6 blocks per SM) unless the grid takes between 5/12 and 9/10
 // of the room: there the next step's blocks, waiting where this one leaves room,
 // pile up on some SMs and the step after runs unevenly.  Chained / not, us a step:
@@ -726,8 +701,10 @@ int launch_fused32(const float* src, float* dst, const StepParams& p, bool wide_
   const dim3 grid = site_grid(p);
   const long long blocks = (long long)grid.x * grid.y, room = (long long)D2Q37_FP32_MIN_BLOCKS * sm_count();
   chain = chain && (blocks * 12 <= room * 5 || blocks * 10 >= room * 9);
-  return launch_pdl32(wide_fp64 ? fused32_kernel<WideF64> : fused32_kernel<WideDF>, grid, stream, chain, src, dst,
-                      p);
+  return launch_pdl(wide_fp64 ? fused32_kernel<WideF64> : fused32_kernel<WideDF>, grid, kBlockY, 0, stream, chain, src,
+                    dst, p)
+             ? done(1)
+             : -1;
 }
 
 template <class W, int BY>
@@ -788,7 +765,7 @@ int batch32_blocks_per_sm(int block_y, bool wide_fp64) {
 
 int launch_fields32(const float* buf, double* rho, double* u, double* T, const StepParams& p, cudaStream_t stream,
                     bool chain) {
-  return launch_pdl32(fields32_kernel, site_grid(p), stream, chain, buf, rho, u, T, p);
+  return launch_pdl(fields32_kernel, site_grid(p), kBlockY, 0, stream, chain, buf, rho, u, T, p) ? done(1) : -1;
 }
 
 }  // namespace d2q37

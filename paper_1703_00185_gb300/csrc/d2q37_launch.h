@@ -3,6 +3,8 @@
 // number of kernels it launched, or -1 if a launch failed.
 #pragma once
 
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "d2q37_lattice.cuh"
@@ -13,6 +15,31 @@ namespace d2q37 {
 cudaError_t upload_shell_consts(const ShellConsts& c);
 
 int sm_count();  // of the current device
+
+// Launch; dependent: as a programmatic dependent of the kernel before it in the
+// stream.  Such a grid may be resident while earlier kernels still write what it
+// reads: after its griddepcontrol.wait those writes are visible to its ordinary
+// loads, but not to loads through the read-only path, whose data must not change
+// while the grid lives.  So no pointer of a kernel launched here is const
+// __restrict__ (which lets the compiler take that path, and move a load above
+// the wait).  The FP64 ones load populations from L2: store_images reads row 3 of
+// the edge columns back, and with it the wall rows of the same sector, which
+// wall_band_kernel may be writing, into the L1 of an SM where the next grid waits.
+template <class... A>
+inline bool launch_pdl(void (*kernel)(A...), dim3 grid, int block, int smem, cudaStream_t stream, bool dependent,
+                       std::common_type_t<A>... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess;
+}
 
 int launch_wrap(double* buf, const StepParams& p, cudaStream_t stream);
 int launch_propagate(const double* src, double* dst, const StepParams& p, cudaStream_t stream);
