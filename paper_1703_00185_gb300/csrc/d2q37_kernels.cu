@@ -38,10 +38,10 @@ constexpr int kWallBlock = 128;
 
 // The batched kernel (D2Q37_BATCH_MIN_BLOCKS x 128 threads per SM, whatever
 // its block_y) reads its parameters from memory instead of the constant bank
-// and spills a little at 128 registers (20 bytes per thread); with 3 blocks of
+// and spills a little at 128 registers (56 to 84 bytes per thread); with 3 blocks of
 // 128 and no spills it was slower (2970 MLUPS against 3150 for 4, an earlier
-// form of the kernel).  The batch's per-lattice shape (block_y = 0), which
-// runs the single-lattice kernels, is faster still on the 64-lattice workload.
+// form of the kernel).  On large batches the tile kernels and the per-lattice
+// shape (block_y = 0), which runs the single-lattice kernels, are faster.
 #ifndef D2Q37_BATCH_MIN_BLOCKS
 #define D2Q37_BATCH_MIN_BLOCKS 4
 #endif
@@ -217,9 +217,8 @@ __device__ __forceinline__ double hop_dot(int cx, int cy, const double (&mx)[3],
 // product and keeps 2^-55 or better absolute precision on the order-1
 // quantities; exact integer sums remove the cancellation that
 // limits the FP64 form near T = 0.5 for the outer shells.  Per population
-// the result is turned into an FP64 number (fx_to_double: the FP64 pipe's
-// integer conversion, or integer operations for the shells of
-// D2Q37_INT_CVT_MASK) and relaxed with one FP64 FMA.  The shell factor omega w_k is carried as
+// the result is turned into an FP64 number (fx_convert: the FP64 pipe's integer
+// conversion, or integer operations for the last shell) and relaxed with one FP64 FMA.  The shell factor omega w_k is carried as
 // c_k 2^E_k with c_k in [0.5, 1).  The ranges that keep every intermediate
 // inside its format hold for rho in (0, 4), |T_bar - 1| < 1 and |u_bar| < 0.35
 // per component; other sites take the FP64 evaluation.
@@ -305,8 +304,10 @@ __device__ __forceinline__ long long mul_shift(long long x, long long y, int sh)
 // exponent field, two ways: the FP64 pipe's 64-bit integer conversion (round
 // to nearest even), or integer operations only (half away from zero).  The
 // last shell's 8 populations take the integer form: the FP64 pipe is the
-// busiest unit (70 %) and the ALU second (55 %); 2048 x 8192 step 2.46 ms,
-// the last two shells 2.45 ms, the last four 2.49 ms, all of them 2.61 ms.
+// busiest unit (72 %) and the ALU second (54 %).  2048 x 8192 step 2.412 ms, the
+// last two shells 2.394 ms, the last four and all of them slower (2.49, 2.61
+// beside 2.46).  The split stays at one: ties round differently, so moving a
+// shell changes the last bits of results.
 __device__ __forceinline__ double fx_to_double_fp64(long long g, int es) {
   const double d = (double)g;  // exact up to its one rounding
   return __hiloint2double(__double2hiint(d) + es, __double2loint(d));
@@ -1181,8 +1182,8 @@ __device__ __forceinline__ u64 splitmix64(u64 v) {
 // FP32 storage, their deviations from the weights.  At u = 0 every population
 // of a shell is rho w C0, C0 = 1 + theta (alpha + theta gamma).  1024 x 4096
 // FP64: 8.8 ms for the call with the temperatures made by one host core
-// (2.1 ns a site) and uploaded, 0.8 ms this way (0.18 ms of
-// HBM writes; the rest is FP64, mostly the division, and the host's sines).
+// (2.1 ns a site) and uploaded, 0.41 ms this way (the kernel 0.39, of which 0.18
+// are HBM writes; the rest is FP64, mostly the division).
 template <class T>
 __global__ void __launch_bounds__(kBlockY) init_rayleigh_taylor_kernel(T* __restrict__ buf, const double* __restrict__ yi,
                                                                        double T_top, double T_bot, u64 seed,
@@ -1250,27 +1251,33 @@ int launch_bc(const double* src, double* dst, const StepParams& p, cudaStream_t 
 
 // The form of a sites kernel: rows per block and warps per SM of a register form
 // (255 registers with 8 warps, 128 with 16), or the staged one (rows = 0).
-// Microseconds a step, "w" = warps of 32 rows per SM, 512 rows unless stated:
-//                          staged  255 regs  128 regs   before the staged form
-//  walls    38 x 512   4 w   13.7      12.9      13.4
-//           76 x 512   8 w   17.0      21.7      15.9
-//          142 x 512  15 w   22.2      22.6      18.0    19.2
-//          185 x 512  19 w   23.9      30.7      25.0
-//          570 x 512  60 w   64.1      87.3      65.5    68.8
-//  periodic 64 x 64          9.5       8.4       8.5     9.0
-//          142 x 512  15 w   22.3      19.4      15.7    17.0
-//          285 x 512  30 w   30.2      37.3      28.4    30.6
-//          570 x 512  60 w   58.3      77.9      60.0    60.1
-//         1140 x 512 120 w  101.5     143.1     109.8   106.5
+// Microseconds a step, "w" = warps of 32 rows per SM; the best of blocks of 32
+// and 128 rows; chained or not as launch_fused has it:
+//                           staged  255 regs  128 regs   before the staged form
+//  walls     38 x 512   4 w   14.3      12.8      14.3
+//            76 x 512   8 w   17.3      21.3      15.9
+//           142 x 512  15 w   22.3      22.9      17.8    18.9
+//           185 x 512  19 w   24.0      31.2      25.1
+//           570 x 512  60 w   64.5      85.7      61.4    68.6
+//          1500 x 512 158 w  139.2     191.8     135.9
+//          2375 x 512 250 w  207.1     291.4     205.6   220.0
+//          8000 x 512 842 w  662.9     949.2     673.3
+//           256 x 8192 431 w 324.1     480.6     338.1
+//  periodic  64 x 64          9.8       8.6       8.4     8.8
+//           142 x 512  15 w   18.3      19.4      15.6    17.1
+//           285 x 512  30 w   30.5      37.5      27.7    30.3
+//           570 x 512  60 w   59.0      77.8      55.3    60.0
+//          1140 x 512 120 w  102.5     143.5     101.1   106.5
+//          1900 x 512 200 w  159.2     231.0     161.0
 struct SiteForm {
   int rows, warps;
 };
 constexpr SiteForm kStaged = {0, 0};
 
 // 128 registers: blocks of 32 rows leave the fewest threads idle (512 x 257
-// periodic 28.3 us, of 128 rows 32.9).  Blocks of 128 have fewer warps with edge
-// rows and are fewer to start: 64 x 64 periodic 8.5 / 8.9 us, 60 lattices of 120 x
-// 240 on four streams 347 / 369.
+// periodic 27.6 us, of 128 rows 32.4).  Blocks of 128 have fewer warps with edge
+// rows and are fewer to start: 60 lattices of 120 x 240 on four streams 347 us, of
+// 32 rows 369.
 SiteForm reg_form(int rows) {
   const bool one = rows > 32 && rows <= 128, full = rows * 10LL >= 9 * 128LL * ((rows + 127) / 128);
   return {one || full ? 128 : 32, 16};
@@ -1283,42 +1290,54 @@ bool form_resident(SiteForm f, int Lx, int rows, int walls) {
   return warps + walls * (kWallBlock / 32) * (f.warps / 8) <= (long long)f.warps * sm_count();
 }
 
+long long stage_tiles(int Lx, int rows) { return (long long)Lx * ((rows + kStageRows - 1) / kStageRows); }
+
+// Whether the staged tiles take no more than nine tenths of the room.
+bool one_wave(int Lx, int rows) { return stage_tiles(Lx, rows) * 10 <= 9LL * kStageBlocks * sm_count(); }
+
 // Whether the staged tiles hold so few rows that 128 registers win at any size
-// (their idle warps keep a third of the SM's warps from running): below 0.8 of
+// (their idle warps keep a third of the SM's warps from running): below 0.92 of
 // 256 rows a tile, below a half where the staged tiles are one wave.  Staged / 128
-// registers: 1500 x 300 (0.59) periodic 117 / 94 us, 1000 x 384 (0.75) 81.5 / 78,
-// 1000 x 450 (0.88) 93.3 / 93.8, 400 x 1200 (0.94) 88 / 94; walls 1500 x 300 113 /
-// 98, 600 x 800 (0.78) 101 / 98, 800 x 640 (0.83) 102 / 103; 256 x 196 (0.75,
-// one wave) 17.4 / 21.9.
-bool poor_fill(int Lx, int rows) {
-  const int tiles = (rows + kStageRows - 1) / kStageRows;
-  const bool one_wave = (long long)Lx * tiles <= (long long)kStageBlocks * sm_count();
-  return rows * 10LL < (one_wave ? 5LL : 8LL) * kStageRows * tiles;
+// registers, walls: 1500 x 300 (0.58) 113.6 / 91.3 us, 4000 x 640 (0.83) 437.5 /
+// 414.6, 4000 x 700 (0.91) 458 / 452, 3000 x 1200 (0.935) 568 / 574, 4000 x 1000
+// (0.97) 622 / 644; periodic 1500 x 300 117.7 / 85.0, 4000 x 640 432 / 408, 4000 x 700
+// 456 / 446, 4000 x 480 (0.94) 304 / 311; one wave: 256 x 196 (0.75) not chained 17.5 /
+// 21.0, 400 x 100 (0.38) 24.3 / 18.3.  Beside other streams' grids below 0.8 (a
+// server's 16 jobs of 200 to 500 columns 54.7 ms, with 0.92 57.5).
+bool poor_fill(int Lx, int rows, bool alone) {
+  const long long room = stage_tiles(1, rows) * kStageRows;
+  return rows * 100LL < (one_wave(Lx, rows) ? 50 : alone ? 92 : 80) * room;
 }
 
-// Up to this many warps of rows per SM 128 registers win without walls, where no
-// second kernel waits for room.
-constexpr int kRegWarps = 40;
-bool few_warps(int Lx, int rows) { return (long long)Lx * ((rows + 31) / 32) <= (long long)kRegWarps * sm_count(); }
+// Up to this many warps of rows per SM 128 registers win (the table above); beside
+// other streams' grids less.
+constexpr int kRegWarps = 150, kRegWarpsShared = 40;
+bool few_warps(int Lx, int rows, bool alone) {
+  return (long long)Lx * ((rows + 31) / 32) <= (long long)(alone ? kRegWarps : kRegWarpsShared) * sm_count();
+}
 
 // alone: no other stream's grids beside this one.  Beside others, walled lattices
-// that do not fill the GPU many times over keep the staged form, which leaves room (a server's burst of 12 jobs 17.5 ms,
-// 19.3 with tiles filled badly in 128 registers; 16 jobs of 200 to 500 columns
-// 54.7, 59.6), and no lattice takes 255 registers.  A walled step that is not
-// chained keeps the staged form too, for the wall-band kernel's room.
+// that do not fill the GPU many times over keep the staged form, which leaves room
+// (a server's burst of 12 jobs 17.5 ms, 19.3 with tiles filled badly in 128
+// registers; 16 jobs of 200 to 500 columns 54.7, 59.6), and no lattice takes 255
+// registers.  Walled lattices of one wave take a register form only where the
+// wall-band kernel has room beside it; else staged blocks leave it some (142 x 512 not
+// chained 18.6 us, 21.9 in 128 registers).
 SiteForm fused_form(const StepParams& p, int rows, int walls, bool chain, bool alone) {
+  const SiteForm reg = reg_form(rows);
   if (p.periodic_y ? alone : chain)
     for (const SiteForm f : {SiteForm{rows > 32 ? 128 : 32, 8}, SiteForm{32, 8}})
       if (form_resident(f, p.Lx, rows, walls)) return f;
-  if (!alone && !p.periodic_y && few_warps(p.Lx, rows)) return kStaged;
-  const SiteForm reg = reg_form(rows);
-  if (poor_fill(p.Lx, rows)) return reg;
-  if (p.periodic_y ? few_warps(p.Lx, rows) : chain && form_resident(reg, p.Lx, rows, walls)) return reg;
-  return kStaged;
+  const bool few = few_warps(p.Lx, rows, alone);
+  if (p.periodic_y) return few || poor_fill(p.Lx, rows, alone) ? reg : kStaged;
+  if (!alone && few) return kStaged;
+  if (chain && form_resident(reg, p.Lx, rows, walls)) return reg;
+  if (poor_fill(p.Lx, rows, alone)) return reg;
+  return alone && few && !one_wave(p.Lx, rows) ? reg : kStaged;
 }
 
 int launch_collide(double* buf, const StepParams& p, cudaStream_t stream) {
-  const SiteForm form = poor_fill(p.Lx, p.Ly) || few_warps(p.Lx, p.Ly) ? reg_form(p.Ly) : kStaged;
+  const SiteForm form = poor_fill(p.Lx, p.Ly, true) || few_warps(p.Lx, p.Ly, true) ? reg_form(p.Ly) : kStaged;
   void (*const kernel)(double*, StepParams) =
       !form.rows ? collide_kernel : form.rows == 128 ? collide_reg_kernel<128> : collide_reg_kernel<32>;
   const int rows = form.rows ? form.rows : kStageRows;
@@ -1340,15 +1359,14 @@ int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream
   const dim3 grid(p.Lx, (Ly + rows - 1) / rows);
   // The next step's blocks wait where this one's leave room.  With 255 registers
   // that hides the launch.  Between half and all of the room they pile up on some
-  // SMs, and the step after runs unevenly (100 x 512 periodic 15.5 us, not chained
-  // 13.4); with walls and more than one wave they keep the wall-band kernel
-  // from its room (570 x 512 67.4 us, 64.1; 185 x 512, one wave, 23.9, 26.5).
-  const long long used = (long long)grid.x * grid.y * (rows / 32);
-  const long long room = (long long)(form.rows ? form.warps : kStageBlocks * kStageRows / 32) * sm_count();
-  if (form.warps != 8)
-    chain = chain && (p.periodic_y ? used * 12 <= room * 5 || used * 10 >= room * 9
-                      : form.rows  ? form_resident(form, p.Lx, Ly, walls)
-                                   : used * 10 <= room * 9);
+  // SMs, and the step after runs unevenly (100 x 512 periodic 15.0 us, not chained
+  // 13.1); with walls and more than one wave they keep the wall-band kernel
+  // from its room (2375 x 512 210.6 us, 207.1; 185 x 512, one wave, 24.0, 27.4).
+  const long long used = (long long)grid.x * grid.y * (rows / 32), room = (long long)form.warps * sm_count();
+  if (p.periodic_y)
+    chain = chain && (form.warps != 16 || used * 12 <= room * 5 || used * 10 >= room * 9);
+  else
+    chain = chain && (form.rows ? form_resident(form, p.Lx, Ly, walls) : one_wave(p.Lx, Ly));
   if (!launch_pdl(sites, grid, rows, form.rows ? 0 : kStageBytes, stream, chain, src, dst, p)) return -1;
   if (p.periodic_y) return done(1);
   if (!launch_pdl(wall_band_kernel, dim3(walls), kWallBlock, 0, stream, overlap, src, dst, p)) return -1;
@@ -1407,8 +1425,9 @@ cudaError_t allow_tile_memory() {
 // long, and the bulk copies add theirs.  Microseconds a step in registers /
 // staged, 128 rows, walls: shared tau and g 3 lattices of 40 x 80 (2 warps) 17.0 /
 // 21.1, 10 of 120 x 240 (63) 81.7 / 83.4, 14 (88) 105.5 / 104.7, 20 (126) 139 /
-// 137, 40 of 100 x 97 (105) 121 / 126, 60 of 120 x 240 (379) 372 / 359, 24 of 1024 x 1024 (5174) 4449 / 4084; their own 10 (63)
-// 85 / 93, 20 (126) 145 / 151, 30 (189) 207 / 210, 60 (379) 394 / 384.
+// 137, 40 of 100 x 97 (105) 121 / 126, 60 of 120 x 240 (379) 372 / 359, 24 of
+// 1024 x 1024 (5174) 4449 / 4084; their own 10 (63) 85 / 93, 20 (126) 145 / 151,
+// 30 (189) 207 / 210, 60 (379) 394 / 384.
 constexpr int kBatchFewWarps = 120, kBatchFewWarpsOwn = 250;
 
 template <int ROWS, int BLOCKS>

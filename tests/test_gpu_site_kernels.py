@@ -78,7 +78,8 @@ def test_long_chains_equal_the_serial_schedule(Lx, Ly, precision):
 
 # (Lx, Ly) on both sides of every rule that picks a form, and blocks whose last one is nearly empty
 FORMS = [(3, 9), (64, 64), (227, 34), (1000, 16), (2000, 35), (76, 512), (100, 512), (142, 515), (152, 515),
-         (130, 257), (130, 260), (256, 196), (400, 100), (500, 516), (470, 262), (460, 191), (40, 1030)]
+         (130, 257), (130, 260), (256, 196), (400, 100), (500, 516), (470, 262), (460, 191), (40, 1030), (1450, 512),
+         (1450, 470)]
 
 
 @pytest.mark.parametrize("Lx,Ly", FORMS)
