@@ -165,7 +165,9 @@ int64_t lbm_launch_count(const lbm_t* h);
 
 /* Per-kernel timing (not in the paper; measurement support).  enable != 0
  * records a CUDA event pair on the handle's stream around every later kernel
- * launch of this handle and clears the totals; 0 stops recording. */
+ * launch of this handle and clears the totals; 0 stops recording.  Timed steps
+ * wait for the one before them, and FP64 steps of small walled lattices run
+ * another form of the sites kernel than untimed ones (the same results). */
 int lbm_set_timing(lbm_t* h, int enable);
 
 /* Totals since timing was enabled: ms[LBM_KIND_COUNT] of device time per
@@ -183,7 +185,8 @@ void lbm_destroy(lbm_t* h);
  *  - block_y > 0, blocks_per_sm = 0: one launch per step with one block per
  *    tile (one column by block_y rows) of every lattice, in FP64 the wall rows
  *    in separate wall tiles of the same launch.  At most 384 lattices, whose
- *    geometry is in the launch's parameters; larger batches use the table below.
+ *    geometry is in the launch's parameters; larger batches, and FP64 ones with
+ *    walls and few sites, use the table below.
  *  - block_y > 0, blocks_per_sm > 0: a persistent grid-stride kernel over the
  *    tiles, each lattice's parameters read from a device table.
  *  - block_y = 0: one launch of the single-lattice fused kernel per lattice,

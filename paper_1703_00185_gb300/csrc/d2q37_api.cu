@@ -320,16 +320,18 @@ int k_collide(lbm_t* h, void* b) {
                           : launch_collide((double*)b, h->sp, h->stream);
 }
 
-// One fused step, chained to the kernel before it in the stream (64 x
-// 64: FP64 15.5 -> 14.2 us a step, with the form for few sites; FP32 storage 5.65
-// -> 5.53 us; 2048 x 8192 FP32: 7.32 -> 7.30 ms for 8).  Not under per-kernel timing, nor in the serial schedule, nor for
-// a job of the server: its blocks waiting for their own stream's step would
-// hold the SMs against the other streams (a burst of 12 jobs: 17.2 -> 20.0 ms).
+// One fused step, chained to the kernel before it in the stream where the
+// launchers find that it helps (64 x 64: FP64 15.6 -> 13.4 us a step, with the form
+// for few sites; double-float FP32 storage 5.7 -> 5.6).  Not under per-kernel
+// timing, nor in the serial schedule, nor for a job of the server: its blocks
+// waiting for their own stream's step would hold the SMs against the other
+// streams (a burst of 12 jobs: 17.2 -> 20.0 ms).
 int k_fused(lbm_t* h, const void* s, void* d) {
   const bool serial = h->prm.kernel == LBM_KERNEL_FUSED_SERIAL, chain = !serial && !h->timing && !h->shares_device;
   return is_fp32(h->prec) ? launch_fused32((const float*)s, (float*)d, h->sp, h->prec == LBM_PRECISION_FP32_FP64,
                                            h->stream, chain)
-                          : launch_fused((const double*)s, (double*)d, h->sp, h->stream, !serial, chain, !h->shares_device);
+                          : launch_fused((const double*)s, (double*)d, h->sp, h->stream, !serial, chain,
+                                         !h->shares_device);
 }
 
 int k_fields(lbm_t* h, const void* b, double* rho, double* u, double* T) {

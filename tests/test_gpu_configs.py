@@ -42,7 +42,7 @@ def oracle_fields(Lx, Ly, seed, T_bot, steps):
 
 def test_batched_workload_lattices_against_oracle():
     """The three smallest lattices of the 64-lattice workload, advanced 100 steps
-    together by the split single launch (one kernel per step)."""
+    together by the one-block-per-tile launch (one kernel per step)."""
     import torch
     jobs = sorted(workloads.batched_lattices(1, 64), key=lambda j: j["Lx"] * j["Ly"])[:3]
     lats = []
