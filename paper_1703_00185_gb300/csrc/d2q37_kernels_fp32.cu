@@ -33,9 +33,9 @@ constexpr int kBlockY = 128;
 #define D2Q37_FP32_MIN_BLOCKS 6
 #endif
 
-template <class P>  // StepParams or BatchGeo32 (NY, Hy)
+template <class P>  // StepParams or BatchLat32 (NY)
 __device__ __forceinline__ long long site_index(const P& p, int x, int y) {
-  return (long long)(x + kHx) * p.NY + (y + p.Hy);
+  return (long long)(x + kHx) * p.NY + (y + kHy32);
 }
 
 // ---- the wide type: FP64 or double-float, behind one set of names ----------
@@ -236,7 +236,7 @@ __device__ __forceinline__ float fixed_to_float(long long v, int ex) {
 // in their theta-parts, G0_k, rho, E, T).  The velocity (|u| << 1) enters
 // only through a = xi.u_bar and q = |u_bar|^2, whose FP32 errors are scaled
 // down by |u|, and the q-parts of K0, K1 are ~q theta: FP32.
-// P: StepParams, or BatchGeo32 (the same collision fields)
+// P: StepParams, or BatchLat32 (the same collision fields)
 template <class W, class P>
 __device__ __forceinline__ void collide_site32(float (&d)[kQ], const P& p) {
   using T = typename W::T;
@@ -408,8 +408,9 @@ __device__ __forceinline__ void store_site32(float* __restrict__ dst, const P& p
 //   rho_w - 1 = (sum_O d - E) / D,   E = B - sum_O w + sum_M w,
 // with E and 1/D carried as (hi, lo) float pairs, so that no rounding of a
 // constant biases the wall's mass the same way every step.
+// w: the lattice's wall constants.
 template <class P>
-__device__ __forceinline__ float wall_rho_minus_1(const float* src, const P& p, int x, int wall) {
+__device__ __forceinline__ float wall_rho_minus_1(const float* src, const P& p, const StepParams& w, int x, int wall) {
   float out_d = 0.0f;
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
@@ -421,13 +422,12 @@ __device__ __forceinline__ float wall_rho_minus_1(const float* src, const P& p, 
       if (wall ? (cy > r) : (cy < -r)) out_d += (src + l * p.plane)[i];
     }
   }
-  const float t = (out_d - p.wall_e32[wall][0]) - p.wall_e32[wall][1];
-  return fmaf(t, p.wall_inv32[wall][0], t * p.wall_inv32[wall][1]);
+  const float t = (out_d - w.wall_e32[wall][0]) - w.wall_e32[wall][1];
+  return fmaf(t, w.wall_inv32[wall][0], t * w.wall_inv32[wall][1]);
 }
 
-template <class P>
-__device__ __forceinline__ float missing32(const P& p, float rho_w_minus_1, int wall, int l) {
-  return fmaf(rho_w_minus_1, p.fw32[wall][l], p.fwmw32[wall][l]);
+__device__ __forceinline__ float missing32(const StepParams& w, float rho_w_minus_1, int wall, int l) {
+  return fmaf(rho_w_minus_1, w.fw32[wall][l], w.fwmw32[wall][l]);
 }
 
 __global__ void __launch_bounds__(256) wrap32_kernel(float* __restrict__ buf, StepParams p) {
@@ -461,9 +461,11 @@ __global__ void __launch_bounds__(256) wrap32_kernel(float* __restrict__ buf, St
 
 // One site of the fused step (pull, wall bc on the wall bands, collide,
 // store with halo images).
-// dst aliases nothing: p may be in shared memory, read again after every store otherwise.
+// w: the lattice's wall constants.  dst aliases nothing: p may be in shared memory,
+// read again after every store otherwise.
 template <class W, class P>
-__device__ __forceinline__ void fused_site32(const float* src, float* __restrict__ dst, const P& p, int x, int y) {
+__device__ __forceinline__ void fused_site32(const float* src, float* __restrict__ dst, const P& p, const StepParams& w,
+                                             int x, int y) {
   // the site's pointer once per thread; each population at an offset that is
   // the same for the whole block (l plane - cx NY - cy)
   const float* q = src + (int)site_index(p, x, y);
@@ -473,11 +475,11 @@ __device__ __forceinline__ void fused_site32(const float* src, float* __restrict
   if (!p.periodic_y && (y < 3 || y >= p.Ly - 3)) {
     const int wall = y >= p.Ly - 3;
     const int r = wall ? p.Ly - 1 - y : y;
-    const float rho_w_m1 = wall_rho_minus_1(src, p, x, wall);
+    const float rho_w_m1 = wall_rho_minus_1(src, p, w, x, wall);
 #pragma unroll
     for (int l = 0; l < kQ; ++l) {
       const int cy = vel_cy(l);
-      if (wall ? (cy < -r) : (cy > r)) d[l] = missing32(p, rho_w_m1, wall, l);
+      if (wall ? (cy < -r) : (cy > r)) d[l] = missing32(w, rho_w_m1, wall, l);
     }
   }
   collide_site32<W>(d, p);
@@ -494,7 +496,7 @@ __global__ void __launch_bounds__(kBlockY, D2Q37_FP32_MIN_BLOCKS) fused32_kernel
   const int x = blockIdx.x;
   const int y = blockIdx.y * kBlockY + threadIdx.x;
   if (y >= p.Ly) return;
-  fused_site32<W>(src, dst, p, x, y);
+  fused_site32<W>(src, dst, p, p, x, y);
 }
 
 // Many lattices in one launch (see batch_fused_kernel of the FP64 kernels).
@@ -507,7 +509,7 @@ __global__ void __launch_bounds__(BY, (D2Q37_FP32_MIN_BLOCKS * 128) / BY) batch_
     const int x = local / e.ytiles;
     const int y = (local - x * e.ytiles) * BY + threadIdx.x;
     const int c = e.cur ^ parity;
-    if (y < e.p.Ly) fused_site32<W>((const float*)e.buf[c], (float*)e.buf[c ^ 1], e.p, x, y);
+    if (y < e.p.Ly) fused_site32<W>((const float*)e.buf[c], (float*)e.buf[c ^ 1], e.p, e.p, x, y);
   }
 }
 
@@ -525,21 +527,12 @@ __global__ void __launch_bounds__(BY, (D2Q37_FP32_MIN_BLOCKS * 128) / BY)
   const int b = blockIdx.x;
   // the lattice's parameters in shared memory: the blocks of an SM serve
   // different lattices, whose parameter slices would crowd the constant cache
-  __shared__ BatchGeo32 g;
+  __shared__ BatchLat32 g;
   static_assert(sizeof(BatchLat32) % sizeof(int) == 0, "BatchLat32 is copied as ints");
+  const int i = tile_entry ? tile_entry[b] : batch_owner(L, b);
   {
-    const int i = tile_entry ? tile_entry[b] : batch_owner(L, b);
     const int* from = (const int*)&L.g[i];
-    int* to = (int*)static_cast<BatchLat32*>(&g);
-    for (int k = threadIdx.x; k < (int)(sizeof(BatchLat32) / sizeof(int)); k += BY) to[k] = from[k];
-    if (threadIdx.x == 0) {
-      const StepParams& p = tab[i].p;
-      g.Hy = kHy32;
-      g.fw32 = p.fw32;
-      g.fwmw32 = p.fwmw32;
-      g.wall_e32 = p.wall_e32;
-      g.wall_inv32 = p.wall_inv32;
-    }
+    for (int k = threadIdx.x; k < (int)(sizeof(BatchLat32) / sizeof(int)); k += BY) ((int*)&g)[k] = from[k];
   }
   __syncthreads();
   const int local = b - g.tile0;
@@ -548,7 +541,7 @@ __global__ void __launch_bounds__(BY, (D2Q37_FP32_MIN_BLOCKS * 128) / BY)
   const int y = yt * BY + threadIdx.x;
   if (y >= g.Ly) return;
   const int c = g.cur ^ parity;
-  fused_site32<W>((const float*)g.buf[c], (float*)g.buf[c ^ 1], g, x, y);
+  fused_site32<W>((const float*)g.buf[c], (float*)g.buf[c ^ 1], g, tab[i].p, x, y);
 }
 
 __global__ void __launch_bounds__(kBlockY) propagate32_kernel(const float* __restrict__ src, float* __restrict__ dst,
@@ -567,7 +560,7 @@ __global__ void __launch_bounds__(128) bc32_kernel(const float* __restrict__ src
   if (t >= 2 * p.Lx) return;
   const int wall = t >= p.Lx;
   const int x = t - wall * p.Lx;
-  const float rho_w_m1 = wall_rho_minus_1(src, p, x, wall);
+  const float rho_w_m1 = wall_rho_minus_1(src, p, p, x, wall);
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     const int y = wall ? p.Ly - 1 - r : r;

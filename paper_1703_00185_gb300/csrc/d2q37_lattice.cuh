@@ -218,17 +218,6 @@ struct BatchLaunch32 {
   BatchLat32 g[kBatchGeo32Max];
 };
 
-// What the FP32 per-site code reads of a lattice of a batched launch: the
-// fields of StepParams under the same names, the wall constants by pointer into
-// the lattice's entry of the BatchEntry table (only wall rows read them).
-struct BatchGeo32 : BatchLat32 {
-  int Hy;
-  const float (*fw32)[kQ];
-  const float (*fwmw32)[kQ];
-  const float (*wall_e32)[2];
-  const float (*wall_inv32)[2];
-};
-
 // Index of the lattice of a launch that owns tile t (tile0 ascending from 0).
 template <class L>
 __device__ __forceinline__ int batch_owner(const L& l, int t) {
