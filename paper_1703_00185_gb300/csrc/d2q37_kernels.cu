@@ -55,6 +55,7 @@ __device__ __forceinline__ long long site_index(const P& p, int x, int y) {
 // Where a site's populations are: in registers, or in the block's shared
 // memory (RowPops), read again each time they are needed.
 struct RegPops {
+  static constexpr bool kSelect = false;  // see largest_high
   const double (&f)[kQ];
   __device__ __forceinline__ double get(int l) const { return f[l]; }
 };
@@ -129,10 +130,25 @@ __device__ __forceinline__ long long fixed_term(double v, unsigned top2, unsigne
   return r;
 }
 
-// The largest magnitude of the populations' high words: its exponent field is
-// the largest exponent.
+// The high word of the population of the largest magnitude: its exponent field
+// is the largest exponent.  Two ways, the same result: the maximum of the high
+// words, or (F::kSelect) the population itself, selected by its high word.  The
+// second costs more, but it is off the common path in the staged kernels, and the
+// pulling ones get a better register allocation with it (2048 x 8192 step 2.411 ->
+// 2.395 ms; 64 lattices with their own tau in tiles of 128 rows 7.08 -> 6.96 ms); in
+// place and in registers the first is faster (separate steps of 1000 x 2050 0.566
+// -> 0.544 ms).
 template <class F>
 __device__ __forceinline__ int largest_high(const F& f) {
+  if constexpr (F::kSelect) {
+    double m = 0.0;
+#pragma unroll
+    for (int l = 0; l < kQ; ++l) {
+      const double v = f.get(l);
+      if ((__double2hiint(v) & 0x7FFFFFFF) > (__double2hiint(m) & 0x7FFFFFFF)) m = v;
+    }
+    return __double2hiint(m);
+  }
   int m = 0;
 #pragma unroll
   for (int l = 0; l < kQ; ++l) m = max(m, __double2hiint(f.get(l)) & 0x7FFFFFFF);
@@ -305,7 +321,7 @@ __device__ __forceinline__ long long mul_shift(long long x, long long y, int sh)
 // to nearest even), or integer operations only (half away from zero).  The
 // last shell's 8 populations take the integer form: the FP64 pipe is the
 // busiest unit (72 %) and the ALU second (54 %).  2048 x 8192 step 2.412 ms, the
-// last two shells 2.394 ms, the last four and all of them slower (2.49, 2.61
+// last two shells 2.394 ms (both before largest_high's last change), the last four and all of them slower (2.49, 2.61
 // beside 2.46).  The split stays at one: ties round differently, so moving a
 // shell changes the last bits of results.
 __device__ __forceinline__ double fx_to_double_fp64(long long g, int es) {
@@ -778,6 +794,7 @@ __host__ __device__ constexpr int odd_hops() {
 // that the compiler does not keep the first reading in registers.
 template <bool PULL, int ROWS = kStageRows>
 struct RowPopsOf {
+  static constexpr bool kSelect = PULL;  // see largest_high
   unsigned a;  // shared address of the row in slot 0; 0: the copies did not land
   static __device__ __forceinline__ constexpr int at(int l) { return l * slot_bytes(ROWS) + (PULL ? vel_cy(l) & 1 : 0) * 8; }
   __device__ __forceinline__ double get(int l) const {
