@@ -49,9 +49,9 @@ ORACLE_NONTRIVIAL_FLOPS_PER_SITE = 17477
 # the flop term of the roofline min(HBM / bytes, FP64 peak / flops)
 ORACLE_CONTRACTED_FLOPS_PER_SITE = 2354
 # DRAM bytes per fused launch at 2048 x 8192, scaled by sites from the ncu
-# capture of the same kernel on 2048 x 1024 (1285.5 MB per launch there, some of
+# capture of the same kernel on 2048 x 1024 (1287.1 MB per launch there, some of
 # it spills)
-FUSED_TRAFFIC_BYTES_2048x8192 = 1285.5e6 * 8
+FUSED_TRAFFIC_BYTES_2048x8192 = 1287.1e6 * 8
 # the same for the FP32-storage double-float kernel, from its capture on
 # 2048 x 2048 (1236.2 MB per launch there, with streaming stores)
 FUSED32_DF_TRAFFIC_BYTES_2048x8192 = 1236.2e6 * 4
