@@ -47,7 +47,7 @@ int launch_bc(const double* src, double* dst, const StepParams& p, cudaStream_t 
 int launch_collide(double* buf, const StepParams& p, cudaStream_t stream);
 // overlap: the wall-band kernel (walls only) is launched as a programmatic
 // dependent of the sites kernel and starts in its tail; false: after it.
-// chain: the first kernel is launched as a programmatic dependent of whatever
+// chain: the first kernel may be launched as a programmatic dependent of whatever
 // kernel precedes it in the stream (it waits for it before its first access).
 // alone: no other stream's grids are expected beside it.
 int launch_fused(const double* src, double* dst, const StepParams& p, cudaStream_t stream, bool overlap = true,
